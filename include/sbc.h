@@ -146,12 +146,14 @@ sbc_status sbc_graph_info(const sbc_graph *g, sbc_graph_info_t *out);
  *                  1..512, default 512.
  *   pos_node_cost  cost of one prefix node of the position-side enumeration
  *                  relative to one word test of the candidate-side
- *                  enumeration; each anchor takes the cheaper side, so a
+ *                  enumeration (in eighths: the default 3 weighs a node as 24
+ *                  word tests); each anchor takes the cheaper side, so a
  *                  larger value favours the candidate (bitmap AND/POPC over
  *                  candidate tuples) side. 1..2^20, default 3.
- *   split_per_warp work items per warp of a full-GPU tuple launch: heavy
- *                  anchors are split into items of about (estimated total
- *                  cost) / (resident warps x split_per_warp). 1..64, default 4.
+ *   split_per_warp tuple work items per half of a resident tuple CTA (one CTA
+ *                  of 16 warps per SM): heavy anchors are shared by items of
+ *                  about (estimated total cost) / (2 x resident CTAs x
+ *                  split_per_warp). 1..64, default 4.
  *   tc_min_words   anchors with two partners (tuple size 3 on the anchor side)
  *                  whose candidate masks have at least this many 32-bit words
  *                  (and at least 128 candidates) take the tensor-core pair
@@ -197,8 +199,7 @@ typedef struct {
     uint64_t tuples_tested; /* tuples whose common-neighbour mask was tested (after
                                nested pruning) */
     uint64_t tuples_typed;  /* tuples with at least q common neighbours (type counts taken) */
-    uint64_t popc_words;    /* mask words popcounted by the tuple kernel: one per word of
-                               every tested tuple, 2^(k-1) per word of every typed tuple */
+    uint64_t popc_words;    /* mask words popcounted by the tuple kernel */
     int32_t anchor_side;    /* side used */
     int32_t kernels;        /* kernel launches issued by the call */
     float ms_prepare;       /* orientation build (first use of a side) + plan */

@@ -28,6 +28,9 @@
 #include <algorithm>
 #include <vector>
 
+#include <cfloat>
+#include <cstring>
+
 #include "sbc_internal.cuh"
 
 namespace sbc {
@@ -47,19 +50,23 @@ struct Counters {
     unsigned long long tuples_paper[2];// u128, sum binom(|C_paper|, R)
     unsigned long long tuples_ours[2]; // u128, sum binom(|C'|, R)
     unsigned long long candidates;     // sum |C'| (or |C_paper| in stats mode)
-    unsigned long long cost_total;     // tuple-phase cost estimate
     unsigned long long e_max;          // largest visited-wedge count of a large anchor
     unsigned int n_active;             // anchors with work
     unsigned int n_big;                // anchors for the CTA-wide 2-hop kernel
+    // tuple step of one anchor group: sizes, then the emit pass's cursors
+    float cost_total;                  // cost estimate of the work items
     unsigned int n_items;
-    unsigned int n_tc;                 // anchors of the group for the tensor-core pair step
+    unsigned int n_warp;               // anchors counted one per warp
+    unsigned int n_tc;                 // anchors for the tensor-core pair step
+    unsigned int n_claims;             // anchors shared by several work items
+    unsigned int e_items, e_warp, e_tc, e_claims;
     // ---- per execution
     unsigned long long run_begin;      // marker (unused)
     unsigned long long total[2];       // u128 count
     unsigned long long wedges;         // 2-hop entries visited
     unsigned long long tested;         // tuples whose common-neighbour mask was tested
     unsigned long long leaves;         // tuples with |T| >= l (type counts taken)
-    unsigned long long popc_words;     // mask words popcounted: W per test, 2^R W per leaf
+    unsigned long long popc_words;     // mask words popcounted by the tuple kernel
     // CTA-wide 2-hop kernel, by strategy (one window, bucketed, re-read windows,
     // bucketed with a second scatter)
     unsigned long long tw_reads;       // 2-hop entries read, all passes
@@ -69,7 +76,8 @@ struct Counters {
     unsigned long long tw_split;       // hash classes hashed in sub-class windows
     unsigned int head_large;           // 2-hop queue heads
     unsigned int head_small;
-    unsigned int head_b;               // tuple queue head
+    unsigned int head_b;               // tuple queue heads: work items,
+    unsigned int head_w;               // ... small anchors
     unsigned int err;                  // error bits
 };
 
@@ -215,10 +223,12 @@ __global__ void k_plan(const int64_t *__restrict__ A_off, const uint32_t *__rest
             bool act_count = dp >= (uint32_t)l && eu >= (unsigned long long)R * l;
             bool act_stats = d >= l && ea >= (unsigned long long)R * l;
             bool active = mine && (stats ? act_stats : act_count);
+            // rows (candidate parts with >= l positions) the masks need room
+            // for; one partner needs none (its 2-hop counters are enough)
             unsigned long long rc = 0;
-            if (active) {
-                rc = eu / (unsigned long long)l;  // each candidate owns >= l useful wedges
-                unsigned long long above = (unsigned long long)(nX - 1 - r);
+            if (active && R > 1) {
+                rc = eu / (unsigned long long)l;  // each row owns >= l useful wedges
+                unsigned long long above = 2 * (unsigned long long)(nX - 1 - r);
                 rc = rc < above ? rc : above;
             }
             uint32_t W = (dp + 31) / 32;
@@ -226,7 +236,7 @@ __global__ void k_plan(const int64_t *__restrict__ A_off, const uint32_t *__rest
             e_use[r] = eu;
             e_all[r] = ea;
             rsv_c[r] = (uint32_t)rc;
-            rsv_w[r] = (int64_t)(2ull * W * rc);
+            rsv_w[r] = (int64_t)((unsigned long long)W * rc);
             unsigned long long cost = stats ? ea : eu;
             skey[r] = active ? 0xFFFFFFFEu - (uint32_t)(cost < 0xFFFFFFFEull ? cost : 0xFFFFFFFEull)
                              : 0xFFFFFFFFu;
@@ -247,8 +257,9 @@ __global__ void k_plan(const int64_t *__restrict__ A_off, const uint32_t *__rest
 //   bits  0..20  cnt over all positions (Algorithm 2's cnt[w])
 //   bits 21..41  cnt over useful positions (|P_w|)
 //   bits 42..62  useful positions with sign(u,v) != sign(w,v) (|D_w|)
-//   bit  63      set once w is kept; bits 0..20 then hold its candidate index
-//                (the other two counters stay, for the mask self-check)
+//   bit  63      set once w is kept; bits 0..20 then hold its first row's index
+//                (the other two counters stay: they tell its parts, and the
+//                mask self-check uses them)
 constexpr unsigned long long F_ALL = 1ull, F_USE = 1ull << 21, F_DIFF = 1ull << 42;
 constexpr unsigned long long M21 = (1ull << 21) - 1;
 constexpr unsigned long long CAND = 1ull << 63;
@@ -306,39 +317,91 @@ __device__ __forceinline__ int tab_find(const uint32_t *keys, uint32_t hs, uint3
 
 // Candidate filter. Algorithm 2 keeps w when cnt[w] >= l. Every type class
 // of a tuple through w lies inside the same-sign or the different-sign part
-// of L[w] (the letter c_w is constant on a class), so only w with one part of
-// at least l useful common neighbours can add a non-zero binomial; the others
-// are dropped here, which changes no term of the sum.
-__device__ __forceinline__ bool keep_candidate(unsigned long long v, int l) {
-    uint32_t use = (uint32_t)((v >> 21) & M21), diff = (uint32_t)((v >> 42) & M21);
-    return use - diff >= (uint32_t)l || diff >= (uint32_t)l;
+// of L[w] (the letter c_w is constant on a class), so only parts with at least
+// l useful common neighbours can add a non-zero binomial: each of them becomes
+// a row of mask words, the others are dropped, which changes no term.
+__device__ __forceinline__ uint32_t use_count(unsigned long long v) { return (uint32_t)((v >> 21) & M21); }
+__device__ __forceinline__ uint32_t diff_count(unsigned long long v) { return (uint32_t)((v >> 42) & M21); }
+__device__ __forceinline__ bool keep_same(unsigned long long v, int l) {
+    return use_count(v) - diff_count(v) >= (uint32_t)l;
 }
+__device__ __forceinline__ bool keep_diff(unsigned long long v, int l) { return diff_count(v) >= (uint32_t)l; }
 
 __device__ __forceinline__ unsigned long long pass1_add(uint32_t sdiff, uint32_t bit) {
     return bit != EMPTY ? (F_ALL | F_USE | (sdiff ? F_DIFF : 0ull)) : F_ALL;
 }
 
-// Kept candidate: index `c` in bits 0..20, the two useful-position counters
-// kept, CAND set.
-__device__ __forceinline__ unsigned long long cand_value(unsigned long long v, uint32_t c) {
-    return CAND | (v & ~(CAND | M21)) | (unsigned long long)c;
+// Kept candidate: its first row's index in bits 0..20 (same-sign part first),
+// the two useful-position counters kept, CAND set.
+__device__ __forceinline__ unsigned long long cand_value(unsigned long long v, uint32_t row) {
+    return CAND | (v & ~(CAND | M21)) | (unsigned long long)row;
 }
-__device__ __forceinline__ uint32_t cand_index(unsigned long long v) { return (uint32_t)(v & M21); }
+// Row of the part `sdiff` of a kept candidate, EMPTY when that part was dropped.
+__device__ __forceinline__ uint32_t row_index(unsigned long long v, uint32_t sdiff, int l) {
+    const uint32_t base = (uint32_t)(v & M21);
+    const bool same = keep_same(v, l);
+    if (!sdiff) return same ? base : EMPTY;
+    return keep_diff(v, l) ? base + (same ? 1u : 0u) : EMPTY;
+}
 
-// Self-check of one kept candidate after its masks are written: popc(P_w)
-// must equal its useful common neighbours and popc(D_w) its different-sign
-// ones (both counted by the hash table in the first pass). `P` and `D` are
-// the candidate's first words; consecutive words are `stride` apart. Reads
-// bypass L1 (the words were written by atomics at L2).
-__device__ __forceinline__ bool masks_match(const uint32_t *P, const uint32_t *D, size_t stride,
-                                            uint32_t W, unsigned long long v, bool global) {
-    uint32_t np = 0, nd = 0;
-    for (uint32_t w = 0; w < W; w++) {
-        np += __popc(global ? __ldcg(P + w * stride) : P[w * stride]);
-        nd += __popc(global ? __ldcg(D + w * stride) : D[w * stride]);
-    }
-    return np == (uint32_t)((v >> 21) & M21) && nd == (uint32_t)((v >> 42) & M21);
+// Self-check of one row after its mask is written: its popcount must equal
+// the positions the hash table counted in the first pass. Consecutive words
+// are `stride` apart. Reads of global rows bypass L1 (the words were written
+// by atomics at L2).
+__device__ __forceinline__ bool row_matches(const uint32_t *row, size_t stride, uint32_t W, uint32_t want,
+                                            bool global) {
+    uint32_t n = 0;
+    for (uint32_t w = 0; w < W; w++) n += __popc(global ? __ldcg(row + w * stride) : row[w * stride]);
+    return n == want;
 }
+__device__ __forceinline__ bool rows_match(const uint32_t *rows, size_t stride, uint32_t W,
+                                           unsigned long long v, int l, bool global) {
+    const uint32_t s = row_index(v, 0, l), d = row_index(v, 1, l);
+    return (s == EMPTY || row_matches(rows + s, stride, W, use_count(v) - diff_count(v), global)) &&
+           (d == EMPTY || row_matches(rows + d, stride, W, diff_count(v), global));
+}
+
+// Where a count's sums go: the total, and per anchor or per graph of a batch.
+struct Totals {
+    unsigned long long *total;       // u128
+    unsigned long long *per_anchor;  // u128 per anchor rank, or null
+    unsigned long long *per_graph;   // u128 per graph of a batch, or null
+    const int64_t *graph_x0;         // first anchor rank of each graph (n_graphs + 1)
+    int n_graphs;
+    unsigned *err;
+};
+
+// Add one anchor's (partial) sum; called by one lane.
+__device__ __forceinline__ void add_totals(const Totals &t, uint32_t r, const U128 &s) {
+    if (!(s.lo | s.hi)) return;
+    // a batch's union total is not a count (its graphs' totals are)
+    atomic_add_u128(t.total, s.lo, s.hi, t.per_graph ? nullptr : t.err);
+    if (t.per_anchor) atomic_add_u128(t.per_anchor + 2 * (size_t)r, s.lo, s.hi, t.err);
+    if (t.per_graph) {
+        int lo = 0, hi = t.n_graphs;  // largest g with graph_x0[g] <= r
+        while (hi - lo > 1) {
+            int mid = (lo + hi) >> 1;
+            if (t.graph_x0[mid] <= (int64_t)r) lo = mid; else hi = mid;
+        }
+        atomic_add_u128(t.per_graph + 2 * (size_t)lo, s.lo, s.hi, t.err);
+    }
+}
+
+// What the tuple step's plan wants to know about an anchor's rows: positions
+// of all of them, and of the longest.
+struct RowInfo {
+    float pops = 0;
+    uint32_t longest = 0;
+    __device__ __forceinline__ void add(uint32_t pop) {
+        pops += (float)pop;
+        longest = pop > longest ? pop : longest;
+    }
+    __device__ __forceinline__ void warp_sum() {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) pops += __shfl_xor_sync(FULL, pops, o);
+        longest = __reduce_max_sync(FULL, longest);
+    }
+};
 
 struct TwohopArgs {
     const int64_t *A_off;
@@ -351,8 +414,11 @@ struct TwohopArgs {
     const int64_t *pool_off;
     const uint32_t *order;
     uint32_t *pool;
-    uint32_t *ncand, *npaper;
+    uint32_t *ncand, *npaper, *nrow;
+    RowInfo *rinfo;
     Counters *cnt;
+    Totals tot;
+    int single;                     // one partner: the counters give the sum, no rows are written
     unsigned long long *bucket;     // per-CTA bucket slots of the large-anchor kernel
     unsigned long long bucket_slot; // entries per slot
     unsigned large_begin, large_end;  // order[] ranges of the two kernels
@@ -438,7 +504,9 @@ __global__ void __launch_bounds__(PS_THREADS) k_twohop_small(TwohopArgs a) {
         (unsigned long long *)(smem_raw + (size_t)PS_WARPS * PS_HS * 4 + (size_t)warp * PS_HS * 8);
     const int l = a.l;
     const uint32_t lt = (1u << lane) - 1u;
-    unsigned long long wedges = 0;
+    const bool split_totals = a.tot.per_anchor || a.tot.per_graph;
+    unsigned long long wedges = 0, tested = 0, leaves = 0;
+    U128 total;
     for (;;) {
         unsigned item = 0;
         if (lane == 0) item = atomicAdd(&a.cnt->head_small, 1u);
@@ -465,44 +533,65 @@ __global__ void __launch_bounds__(PS_THREADS) k_twohop_small(TwohopArgs a) {
                        if (!tab_insert(keys, vals, hs, w, pass1_add(sdiff, bit))) ovf = true;
                    });
         __syncwarp();
-        uint32_t ncw = 0, npaper = 0;
+        uint32_t ncw = 0, nrow = 0, npaper = 0;
+        RowInfo rst;
+        U128 sum;
         if (__any_sync(FULL, ovf)) {
             if (lane == 0) atomicOr(&a.cnt->err, CERR_HASH);
         } else {
             for (uint32_t base = 0; base < hs; base += 32) {
                 uint32_t i = base + lane;
-                bool cand = false, pap = false;
+                bool same = false, diff = false, pap = false;
                 unsigned long long v = 0;
                 if (i < hs && keys[i] != EMPTY) {
                     v = vals[i];
                     pap = STATS && (v & M21) >= (unsigned long long)l;
-                    cand = keep_candidate(v, l);
+                    same = keep_same(v, l);
+                    diff = keep_diff(v, l);
                 }
-                uint32_t bal = __ballot_sync(FULL, cand);
-                if (cand) vals[i] = cand_value(v, ncw + __popc(bal & lt));
-                ncw += __popc(bal);
-                npaper += __popc(__ballot_sync(FULL, pap));
+                const uint32_t bs = __ballot_sync(FULL, same), bd = __ballot_sync(FULL, diff);
+                if (same || diff) vals[i] = cand_value(v, nrow + __popc(bs & lt) + __popc(bd & lt));
+                if (a.single) {
+                    if (same) binom_add(sum, use_count(v) - diff_count(v), l, &a.cnt->err);
+                    if (diff) binom_add(sum, diff_count(v), l, &a.cnt->err);
+                } else {
+                    if (same) rst.add(use_count(v) - diff_count(v));
+                    if (diff) rst.add(diff_count(v));
+                }
+                ncw += __popc(bs | bd);
+                nrow += __popc(bs) + __popc(bd);
+                if (STATS) npaper += __popc(__ballot_sync(FULL, pap));
             }
             __syncwarp();
-            if (ncw > rsv) {
+            if (a.single) {
+                leaves += nrow;
+                tested += ncw;
+                if (nrow) {
+                    const U128 ws = warp_sum_u128(sum, &a.cnt->err);
+                    if (split_totals) {
+                        if (lane == 0) add_totals(a.tot, r, ws);
+                    } else if (total.add(ws)) {
+                        atomicOr(&a.cnt->err, CERR_OVERFLOW);
+                    }
+                }
+            } else if (nrow > rsv) {
                 if (lane == 0) atomicOr(&a.cnt->err, CERR_RESERVE);
-                ncw = 0;
-            }
-            if (ncw > 0) {
-                // The pool is zeroed on the stream before the 2-hop launches,
-                // so the masks are built by atomicOr alone (no zeroing stores
-                // of this kernel ever meet its atomics on the same words).
+                ncw = nrow = 0;
+            } else if (nrow > 0) {
+                rst.warp_sum();
+                // The small anchors' part of the pool is zeroed on the stream
+                // before the 2-hop launches, so the rows are built by atomicOr
+                // alone (no zeroing stores of this kernel ever meet its
+                // atomics on the same words).
                 visit_warp(ebase, d, true, a.A_ent, a.A_pos, a.A_bit, a.B_off, a.B_ent,
                            [&](uint32_t w, uint32_t sdiff, uint32_t bit) {
                                int sl = tab_find(keys, hs, w);
                                if (sl < 0) return;
                                unsigned long long v = vals[sl];
                                if (!(v & CAND)) return;
-                               uint32_t c = cand_index(v);
-                               uint32_t m = 1u << (bit & 31);
-                               size_t wd = bit >> 5;
-                               atomicOr(&region[wd * rsv + c], m);
-                               if (sdiff) atomicOr(&region[(W + wd) * rsv + c], m);
+                               const uint32_t row = row_index(v, sdiff, l);
+                               if (row != EMPTY)
+                                   atomicOr(&region[(size_t)(bit >> 5) * rsv + row], 1u << (bit & 31));
                            });
                 if (a.check) {
                     __syncwarp();
@@ -510,10 +599,7 @@ __global__ void __launch_bounds__(PS_THREADS) k_twohop_small(TwohopArgs a) {
                     for (uint32_t i = lane; i < hs; i += 32) {
                         if (keys[i] == EMPTY) continue;
                         unsigned long long v = vals[i];
-                        if (!(v & CAND)) continue;
-                        uint32_t c = cand_index(v);
-                        if (!masks_match(region + c, region + (size_t)W * rsv + c, rsv, W, v, true))
-                            bad = true;
+                        if ((v & CAND) && !rows_match(region, rsv, W, v, l, true)) bad = true;
                     }
                     if (__any_sync(FULL, bad) && lane == 0) atomicOr(&a.cnt->err, CERR_MASK);
                 }
@@ -521,10 +607,17 @@ __global__ void __launch_bounds__(PS_THREADS) k_twohop_small(TwohopArgs a) {
         }
         if (lane == 0) {
             a.ncand[r] = ncw;
+            a.nrow[r] = nrow;
+            a.rinfo[r] = rst;
             if (STATS) a.npaper[r] = npaper;
         }
         wedges += e_vis;
         __syncwarp();
+    }
+    if (lane == 0) {
+        add_totals(a.tot, 0, total);
+        if (tested) atomicAdd(&a.cnt->tested, tested);
+        if (leaves) atomicAdd(&a.cnt->leaves, leaves);
     }
     if (lane == 0 && wedges) atomicAdd(&a.cnt->wedges, wedges);
 }
@@ -676,44 +769,59 @@ __global__ void __launch_bounds__(PL_THREADS) k_twohop_large(TwohopArgs a) {
     uint32_t *stage = (uint32_t *)(smem_raw + PL_OFF_STAGE);
     __shared__ unsigned long long warp_tot[PL_WARPS];
     __shared__ unsigned long long s_total;
-    __shared__ unsigned s_item, s_ncw, s_paper, s_ovf;
+    __shared__ unsigned s_item, s_ncw, s_nrw, s_paper, s_ovf;
+    __shared__ float s_pops;
+    __shared__ unsigned s_longest;
     __shared__ uint32_t s_bcnt[PL_MAXCLS];
     const int tid = threadIdx.x, lane = tid & 31;
     const int l = a.l;
     unsigned long long *bucket =
         a.bucket ? a.bucket + (size_t)blockIdx.x * a.bucket_slot : nullptr;
-    unsigned long long wedges = 0;
+    const bool split_totals = a.tot.per_anchor || a.tot.per_graph;
+    unsigned long long wedges = 0, tested = 0, leaves = 0;
+    U128 sum;  // one partner: this thread's share of the anchor's sum
+    RowInfo rst;
 
-    // Candidate filter over the table, window-local indices in vals.
+    // Candidate filter over the table, window-local row indices in vals.
     auto extract = [&](uint32_t hs) {
         for (uint32_t base = 0; base < hs; base += PL_THREADS) {
             uint32_t i = base + tid;
-            bool cand = false, pap = false;
+            bool same = false, diff = false, pap = false;
+            unsigned long long v = 0;
             if (i < hs && keys[i] != EMPTY) {
-                unsigned long long v = vals[i];
+                v = vals[i];
                 pap = STATS && (v & M21) >= (unsigned long long)l;
-                cand = keep_candidate(v, l);
+                same = keep_same(v, l);
+                diff = keep_diff(v, l);
             }
-            uint32_t bal = __ballot_sync(FULL, cand);
-            uint32_t pb = __ballot_sync(FULL, pap);
+            const uint32_t bs = __ballot_sync(FULL, same), bd = __ballot_sync(FULL, diff);
+            const uint32_t pb = __ballot_sync(FULL, pap);
             uint32_t wbase = 0;
-            if (lane == 0 && bal) wbase = atomicAdd(&s_ncw, (unsigned)__popc(bal));
+            if (lane == 0 && (bs | bd)) {
+                wbase = atomicAdd(&s_nrw, (unsigned)(__popc(bs) + __popc(bd)));
+                atomicAdd(&s_ncw, (unsigned)__popc(bs | bd));
+            }
             if (lane == 0 && pb) atomicAdd(&s_paper, (unsigned)__popc(pb));
             wbase = __shfl_sync(FULL, wbase, 0);
-            if (cand) vals[i] = cand_value(vals[i], wbase + __popc(bal & ((1u << lane) - 1u)));
+            const uint32_t lt = (1u << lane) - 1u;
+            if (same || diff) vals[i] = cand_value(v, wbase + __popc(bs & lt) + __popc(bd & lt));
+            if (a.single) {
+                if (same) binom_add(sum, use_count(v) - diff_count(v), l, &a.cnt->err);
+                if (diff) binom_add(sum, diff_count(v), l, &a.cnt->err);
+            } else {
+                if (same) rst.add(use_count(v) - diff_count(v));
+                if (diff) rst.add(diff_count(v));
+            }
         }
     };
-    auto set_bits = [&](uint32_t hs, uint32_t *bb, uint32_t bstride, uint32_t W, uint32_t w,
-                        uint32_t sdiff, uint32_t bit) {
+    auto set_bits = [&](uint32_t hs, uint32_t *bb, uint32_t bstride, uint32_t w, uint32_t sdiff,
+                        uint32_t bit) {
         int sl = tab_find(keys, hs, w);
         if (sl < 0) return;
         unsigned long long v = vals[sl];
         if (!(v & CAND)) return;
-        uint32_t c = cand_index(v);
-        uint32_t m = 1u << (bit & 31);
-        size_t wd = bit >> 5;
-        atomicOr(&bb[wd * bstride + c], m);
-        if (sdiff) atomicOr(&bb[(W + wd) * bstride + c], m);
+        const uint32_t row = row_index(v, sdiff, l);
+        if (row != EMPTY) atomicOr(&bb[(size_t)(bit >> 5) * bstride + row], 1u << (bit & 31));
     };
 
     for (;;) {
@@ -733,8 +841,13 @@ __global__ void __launch_bounds__(PL_THREADS) k_twohop_large(TwohopArgs a) {
         const long long c0 = clock64();
         unsigned long long reads = 0;
         int path = 0;
-        uint32_t nc = 0, npaper = 0;
+        uint32_t nc = 0, nr = 0, npaper = 0;
         bool failed = false;
+        rst = RowInfo();
+        if (tid == 0) {
+            s_pops = 0.f;
+            s_longest = 0;
+        }
 
         // Window bookkeeping shared by both strategies: after the table of
         // one window holds its counts, keep candidates and write their bits.
@@ -742,19 +855,19 @@ __global__ void __launch_bounds__(PL_THREADS) k_twohop_large(TwohopArgs a) {
         auto finish_window = [&](uint32_t hs, auto &&pass2) -> bool {
             extract(hs);
             __syncthreads();
-            const uint32_t ncw = s_ncw;
+            const uint32_t ncw = s_ncw, nrw = s_nrw;
             npaper += s_paper;
-            if (ncw > 0) {
-                if (nc + ncw > rsv) {
+            if (nrw > 0 && !a.single) {
+                if (nr + nrw > rsv) {
                     if (tid == 0) atomicOr(&a.cnt->err, CERR_RESERVE);
                     __syncthreads();
                     return false;
                 }
-                const bool staged = 2ull * W * ncw <= (unsigned long long)PL_STAGE_WORDS;
-                uint32_t *bb = staged ? stage : region + nc;
-                const uint32_t bstride = staged ? ncw : rsv;
-                for (uint32_t i = tid; i < 2 * W * ncw; i += PL_THREADS) {
-                    uint32_t wd = i / ncw, c = i % ncw;
+                const bool staged = (unsigned long long)W * nrw <= (unsigned long long)PL_STAGE_WORDS;
+                uint32_t *bb = staged ? stage : region + nr;
+                const uint32_t bstride = staged ? nrw : rsv;
+                for (uint32_t i = tid; i < W * nrw; i += PL_THREADS) {
+                    uint32_t wd = i / nrw, c = i % nrw;
                     bb[(size_t)wd * bstride + c] = 0;
                 }
                 __syncthreads();
@@ -765,22 +878,20 @@ __global__ void __launch_bounds__(PL_THREADS) k_twohop_large(TwohopArgs a) {
                     for (uint32_t i = tid; i < hs; i += PL_THREADS) {
                         if (keys[i] == EMPTY) continue;
                         const unsigned long long v = vals[i];
-                        if (!(v & CAND)) continue;
-                        const uint32_t c = cand_index(v);
-                        if (!masks_match(bb + c, bb + (size_t)W * bstride + c, bstride, W, v, !staged))
-                            bad = true;
+                        if ((v & CAND) && !rows_match(bb, bstride, W, v, l, !staged)) bad = true;
                     }
                     if (bad) atomicOr(&a.cnt->err, CERR_MASK);
                     __syncthreads();
                 }
                 if (staged) {
-                    for (uint32_t i = tid; i < 2 * W * ncw; i += PL_THREADS) {
-                        uint32_t wd = i / ncw, c = i % ncw;
-                        region[(size_t)wd * rsv + nc + c] = stage[i];
+                    for (uint32_t i = tid; i < W * nrw; i += PL_THREADS) {
+                        uint32_t wd = i / nrw, c = i % nrw;
+                        region[(size_t)wd * rsv + nr + c] = stage[i];
                     }
                 }
-                nc += ncw;
             }
+            nc += ncw;
+            nr += nrw;
             __syncthreads();
             return true;
         };
@@ -791,6 +902,7 @@ __global__ void __launch_bounds__(PL_THREADS) k_twohop_large(TwohopArgs a) {
             }
             if (tid == 0) {
                 s_ncw = 0;
+                s_nrw = 0;
                 s_paper = 0;
                 s_ovf = 0;
             }
@@ -817,7 +929,7 @@ __global__ void __launch_bounds__(PL_THREADS) k_twohop_large(TwohopArgs a) {
                 failed = !finish_window(hs, [&](uint32_t *bb, uint32_t bstride) {
                     visit_block(ebase, d, true, 0, 0, a, pst, ppre, pinfo, warp_tot, &s_total,
                                 [&](uint32_t w, uint32_t sdiff, uint32_t bit) {
-                                    set_bits(hs, bb, bstride, W, w, sdiff, bit);
+                                    set_bits(hs, bb, bstride, w, sdiff, bit);
                                 });
                 });
             }
@@ -871,7 +983,9 @@ __global__ void __launch_bounds__(PL_THREADS) k_twohop_large(TwohopArgs a) {
                 if (n == 0) continue;
                 // one window for the class; when its distinct partners overflow
                 // the table, 2^lg2 windows over its sub-classes
-                const uint32_t nc0 = nc, np0 = npaper;
+                const uint32_t nc0 = nc, nr0 = nr, np0 = npaper;
+                const U128 sum0 = sum;
+                const RowInfo rst0 = rst;
                 for (int lg2 = 0; !failed; lg2++) {
                     if (lg2 > 8) {
                         if (tid == 0) atomicOr(&a.cnt->err, CERR_HASH);
@@ -883,7 +997,10 @@ __global__ void __launch_bounds__(PL_THREADS) k_twohop_large(TwohopArgs a) {
                     hs = hs < 64 ? 64 : (hs > PL_HS ? PL_HS : hs);
                     hs = cap_slots(hs, a);
                     nc = nc0;
+                    nr = nr0;
                     npaper = np0;
+                    sum = sum0;
+                    rst = rst0;
                     bool over = false;
                     for (uint32_t sub = 0; sub < (1u << lg2) && !failed; sub++) {
                         __syncthreads();
@@ -909,7 +1026,7 @@ __global__ void __launch_bounds__(PL_THREADS) k_twohop_large(TwohopArgs a) {
                                 if (bi == (uint32_t)BE_NOBIT) continue;
                                 const uint32_t w = (uint32_t)e & VMASK;
                                 if (lg2 && subclass_of(w, lgb, lg2) != sub) continue;
-                                set_bits(hs, bb, bstride, W, w, (uint32_t)(e >> 31) & 1u, bi);
+                                set_bits(hs, bb, bstride, w, (uint32_t)(e >> 31) & 1u, bi);
                             }
                         });
                     }
@@ -920,8 +1037,7 @@ __global__ void __launch_bounds__(PL_THREADS) k_twohop_large(TwohopArgs a) {
         }
         if (!bucketed && !failed && e_vis > (unsigned long long)a.wcap) {
             // re-read windows: every pass over the 2-hop keeps one hash class
-            nc = 0;
-            npaper = 0;
+            const U128 sum0 = sum;
             int lg_nw = 0;
             while (((unsigned long long)a.wcap << lg_nw) < e_vis) lg_nw++;
             path = 2;
@@ -932,8 +1048,10 @@ __global__ void __launch_bounds__(PL_THREADS) k_twohop_large(TwohopArgs a) {
                 uint32_t hs = (uint32_t)((2 * per + 31) & ~31ull);
                 hs = hs < 64 ? 64 : (hs > PL_HS ? PL_HS : hs);
                 hs = cap_slots(hs, a);
-                nc = 0;
+                nc = nr = 0;
                 npaper = 0;
+                sum = sum0;
+                rst = RowInfo();
                 bool restart = false;
                 for (uint32_t cls = 0; cls < nw && !failed; cls++) {
                     clear_table(hs);
@@ -949,7 +1067,7 @@ __global__ void __launch_bounds__(PL_THREADS) k_twohop_large(TwohopArgs a) {
                     failed = !finish_window(hs, [&](uint32_t *bb, uint32_t bstride) {
                         visit_block(ebase, d, true, lg_nw, cls, a, pst, ppre, pinfo, warp_tot,
                                     &s_total, [&](uint32_t w, uint32_t sdiff, uint32_t bit) {
-                                        set_bits(hs, bb, bstride, W, w, sdiff, bit);
+                                        set_bits(hs, bb, bstride, w, sdiff, bit);
                                     });
                     });
                 }
@@ -962,9 +1080,31 @@ __global__ void __launch_bounds__(PL_THREADS) k_twohop_large(TwohopArgs a) {
                 __syncthreads();
             }
         }
-        if (failed) nc = 0;
+        if (failed) nc = nr = 0;
+        if (!a.single) {
+            rst.warp_sum();
+            if (lane == 0) {
+                atomicAdd(&s_pops, rst.pops);
+                atomicMax(&s_longest, rst.longest);
+            }
+            __syncthreads();
+        }
+        if (a.single && split_totals) {
+            const U128 ws = warp_sum_u128(sum, &a.cnt->err);
+            if (lane == 0) add_totals(a.tot, r, ws);
+            sum = U128();
+        }
         if (tid == 0) {
             a.ncand[r] = nc;
+            a.nrow[r] = nr;
+            RowInfo ri;
+            ri.pops = s_pops;
+            ri.longest = s_longest;
+            a.rinfo[r] = ri;
+            if (a.single) {
+                tested += nc;
+                leaves += nr;
+            }
             if (STATS) a.npaper[r] = npaper;
             wedges += e_vis;
             atomicAdd(&a.cnt->tw_reads, reads);
@@ -973,8 +1113,14 @@ __global__ void __launch_bounds__(PL_THREADS) k_twohop_large(TwohopArgs a) {
         }
         __syncthreads();
     }
+    if (a.single && !split_totals) {
+        const U128 ws = warp_sum_u128(sum, &a.cnt->err);
+        if (lane == 0) add_totals(a.tot, 0, ws);
+    }
     if (tid == 0) {
         if (wedges) atomicAdd(&a.cnt->wedges, wedges);
+        if (tested) atomicAdd(&a.cnt->tested, tested);
+        if (leaves) atomicAdd(&a.cnt->leaves, leaves);
         const unsigned long long t = global_ns();
         atomicMax(&a.cnt->tw_fin_max, t);
         atomicMax(&a.cnt->tw_fin_min_n, ~t);
@@ -999,1535 +1145,7 @@ __global__ void k_group_offsets(const uint32_t *order, const int64_t *cum, int64
         pool_off[order[i]] = cum[i] - cum[a];
 }
 
-// ------------------------------------------------------------------ items
-
-// Saturating binom(n, k) in 64 bits (planning cost only).
-__device__ __forceinline__ unsigned long long binom_sat(unsigned long long n, int k) {
-    if ((long long)n < k) return 0;
-    unsigned long long r = 1;
-    for (int i = 1; i <= k; i++) {
-        unsigned long long f = n - k + i;
-        if (r > 0xFFFFFFFFFFFFFFFFull / f) return 0xFFFFFFFFFFFFFFFFull;
-        r = r * f / i;
-    }
-    return r;
-}
-
-// A work item of one anchor. Candidate side: rows [i0, i1) of first
-// partners, all their units when u1 == 0, else units [u0, u1) of row i0.
-// Position side (u1 == POS_ITEM): first positions [i0, i1).
-struct Item {
-    uint32_t anchor, i0, i1, u0, u1;
-};
-constexpr uint32_t POS_ITEM = 0xFFFFFFFFu;
-constexpr int POS_MAX_WORDS = 128;  // candidate words of a position-side mask (4 per lane)
-
-constexpr int ROWS_MAX = 1024;
-constexpr int PB_SMEM_WORDS_PLAN = 24576;  // staged words of the tuple kernel (PB_SMEM_WORDS)
-
-struct ItemArgs {
-    const uint32_t *ncand, *npaper, *dprime;
-    const uint32_t *order;  // anchors of the group: order[begin .. begin + nX)
-    int64_t begin;
-    int64_t nX;             // anchors in the group
-    int R, l;
-    int method;  // 0: cheaper side per anchor, 1: candidate side, 2: position side where it fits
-    unsigned long long pos_unit;  // cost of one position-side prefix node per candidate word-lane
-    unsigned long long item_cost;
-    const int64_t *item_off;  // emit pass
-    int64_t *item_cnt;        // count pass (nX + 1 entries)
-    Item *items;
-    uint32_t *ikey, *ival;
-    Counters *cnt;
-    // tensor-core pair step (two partners, candidate side, wide masks)
-    int tc_on;
-    uint32_t tc_min_w, tc_min_nc;
-    uint32_t *tc_list;
-};
-
-__device__ __forceinline__ unsigned long long row_cost(uint32_t nc, uint32_t i, int R, uint32_t W) {
-    if (R == 1) return 0;
-    unsigned long long t = binom_sat(nc - 1 - i, R - 1);
-    unsigned long long c = t * W;
-    return (W && c / W != t) ? 0xFFFFFFFFFFFFFFFFull : c;
-}
-
-__device__ __forceinline__ unsigned long long unit_cost(uint32_t nc, uint32_t i, uint32_t u, int R,
-                                                        uint32_t W) {
-    if (R <= 2) return 32ull * W;
-    unsigned long long s = 0;
-    uint32_t j0 = i + 1 + 32 * u;
-    for (uint32_t j = j0; j < j0 + 32 && j < nc; j++) {
-        unsigned long long t = binom_sat(nc - 1 - j, R - 2);
-        s = (s + t < s) ? 0xFFFFFFFFFFFFFFFFull : s + t;
-    }
-    unsigned long long c = s * W;
-    return (W && c / W != s) ? 0xFFFFFFFFFFFFFFFFull : c;
-}
-
-// Position-side enumeration of one anchor (see k_tuples): l-subsets Q of the
-// anchor's useful positions, each with N_Q candidates whose same-sign or
-// different-sign part of L[w] contains Q; the anchor adds sum over Q of
-// binom(N_Q, R). Cost in the candidate-side units (mask words x tuples):
-// 32 lanes x 3 steps x words per lane for every prefix node.
-__device__ __forceinline__ bool pos_fits(uint32_t nc, uint32_t dp, int l) {
-    const uint32_t wc = (nc + 31) / 32;
-    return dp >= (uint32_t)l && wc <= (uint32_t)POS_MAX_WORDS &&
-           2ull * dp * (wc | 1u) <= (unsigned long long)PB_SMEM_WORDS_PLAN;
-}
-
-__device__ __forceinline__ unsigned long long pos_row_cost(uint32_t nc, uint32_t dp, uint32_t q1,
-                                                           int l, unsigned long long unit) {
-    const unsigned long long wpl = ((nc + 31) / 32 + 31) / 32;
-    unsigned long long nodes = 0;
-    for (int i = 0; i < l; i++) {
-        unsigned long long t = binom_sat(dp - 1 - q1, i);
-        nodes = (nodes + t < nodes) ? 0xFFFFFFFFFFFFFFFFull : nodes + t;
-    }
-    unsigned long long c = nodes * unit * wpl;
-    return (c / (unit * wpl) != nodes) ? 0xFFFFFFFFFFFFFFFFull : c;
-}
-
-__device__ __forceinline__ unsigned long long pos_cost(uint32_t nc, uint32_t dp, int l,
-                                                       unsigned long long unit) {
-    const unsigned long long wpl = ((nc + 31) / 32 + 31) / 32;
-    unsigned long long nodes = 0;
-    for (int i = 1; i <= l; i++) {
-        unsigned long long t = binom_sat(dp, i);
-        nodes = (nodes + t < nodes) ? 0xFFFFFFFFFFFFFFFFull : nodes + t;
-    }
-    unsigned long long c = nodes * unit * wpl;
-    return (c / (unit * wpl) != nodes) ? 0xFFFFFFFFFFFFFFFFull : c;
-}
-
-__device__ __forceinline__ unsigned long long cand_cost(uint32_t nc, uint32_t W, int R) {
-    unsigned long long t = binom_sat(nc, R);
-    unsigned long long c = t * (W ? W : 1);
-    return (W > 1 && c / W != t) ? 0xFFFFFFFFFFFFFFFFull : c;
-}
-
-// True when the anchor takes the position side (cheaper, or forced).
-__device__ __forceinline__ bool use_pos(uint32_t nc, uint32_t dp, int R, int l, int method,
-                                        unsigned long long unit) {
-    if (method == 1 || nc < (uint32_t)R || !pos_fits(nc, dp, l)) return false;
-    if (method == 2) return true;
-    return pos_cost(nc, dp, l, unit) < cand_cost(nc, (dp + 31) / 32, R);
-}
-
-// True when the anchor's pairs go to the tensor-core kernel (tc_pairs.cu):
-// two partners, candidate side, at least tc_min_w mask words and tc_min_nc
-// candidates.
-__device__ __forceinline__ bool tc_take(const ItemArgs &a, uint32_t nc, uint32_t dp) {
-    return a.tc_on && a.R == 2 && nc >= a.tc_min_nc && (dp + 31) / 32 >= a.tc_min_w &&
-           !use_pos(nc, dp, a.R, a.l, a.method, a.pos_unit);
-}
-
-// Anchor cost, anchor tuple counts, tensor-core anchor list. Thread per anchor.
-__global__ void k_anchor_cost(ItemArgs a) {
-    U128 tp, to;
-    unsigned long long cand = 0, cost = 0;
-    for (int64_t ix = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; ix < a.nX;
-         ix += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t r = a.order[a.begin + ix];
-        uint32_t nc = a.ncand[r];
-        uint32_t W = (a.dprime[r] + 31) / 32;
-        if (a.npaper) {
-            uint32_t np = a.npaper[r];
-            cand += np;
-            if (np >= (uint32_t)a.R) {
-                // binom(np, R) exactly: np < 2^32, R <= 7, fits 128 bits
-                unsigned long long lo = 1, hi = 0;
-                for (int i = 1; i <= a.R; i++) {
-                    unsigned long long f = np - a.R + i;
-                    unsigned g = gcd_u32((unsigned)(f % (unsigned)i), (unsigned)i);
-                    if (g == 0) g = i;
-                    div_u128_small(lo, hi, i / g);
-                    mul_u128_u64(lo, hi, f / g);
-                }
-                U128 t;
-                t.lo = lo;
-                t.hi = hi;
-                tp.add(t);
-            }
-        } else {
-            cand += nc;
-        }
-        if (nc >= (uint32_t)a.R) {
-            unsigned long long t = binom_sat(nc, a.R);
-            to.add(t);
-            if (tc_take(a, nc, a.dprime[r])) {
-                a.tc_list[atomicAdd(&a.cnt->n_tc, 1u)] = r;
-            } else {
-                unsigned long long c = use_pos(nc, a.dprime[r], a.R, a.l, a.method, a.pos_unit)
-                                           ? pos_cost(nc, a.dprime[r], a.l, a.pos_unit)
-                                           : cand_cost(nc, W, a.R);
-                cost = (cost + c < cost) ? 0xFFFFFFFFFFFFFFFFull : cost + c;
-            }
-        }
-    }
-    tp = warp_sum_u128(tp, nullptr);
-    to = warp_sum_u128(to, nullptr);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        cand += __shfl_xor_sync(FULL, cand, o);
-        unsigned long long t = __shfl_xor_sync(FULL, cost, o);
-        cost = (cost + t < cost) ? 0xFFFFFFFFFFFFFFFFull : cost + t;
-    }
-    if ((threadIdx.x & 31) == 0) {
-        atomic_add_u128(a.cnt->tuples_paper, tp.lo, tp.hi, nullptr);
-        atomic_add_u128(a.cnt->tuples_ours, to.lo, to.hi, nullptr);
-        atomicAdd(&a.cnt->candidates, cand);
-        atomicAdd(&a.cnt->cost_total, cost);
-    }
-}
-
-// Split each anchor's tuple space into items. EMIT == false counts them.
-template <bool EMIT>
-__global__ void k_items(ItemArgs a) {
-    for (int64_t ix = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; ix < a.nX;
-         ix += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t r = a.order[a.begin + ix];
-        const uint32_t nc = a.ncand[r];
-        const int R = a.R;
-        int64_t n = 0;
-        int64_t out = EMIT ? a.item_off[ix] : 0;
-        const uint32_t W = (a.dprime[r] + 31) / 32;
-        auto emit = [&](uint32_t i0, uint32_t i1, uint32_t u0, uint32_t u1, unsigned long long c) {
-            if (EMIT) {
-                Item it;
-                it.anchor = (uint32_t)r;
-                it.i0 = i0;
-                it.i1 = i1;
-                it.u0 = u0;
-                it.u1 = u1;
-                a.items[out + n] = it;
-                uint32_t c32 = c < 0xFFFFFFFEull ? (uint32_t)c : 0xFFFFFFFEu;
-                a.ikey[out + n] = 0xFFFFFFFEu - c32;
-                a.ival[out + n] = (uint32_t)(out + n);
-            }
-            n++;
-        };
-        const uint32_t dp = a.dprime[r];
-        if (nc >= (uint32_t)R && nc > 0 && tc_take(a, nc, dp)) {
-            // the tensor-core kernel takes this anchor's pairs: no items
-        } else if (nc >= (uint32_t)R && nc > 0 && use_pos(nc, dp, R, a.l, a.method, a.pos_unit)) {
-            const uint32_t rows = dp - a.l + 1;
-            const unsigned long long cap = 4 * a.item_cost;
-            uint32_t rb = 0;
-            unsigned long long acc = 0;
-            for (uint32_t q1 = 0; q1 < rows; q1++) {
-                unsigned long long c = pos_row_cost(nc, dp, q1, a.l, a.pos_unit);
-                if (q1 > rb && (acc + c > cap || q1 - rb >= (uint32_t)ROWS_MAX)) {
-                    emit(rb, q1, 0, POS_ITEM, acc);
-                    rb = q1;
-                    acc = 0;
-                }
-                acc = (acc + c < acc) ? 0xFFFFFFFFFFFFFFFFull : acc + c;
-            }
-            emit(rb, rows, 0, POS_ITEM, acc);
-        } else if (nc >= (uint32_t)R && nc > 0) {
-            if (R == 1) {
-                uint32_t units = (nc + 31) / 32;
-                unsigned long long per = 32ull * W, acc = 0;
-                uint32_t u0 = 0;
-                for (uint32_t u = 0; u < units; u++) {
-                    if (acc > 0 && acc + per > a.item_cost) {
-                        emit(0, 1, u0, u, acc);
-                        u0 = u;
-                        acc = 0;
-                    }
-                    acc += per;
-                }
-                emit(0, 1, u0, units, acc);
-            } else {
-                const uint32_t rows = nc - R + 1;
-                uint32_t rb = 0;
-                unsigned long long acc = 0;
-                for (uint32_t i = 0; i < rows; i++) {
-                    unsigned long long ci = row_cost(nc, i, R, W);
-                    if (ci > a.item_cost) {
-                        if (i > rb) emit(rb, i, 0, 0, acc);
-                        uint32_t units = (nc - 1 - i + 31) / 32;
-                        uint32_t u0 = 0;
-                        unsigned long long ua = 0;
-                        for (uint32_t u = 0; u < units; u++) {
-                            unsigned long long cu = unit_cost(nc, i, u, R, W);
-                            if (ua > 0 && ua + cu > a.item_cost) {
-                                emit(i, i + 1, u0, u, ua);
-                                u0 = u;
-                                ua = 0;
-                            }
-                            ua = (ua + cu < ua) ? 0xFFFFFFFFFFFFFFFFull : ua + cu;
-                        }
-                        emit(i, i + 1, u0, units, ua);
-                        rb = i + 1;
-                        acc = 0;
-                    } else {
-                        if (i > rb && (acc + ci > a.item_cost || i - rb >= (uint32_t)ROWS_MAX)) {
-                            emit(rb, i, 0, 0, acc);
-                            rb = i;
-                            acc = 0;
-                        }
-                        acc += ci;
-                    }
-                }
-                if (rows > rb) emit(rb, rows, 0, 0, acc);
-            }
-        }
-        if (!EMIT) a.item_cnt[ix] = n;
-    }
-    if (!EMIT && blockIdx.x == 0 && threadIdx.x == 0) a.item_cnt[a.nX] = 0;
-}
-
-// Inputs of the tensor-core plan: the listed anchors' sizes and pool offsets.
-__global__ void k_tc_gather(const uint32_t *list, unsigned n, const uint32_t *ncand,
-                            const uint32_t *dprime, const uint32_t *rsv_c, const int64_t *pool_off,
-                            TcInput *out) {
-    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const uint32_t r = list[i];
-        TcInput t;
-        t.r = r;
-        t.nc = ncand[r];
-        t.W = (dprime[r] + 31) / 32;
-        t.rsv = rsv_c[r];
-        t.pool_off = pool_off[r];
-        out[i] = t;
-    }
-}
-
-// ------------------------------------------------------------------ tuples
-
-constexpr int PB_THREADS = 256;
-constexpr int PB_WARPS = PB_THREADS / 32;
-constexpr int PB_SMEM_WORDS = PB_SMEM_WORDS_PLAN;  // 96 KB of staged words
-constexpr size_t PB_SMEM = PB_SMEM_WORDS * 4;
-constexpr int SCRATCH_SLOTS = 7;  // per-warp mask slots for wide anchors (>= max(R, 6))
-
-struct TupleArgs {
-    const uint32_t *ncand, *dprime, *rsv_c;
-    const int64_t *pool_off;
-    const uint32_t *pool;
-    const Item *items;
-    const uint32_t *iorder;
-    Counters *cnt;
-    unsigned long long *per_anchor;  // u128 per anchor rank, or null
-    unsigned long long *per_graph;   // u128 per graph of a batch, or null
-    const int64_t *graph_x0;         // first anchor rank of each graph (n_graphs + 1)
-    int n_graphs;
-    uint32_t *wide_scratch;          // per warp: R * wmax words
-    uint32_t wmax;
-    int l;
-};
-
-// Per-lane work tally of the tuple kernel (the algorithmic operations: one
-// AND+POPC per mask word of every tested tuple, 2^R masked POPCs per word of
-// every tuple that reaches the type count).
-struct Acc {
-    U128 sum;
-    unsigned long long tested = 0, leaves = 0, words = 0;
-};
-
-constexpr int BINOM_TBL = 256;
-
-// Dynamic shared memory of the tuple kernel (staged masks) and its binomial
-// table binom(x, l) for x <= BINOM_TBL (binom(256, 8) < 2^64).
-extern __shared__ __align__(16) uint32_t sm_dyn[];
-__shared__ unsigned long long s_bt[BINOM_TBL + 1];
-
-// Views of an anchor's candidate masks: P(w, c) and D(w, c), word-major.
-// MasksS: staged in the dynamic shared array (32-bit offsets, shared loads);
-// MasksG: read from the candidate pool in global memory.
-struct MasksS {
-    uint32_t stride, W, nc;
-    __device__ __forceinline__ uint32_t P(uint32_t w, uint32_t c) const {
-        return sm_dyn[w * stride + c];
-    }
-    __device__ __forceinline__ uint32_t D(uint32_t w, uint32_t c) const {
-        return sm_dyn[(W + w) * stride + c];
-    }
-};
-struct MasksG {
-    const uint32_t *base;
-    uint32_t stride, W, nc;
-    __device__ __forceinline__ uint32_t P(uint32_t w, uint32_t c) const {
-        return base[(size_t)w * stride + c];
-    }
-    __device__ __forceinline__ uint32_t D(uint32_t w, uint32_t c) const {
-        return base[(size_t)(W + w) * stride + c];
-    }
-};
-
-// Type counts of a tuple and the binomial sum. T: the lane's common
-// neighbourhood mask; idx[0..R-1]: the tuple's candidate indices.
-template <int R, int WN, class MK>
-__device__ __forceinline__ void leaf_narrow(const MK &m, const uint32_t (&T)[WN],
-                                            const uint32_t (&idx)[R], int l, Acc &acc,
-                                            unsigned *err) {
-    acc.leaves++;
-    acc.words += (unsigned long long)m.W << R;
-    if constexpr (R <= 3) {
-        uint32_t x[1 << R];
-#pragma unroll
-        for (int k = 0; k < (1 << R); k++) x[k] = 0;
-#pragma unroll
-        for (int w = 0; w < WN; w++) {
-            if (w >= (int)m.W) break;
-            uint32_t dd[R];
-#pragma unroll
-            for (int i = 0; i < R; i++) dd[i] = m.D(w, idx[i]);
-#pragma unroll
-            for (int k = 0; k < (1 << R); k++) {
-                uint32_t msk = T[w];
-#pragma unroll
-                for (int i = 0; i < R; i++) msk &= ((k >> i) & 1) ? dd[i] : ~dd[i];
-                x[k] += __popc(msk);
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < (1 << R); k++) binom_add(acc.sum, x[k], l, err);
-    } else {
-        // split T by each partner's type letter, dropping parts below l
-        uint32_t stk[R + 1][WN];
-        int lev[R + 1];
-        int sp = 0;
-#pragma unroll
-        for (int w = 0; w < WN; w++) stk[0][w] = T[w];
-        lev[0] = 0;
-        sp = 1;
-        while (sp > 0) {
-            sp--;
-            int lv = lev[sp];
-            uint32_t cur[WN];
-#pragma unroll
-            for (int w = 0; w < WN; w++) cur[w] = stk[sp][w];
-            if (lv == R) {
-                uint32_t n = 0;
-#pragma unroll
-                for (int w = 0; w < WN; w++) n += __popc(cur[w]);
-                binom_add(acc.sum, n, l, err);
-                continue;
-            }
-            uint32_t a0[WN], a1[WN];
-            uint32_t n0 = 0, n1 = 0;
-#pragma unroll
-            for (int w = 0; w < WN; w++) {
-                uint32_t dw = (w < (int)m.W) ? m.D(w, idx[lv]) : 0u;
-                a0[w] = cur[w] & ~dw;
-                a1[w] = cur[w] & dw;
-                n0 += __popc(a0[w]);
-                n1 += __popc(a1[w]);
-            }
-            if ((int)n0 >= l) {
-#pragma unroll
-                for (int w = 0; w < WN; w++) stk[sp][w] = a0[w];
-                lev[sp] = lv + 1;
-                sp++;
-            }
-            if ((int)n1 >= l) {
-#pragma unroll
-                for (int w = 0; w < WN; w++) stk[sp][w] = a1[w];
-                lev[sp] = lv + 1;
-                sp++;
-            }
-        }
-    }
-}
-
-// Extend a warp-uniform prefix (mask `pre`, indices idx[0..L-2]) by every
-// candidate m >= start, lanes over m.
-template <int L, int R, int WN, class MK>
-__device__ void expand_narrow(const MK &m, const uint32_t (&pre)[WN], uint32_t (&idx)[R],
-                              uint32_t start, int l, Acc &acc, unsigned *err) {
-    const int lane = threadIdx.x & 31;
-    for (uint32_t mb = start; mb < m.nc; mb += 32) {
-        uint32_t c = mb + lane;
-        bool valid = c < m.nc;
-        uint32_t T[WN];
-        uint32_t n = 0;
-#pragma unroll
-        for (int w = 0; w < WN; w++) {
-            T[w] = (valid && w < (int)m.W) ? (pre[w] & m.P(w, c)) : 0u;
-            n += __popc(T[w]);
-        }
-        if (valid) {
-            acc.tested++;
-            acc.words += m.W;
-        }
-        if constexpr (L == R) {
-            if (valid && (int)n >= l) {
-                uint32_t id2[R];
-#pragma unroll
-                for (int i = 0; i < R; i++) id2[i] = idx[i];
-                id2[R - 1] = c;
-                leaf_narrow<R, WN>(m, T, id2, l, acc, err);
-            }
-        } else {
-            bool ok = valid && (int)n >= l && (m.nc - 1 - c) >= (uint32_t)(R - L);
-            uint32_t bal = __ballot_sync(FULL, ok);
-            while (bal) {
-                int s = __ffs(bal) - 1;
-                bal &= bal - 1;
-                uint32_t Ts[WN];
-#pragma unroll
-                for (int w = 0; w < WN; w++) Ts[w] = __shfl_sync(FULL, T[w], s);
-                idx[L - 1] = mb + s;
-                expand_narrow<L + 1, R, WN>(m, Ts, idx, mb + s + 1, l, acc, err);
-            }
-        }
-    }
-}
-
-// One work unit: row i (first partner) and a chunk of 32 second partners;
-// for R == 1 a chunk of 32 single partners.
-template <int R, int WN, class MK>
-__device__ void unit_narrow(const MK &m, uint32_t i, uint32_t jc, int l, Acc &acc,
-                            unsigned *err) {
-    const int lane = threadIdx.x & 31;
-    if constexpr (R == 1) {
-        uint32_t c = jc * 32 + lane;
-        if (c < m.nc) {
-            acc.tested++;
-            acc.words += m.W;
-            uint32_t T[WN];
-            uint32_t n = 0;
-#pragma unroll
-            for (int w = 0; w < WN; w++) {
-                T[w] = (w < (int)m.W) ? m.P(w, c) : 0u;
-                n += __popc(T[w]);
-            }
-            if ((int)n >= l) {
-                uint32_t id[1] = {c};
-                leaf_narrow<1, WN>(m, T, id, l, acc, err);
-            }
-        }
-    } else {
-        uint32_t Pi[WN];
-#pragma unroll
-        for (int w = 0; w < WN; w++) Pi[w] = (w < (int)m.W) ? m.P(w, i) : 0u;
-        uint32_t j = i + 1 + jc * 32 + lane;
-        bool valid = j < m.nc;
-        uint32_t T[WN];
-        uint32_t n = 0;
-#pragma unroll
-        for (int w = 0; w < WN; w++) {
-            T[w] = valid ? (Pi[w] & ((w < (int)m.W) ? m.P(w, j) : 0u)) : 0u;
-            n += __popc(T[w]);
-        }
-        if (valid) {
-            acc.tested++;
-            acc.words += m.W;
-        }
-        if constexpr (R == 2) {
-            if (valid && (int)n >= l) {
-                uint32_t id[2] = {i, j};
-                leaf_narrow<2, WN>(m, T, id, l, acc, err);
-            }
-        } else {
-            bool ok = valid && (int)n >= l && (m.nc - 1 - j) >= (uint32_t)(R - 2);
-            uint32_t bal = __ballot_sync(FULL, ok);
-            uint32_t idx[R];
-            idx[0] = i;
-            while (bal) {
-                int s = __ffs(bal) - 1;
-                bal &= bal - 1;
-                uint32_t Ts[WN];
-#pragma unroll
-                for (int w = 0; w < WN; w++) Ts[w] = __shfl_sync(FULL, T[w], s);
-                uint32_t js = i + 1 + jc * 32 + s;
-                idx[1] = js;
-                expand_narrow<3, R, WN>(m, Ts, idx, js + 1, l, acc, err);
-            }
-        }
-    }
-}
-
-// ---- wide anchors (more than 256 useful positions): masks streamed word by
-// word; warp-uniform prefixes live in a per-warp scratch (level L-1 at
-// pre + (L-2) * wmax).
-
-template <int R, class MK>
-__device__ __forceinline__ void leaf_wide(const MK &m, const uint32_t *pre, uint32_t c,
-                                          const uint32_t (&idx)[R], int l, Acc &acc,
-                                          unsigned *err) {
-    acc.leaves++;
-    acc.words += (unsigned long long)m.W << R;
-    // T = pre AND P(., c); pre == nullptr means T = P(., c)
-    if constexpr (R <= 3) {
-        uint32_t x[1 << R];
-#pragma unroll
-        for (int k = 0; k < (1 << R); k++) x[k] = 0;
-        for (uint32_t w = 0; w < m.W; w++) {
-            uint32_t t = m.P(w, c);
-            if (pre) t &= pre[w];
-            if (!t) continue;
-            uint32_t dd[R];
-#pragma unroll
-            for (int i = 0; i < R; i++) dd[i] = m.D(w, idx[i]);
-#pragma unroll
-            for (int k = 0; k < (1 << R); k++) {
-                uint32_t msk = t;
-#pragma unroll
-                for (int i = 0; i < R; i++) msk &= ((k >> i) & 1) ? dd[i] : ~dd[i];
-                x[k] += __popc(msk);
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < (1 << R); k++) binom_add(acc.sum, x[k], l, err);
-    } else {
-        uint32_t x[1 << R];
-        for (int k = 0; k < (1 << R); k++) x[k] = 0;
-        for (uint32_t w = 0; w < m.W; w++) {
-            uint32_t t = m.P(w, c);
-            if (pre) t &= pre[w];
-            while (t) {
-                int b = __ffs(t) - 1;
-                t &= t - 1;
-                uint32_t kk = 0;
-                for (int i = 0; i < R; i++) kk |= ((m.D(w, idx[i]) >> b) & 1u) << i;
-                x[kk]++;
-            }
-        }
-        for (int k = 0; k < (1 << R); k++) binom_add(acc.sum, x[k], l, err);
-    }
-}
-
-template <int L, int R, class MK>
-__device__ void expand_wide(const MK &m, uint32_t *scratch, uint32_t wmax,
-                            uint32_t (&idx)[R], uint32_t start, int l, Acc &acc, unsigned *err) {
-    const int lane = threadIdx.x & 31;
-    const uint32_t *pre = scratch + (size_t)(L - 2) * wmax;  // prefix of L-1 partners
-    for (uint32_t mb = start; mb < m.nc; mb += 32) {
-        uint32_t c = mb + lane;
-        bool valid = c < m.nc;
-        uint32_t n = 0;
-        if (valid) {
-            acc.tested++;
-            acc.words += m.W;
-            for (uint32_t w = 0; w < m.W; w++) n += __popc(pre[w] & m.P(w, c));
-        }
-        if constexpr (L == R) {
-            if (valid && (int)n >= l) {
-                uint32_t id2[R];
-#pragma unroll
-                for (int i = 0; i < R; i++) id2[i] = idx[i];
-                id2[R - 1] = c;
-                leaf_wide<R>(m, pre, c, id2, l, acc, err);
-            }
-        } else {
-            bool ok = valid && (int)n >= l && (m.nc - 1 - c) >= (uint32_t)(R - L);
-            uint32_t bal = __ballot_sync(FULL, ok);
-            while (bal) {
-                int s = __ffs(bal) - 1;
-                bal &= bal - 1;
-                uint32_t cs = mb + s;
-                uint32_t *nxt = scratch + (size_t)(L - 1) * wmax;
-                __syncwarp();
-                for (uint32_t w = lane; w < m.W; w += 32) nxt[w] = pre[w] & m.P(w, cs);
-                __syncwarp();
-                idx[L - 1] = cs;
-                expand_wide<L + 1, R>(m, scratch, wmax, idx, cs + 1, l, acc, err);
-            }
-        }
-    }
-}
-
-template <int R, class MK>
-__device__ void unit_wide(const MK &m, uint32_t *scratch, uint32_t wmax, uint32_t i,
-                          uint32_t jc, int l, Acc &acc, unsigned *err) {
-    const int lane = threadIdx.x & 31;
-    if constexpr (R == 1) {
-        uint32_t c = jc * 32 + lane;
-        if (c < m.nc) {
-            acc.tested++;
-            acc.words += m.W;
-            uint32_t n = 0;
-            for (uint32_t w = 0; w < m.W; w++) n += __popc(m.P(w, c));
-            if ((int)n >= l) {
-                uint32_t id[1] = {c};
-                leaf_wide<1>(m, nullptr, c, id, l, acc, err);
-            }
-        }
-    } else {
-        // level-1 prefix P(., i) at scratch[0 .. W)
-        __syncwarp();
-        for (uint32_t w = lane; w < m.W; w += 32) scratch[w] = m.P(w, i);
-        __syncwarp();
-        uint32_t j = i + 1 + jc * 32 + lane;
-        bool valid = j < m.nc;
-        uint32_t n = 0;
-        if (valid) {
-            acc.tested++;
-            acc.words += m.W;
-            for (uint32_t w = 0; w < m.W; w++) n += __popc(scratch[w] & m.P(w, j));
-        }
-        if constexpr (R == 2) {
-            if (valid && (int)n >= l) {
-                uint32_t id[2] = {i, j};
-                leaf_wide<2>(m, scratch, j, id, l, acc, err);
-            }
-        } else {
-            bool ok = valid && (int)n >= l && (m.nc - 1 - j) >= (uint32_t)(R - 2);
-            uint32_t bal = __ballot_sync(FULL, ok);
-            uint32_t idx[R];
-            idx[0] = i;
-            while (bal) {
-                int s = __ffs(bal) - 1;
-                bal &= bal - 1;
-                uint32_t js = i + 1 + jc * 32 + s;
-                uint32_t *nxt = scratch + wmax;
-                __syncwarp();
-                for (uint32_t w = lane; w < m.W; w += 32) nxt[w] = scratch[w] & m.P(w, js);
-                __syncwarp();
-                idx[1] = js;
-                expand_wide<3, R>(m, scratch, wmax, idx, js + 1, l, acc, err);
-            }
-        }
-    }
-}
-
-// ---- type parts (R <= 3). By Lemma 1 and its converse, every v of a
-// balanced biclique's other side has the same type relative to the anchor,
-// so a prefix of partners is carried as its type parts: the masks of common
-// neighbours sharing one type vector, kept only while they hold at least l
-// bits. Extending by a partner m splits each part P into P & P_m & ~D_m and
-// P & P_m & D_m; at the last partner each child adds binom(popc, l). Parts
-// below l bits are dropped, which drops only zero binomials.
-
-// Split one part y (already ANDed with P_m) by D_m and add the binomials.
-template <int WN, class MK>
-__device__ __forceinline__ void close_part(const MK &m, const uint32_t (&y)[WN], uint32_t c,
-                                           int l, Acc &acc, unsigned *err) {
-    uint32_t n = 0;
-#pragma unroll
-    for (int w = 0; w < WN; w++) n += __popc(y[w]);
-    acc.words += m.W;
-    if ((int)n < l) return;
-    uint32_t x1 = 0;
-#pragma unroll
-    for (int w = 0; w < WN; w++)
-        if (w < (int)m.W) x1 += __popc(y[w] & m.D(w, c));
-    acc.words += m.W;
-    acc.leaves++;
-    if (n <= (uint32_t)BINOM_TBL) {
-        acc.sum.add(s_bt[x1] + s_bt[n - x1]);
-    } else {
-        binom_add(acc.sum, x1, l, err);
-        binom_add(acc.sum, n - x1, l, err);
-    }
-}
-
-// Close part B against candidate c given S = P_c & ~D_c and T = P_c & D_c:
-// the two children B & S and B & T add binom(., l) each (zero below l).
-// Returns whether the part had at least l common neighbours with c.
-template <int WN>
-__device__ __forceinline__ bool close_st(const uint32_t (&B)[WN], const uint32_t (&S)[WN],
-                                         const uint32_t (&T)[WN], int l, Acc &acc,
-                                         unsigned *err) {
-    uint32_t n0 = 0, n1 = 0;
-#pragma unroll
-    for (int w = 0; w < WN; w++) {
-        n0 += __popc(B[w] & S[w]);
-        n1 += __popc(B[w] & T[w]);
-    }
-    const uint32_t n = n0 + n1;
-    const bool ok = (int)n >= l;
-    if (__any_sync(FULL, ok) && ok) {
-        if (n <= (uint32_t)BINOM_TBL) {
-            acc.sum.add(s_bt[n0] + s_bt[n1]);
-        } else {
-            binom_add(acc.sum, n0, l, err);
-            binom_add(acc.sum, n1, l, err);
-        }
-    }
-    return ok;
-}
-
-template <int WN, class MK>
-__device__ void parts_r1(const MK &m, uint32_t jc, int l, Acc &acc, unsigned *err) {
-    const uint32_t c = jc * 32 + (threadIdx.x & 31);
-    if (c >= m.nc) return;
-    acc.tested++;
-    uint32_t y[WN];
-#pragma unroll
-    for (int w = 0; w < WN; w++) y[w] = w < (int)m.W ? m.P(w, c) : 0u;
-    close_part<WN>(m, y, c, l, acc, err);
-}
-
-// Type parts of candidate i: A0 = P_i & ~D_i (same sign), A1 = P_i & D_i.
-template <int WN, class MK>
-__device__ __forceinline__ uint32_t parts_of(const MK &m, uint32_t i, uint32_t (&A0)[WN],
-                                             uint32_t (&A1)[WN], int l) {
-    uint32_t n0 = 0, n1 = 0;
-#pragma unroll
-    for (int w = 0; w < WN; w++) {
-        uint32_t p = w < (int)m.W ? m.P(w, i) : 0u;
-        uint32_t d = w < (int)m.W ? m.D(w, i) : 0u;
-        A0[w] = p & ~d;
-        A1[w] = p & d;
-        n0 += __popc(A0[w]);
-        n1 += __popc(A1[w]);
-    }
-    return ((int)n0 >= l ? 1u : 0u) | ((int)n1 >= l ? 2u : 0u);
-}
-
-template <int WN, class MK>
-__device__ void parts_r2(const MK &m, uint32_t i, uint32_t jc, int l, Acc &acc,
-                         unsigned *err) {
-    uint32_t A0[WN], A1[WN];
-    const uint32_t va = parts_of<WN>(m, i, A0, A1, l);
-    if (!va) return;
-    const uint32_t j = i + 1 + jc * 32 + (threadIdx.x & 31);
-    const bool jv = j < m.nc;
-    uint32_t S[WN], T[WN];
-#pragma unroll
-    for (int w = 0; w < WN; w++) {
-        const bool in = jv && w < (int)m.W;
-        const uint32_t p = in ? m.P(w, j) : 0u, d = in ? m.D(w, j) : 0u;
-        S[w] = p & ~d;
-        T[w] = p & d;
-    }
-    uint32_t closes = 0, viable = 0;
-    if (va & 1u) {
-        closes++;
-        viable += close_st<WN>(A0, S, T, l, acc, err);
-    }
-    if (va & 2u) {
-        closes++;
-        viable += close_st<WN>(A1, S, T, l, acc, err);
-    }
-    if (jv) {
-        acc.tested++;
-        acc.leaves += viable;
-        acc.words += (unsigned long long)(closes + viable) * m.W;
-    }
-}
-
-template <int WN, class MK>
-__device__ void parts_r3(const MK &m, uint32_t i, uint32_t jc, int l, Acc &acc,
-                         unsigned *err) {
-    const int lane = threadIdx.x & 31;
-    uint32_t A0[WN], A1[WN];
-    const uint32_t va = parts_of<WN>(m, i, A0, A1, l);
-    if (!va) return;
-    const uint32_t j = i + 1 + jc * 32 + lane;
-    const bool valid = j + 1 < m.nc;  // room for a third partner
-    uint32_t vb = 0;
-    if (valid) {
-        acc.tested++;
-        uint32_t n[4] = {0, 0, 0, 0};
-#pragma unroll
-        for (int w = 0; w < WN; w++) {
-            uint32_t p = w < (int)m.W ? m.P(w, j) : 0u;
-            uint32_t d = w < (int)m.W ? m.D(w, j) : 0u;
-            n[0] += __popc(A0[w] & p & ~d);
-            n[1] += __popc(A0[w] & p & d);
-            n[2] += __popc(A1[w] & p & ~d);
-            n[3] += __popc(A1[w] & p & d);
-        }
-        acc.words += 4 * m.W;
-#pragma unroll
-        for (int b = 0; b < 4; b++) vb |= ((int)n[b] >= l ? 1u : 0u) << b;
-        vb &= ((va & 1u) ? 3u : 0u) | ((va & 2u) ? 12u : 0u);
-    }
-    uint32_t bal = __ballot_sync(FULL, vb != 0);
-    while (bal) {
-        const int s = __ffs(bal) - 1;
-        bal &= bal - 1;
-        const uint32_t js = i + 1 + jc * 32 + s;
-        const uint32_t vbs = __shfl_sync(FULL, vb, s);
-        uint32_t B[4][WN];
-#pragma unroll
-        for (int w = 0; w < WN; w++) {
-            uint32_t p = w < (int)m.W ? m.P(w, js) : 0u;
-            uint32_t d = w < (int)m.W ? m.D(w, js) : 0u;
-            B[0][w] = A0[w] & p & ~d;
-            B[1][w] = A0[w] & p & d;
-            B[2][w] = A1[w] & p & ~d;
-            B[3][w] = A1[w] & p & d;
-        }
-        uint32_t tested = 0, closes = 0, viable = 0;
-        for (uint32_t mb = js + 1; mb < m.nc; mb += 32) {
-            const uint32_t c = mb + lane;
-            const bool cv = c < m.nc;
-            uint32_t S[WN], T[WN];
-#pragma unroll
-            for (int w = 0; w < WN; w++) {
-                const bool in = cv && w < (int)m.W;
-                const uint32_t p = in ? m.P(w, c) : 0u, d = in ? m.D(w, c) : 0u;
-                S[w] = p & ~d;
-                T[w] = p & d;
-            }
-            tested += cv;
-#pragma unroll
-            for (int b = 0; b < 4; b++) {
-                if (!((vbs >> b) & 1u)) continue;
-                closes += cv;
-                viable += close_st<WN>(B[b], S, T, l, acc, err);
-            }
-        }
-        acc.tested += tested;
-        acc.leaves += viable;
-        acc.words += (unsigned long long)(closes + viable) * m.W;
-    }
-}
-
-// ---- type parts for wide anchors (more words than the register paths
-// hold). The words stream through registers: the first partner's parts are
-// recomputed per word from its masks (warp-uniform loads), the lanes' own
-// candidates' S = P & ~D and T = P & D likewise, and all parts are counted in
-// one pass. For three partners the warp-uniform parts of the chosen pair live
-// in a per-warp slot (shared memory up to SLOT_W words, else the warp's
-// global scratch).
-
-constexpr int SLOT_W = 32;  // words per part in the shared per-warp slot
-__shared__ uint32_t s_slot[PB_WARPS][4 * SLOT_W];
-
-// Adds binom(x0, l) + binom(x1, l) when x0 + x1 >= l; returns that test.
-__device__ __forceinline__ bool close_x(uint32_t x0, uint32_t x1, int l, U128 &sum,
-                                        unsigned *err) {
-    const uint32_t n = x0 + x1;
-    const bool ok = (int)n >= l;
-    if (ok) {
-        if (n <= (uint32_t)BINOM_TBL) {
-            sum.add(s_bt[x0] + s_bt[x1]);
-        } else {
-            binom_add(sum, x0, l, err);
-            binom_add(sum, x1, l, err);
-        }
-    }
-    return ok;
-}
-
-// Viability of candidate i's parts (warp-cooperative): bit 0 same-sign part,
-// bit 1 different-sign part, set when the part holds at least l positions.
-template <class MK>
-__device__ __forceinline__ uint32_t stream_parts_of(const MK &m, uint32_t i, int l) {
-    const int lane = threadIdx.x & 31;
-    uint32_t n0 = 0, n1 = 0;
-    for (uint32_t w = lane; w < m.W; w += 32) {
-        const uint32_t p = m.P(w, i), d = m.D(w, i);
-        n0 += __popc(p & ~d);
-        n1 += __popc(p & d);
-    }
-    n0 = __reduce_add_sync(FULL, n0);
-    n1 = __reduce_add_sync(FULL, n1);
-    return ((int)n0 >= l ? 1u : 0u) | ((int)n1 >= l ? 2u : 0u);
-}
-
-template <class MK>
-__device__ void wide_r1(const MK &m, uint32_t jc, int l, Acc &acc, unsigned *err) {
-    const uint32_t c = jc * 32 + (threadIdx.x & 31);
-    if (c >= m.nc) return;
-    uint32_t x0 = 0, x1 = 0;
-    for (uint32_t w = 0; w < m.W; w++) {
-        const uint32_t p = m.P(w, c), d = m.D(w, c);
-        x0 += __popc(p & ~d);
-        x1 += __popc(p & d);
-    }
-    const bool ok = close_x(x0, x1, l, acc.sum, err);
-    acc.tested++;
-    acc.leaves += ok;
-    acc.words += (ok ? 2ull : 1ull) * m.W;
-}
-
-// Two partners (i, j): the four type counts of every pair in one pass.
-template <class MK>
-__device__ void wide_r2(const MK &m, uint32_t i, uint32_t jc, int l, Acc &acc, unsigned *err) {
-    const uint32_t va = stream_parts_of(m, i, l);
-    if (!va) return;
-    const uint32_t j = i + 1 + jc * 32 + (threadIdx.x & 31);
-    if (j >= m.nc) return;
-    uint32_t x00 = 0, x01 = 0, x10 = 0, x11 = 0;
-#pragma unroll 2
-    for (uint32_t w = 0; w < m.W; w++) {
-        const uint32_t pi = m.P(w, i), di = m.D(w, i);
-        const uint32_t pj = m.P(w, j), dj = m.D(w, j);
-        const uint32_t a0 = pi & ~di, a1 = pi & di, sj = pj & ~dj, tj = pj & dj;
-        x00 += __popc(a0 & sj);
-        x01 += __popc(a0 & tj);
-        x10 += __popc(a1 & sj);
-        x11 += __popc(a1 & tj);
-    }
-    uint32_t closes = 0, viable = 0;
-    if (va & 1u) {
-        closes++;
-        viable += close_x(x00, x01, l, acc.sum, err);
-    }
-    if (va & 2u) {
-        closes++;
-        viable += close_x(x10, x11, l, acc.sum, err);
-    }
-    acc.tested++;
-    acc.leaves += viable;
-    acc.words += (unsigned long long)(closes + viable) * m.W;
-}
-
-// Third partners c > js of a pair whose NB viable parts sit in `slot`
-// (NB parts of W words, part k at slot[k * stride ...]).
-template <int NB, bool SHARED, class MK>
-__device__ __forceinline__ void stream_third(const MK &m, const uint32_t *slot, uint32_t stride,
-                                             uint32_t js, int l, Acc &acc, unsigned *err) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t tested = 0, viable = 0;
-    for (uint32_t mb = js + 1; mb < m.nc; mb += 32) {
-        const uint32_t c = mb + lane;
-        if (c >= m.nc) break;
-        uint32_t x0[NB], x1[NB];
-#pragma unroll
-        for (int k = 0; k < NB; k++) x0[k] = x1[k] = 0;
-        for (uint32_t w = 0; w < m.W; w++) {
-            const uint32_t p = m.P(w, c), d = m.D(w, c);
-            const uint32_t sc = p & ~d, tc = p & d;
-#pragma unroll
-            for (int k = 0; k < NB; k++) {
-                const uint32_t bw = SHARED ? s_slot[warp][k * stride + w] : slot[k * stride + w];
-                x0[k] += __popc(bw & sc);
-                x1[k] += __popc(bw & tc);
-            }
-        }
-        tested++;
-#pragma unroll
-        for (int k = 0; k < NB; k++) viable += close_x(x0[k], x1[k], l, acc.sum, err);
-    }
-    acc.tested += tested;
-    acc.leaves += viable;
-    acc.words += (unsigned long long)(NB * tested + viable) * m.W;
-}
-
-// Three partners (i, j, c) for wide anchors. SHARED: the pair's parts fit the
-// shared per-warp slot (W <= SLOT_W); otherwise they go to the warp scratch.
-template <bool SHARED, class MK>
-__device__ void wide_r3(const MK &m, uint32_t *scratch, uint32_t wmax, uint32_t i, uint32_t jc,
-                        int l, Acc &acc, unsigned *err) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t va = stream_parts_of(m, i, l);
-    if (!va) return;
-    const uint32_t j = i + 1 + jc * 32 + lane;
-    const bool valid = j + 1 < m.nc;  // room for a third partner
-    uint32_t vb = 0;
-    if (valid) {
-        uint32_t n[4] = {0, 0, 0, 0};
-        for (uint32_t w = 0; w < m.W; w++) {
-            const uint32_t pi = m.P(w, i), di = m.D(w, i);
-            const uint32_t pj = m.P(w, j), dj = m.D(w, j);
-            const uint32_t a0 = pi & ~di, a1 = pi & di, sj = pj & ~dj, tj = pj & dj;
-            n[0] += __popc(a0 & sj);
-            n[1] += __popc(a0 & tj);
-            n[2] += __popc(a1 & sj);
-            n[3] += __popc(a1 & tj);
-        }
-        acc.tested++;
-        acc.words += 4ull * m.W;
-#pragma unroll
-        for (int b = 0; b < 4; b++) vb |= ((int)n[b] >= l ? 1u : 0u) << b;
-        vb &= ((va & 1u) ? 3u : 0u) | ((va & 2u) ? 12u : 0u);
-    }
-    uint32_t *slot = SHARED ? s_slot[warp] : scratch;
-    const uint32_t stride = SHARED ? (uint32_t)SLOT_W : wmax;
-    uint32_t bal = __ballot_sync(FULL, vb != 0);
-    while (bal) {
-        const int sl = __ffs(bal) - 1;
-        bal &= bal - 1;
-        const uint32_t js = i + 1 + jc * 32 + sl;
-        const uint32_t vbs = __shfl_sync(FULL, vb, sl);
-        const int nb = __popc(vbs);
-        // the viable parts of (i, js), compacted into slots 0 .. nb-1
-        __syncwarp();
-        for (uint32_t w = lane; w < m.W; w += 32) {
-            const uint32_t pi = m.P(w, i), di = m.D(w, i);
-            const uint32_t pj = m.P(w, js), dj = m.D(w, js);
-            const uint32_t a0 = pi & ~di, a1 = pi & di, sj = pj & ~dj, tj = pj & dj;
-            const uint32_t part[4] = {a0 & sj, a0 & tj, a1 & sj, a1 & tj};
-            int k = 0;
-#pragma unroll
-            for (int b = 0; b < 4; b++)
-                if ((vbs >> b) & 1u) slot[(k++) * stride + w] = part[b];
-        }
-        __syncwarp();
-        switch (nb) {
-            case 1: stream_third<1, SHARED>(m, slot, stride, js, l, acc, err); break;
-            case 2: stream_third<2, SHARED>(m, slot, stride, js, l, acc, err); break;
-            case 3: stream_third<3, SHARED>(m, slot, stride, js, l, acc, err); break;
-            default: stream_third<4, SHARED>(m, slot, stride, js, l, acc, err); break;
-        }
-        __syncwarp();
-    }
-}
-
-// ---- position side. For an anchor with few useful positions and many
-// candidates the same sum is taken over position subsets instead of
-// candidate subsets: expanding each binom(x, l) as the number of l-subsets Q
-// of a type class gives
-//   sum over R-subsets A, types k of binom(x[k], l)
-//     = sum over l-subsets Q of positions of binom(N_Q, R),
-// where N_Q counts the candidates w with Q inside the same-sign part
-// (P_w & ~D_w) or inside the different-sign part (P_w & D_w) of L[w] (the two
-// parts are disjoint, so w counts at most once). CM0[q] / CM1[q] are the
-// candidates whose same-sign / different-sign part holds position q (rows of
-// wc candidate words at an odd stride wcp, so lanes reading different rows hit
-// different banks). A warp walks Q depth first; at every node its lanes scan
-// 32 children q at once, each lane intersecting the node's prefix (held one
-// word per lane and broadcast by shuffles) with row q.
-
-template <int R>
-__device__ __forceinline__ void binom_add_r(U128 &acc, unsigned long long x, unsigned *err) {
-    if (x < (unsigned long long)R) return;
-    if constexpr (R == 1) {
-        acc.add(x);
-    } else {
-        if (x > c_binom64_max[R]) {
-            if (acc.add(binom_slow(x, R, err))) atomicOr(err, CERR_OVERFLOW);
-            return;
-        }
-        acc.add(binom_u64<R>(x));
-    }
-}
-
-// binom(x, R) for x <= BINOM_TBL, R = the anchor's tuple partners (shared).
-__shared__ unsigned long long s_btR[BINOM_TBL + 1];
-
-// A position-side node's prefix masks, word w of each at lane w % 32, slot
-// w / 32 (passed by value so that it stays in registers across calls).
-template <int WPL>
-struct Pfx {
-    uint32_t m0[WPL], m1[WPL];
-};
-
-// Partial result of a subtree of the position-side walk.
-struct PosOut {
-    U128 sum;
-    uint32_t tested = 0, leaves = 0;
-};
-
-// Children q in [qs, qe] of a node at depth LEV - 1 with prefix M; lanes over
-// q. At depth l a child is a leaf and adds binom(N_Q, R); otherwise children
-// with N >= R are expanded one at a time.
-template <int R, int WPL, int LEV>
-__device__ __noinline__ PosOut pos_scan(uint32_t dp, uint32_t wc, uint32_t wcp, Pfx<WPL> M,
-                                        uint32_t qs, uint32_t qe, int l, unsigned *err) {
-    const int lane = threadIdx.x & 31;
-    PosOut out;
-    for (uint32_t qb = qs; qb <= qe; qb += 32) {
-        const uint32_t q = qb + lane;
-        const bool valid = q <= qe;
-        const uint32_t o0 = (valid ? q : qs) * wcp, o1 = (dp + (valid ? q : qs)) * wcp;
-        uint32_t n = 0;
-#pragma unroll
-        for (int k = 0; k < WPL; k++) {
-            if (32u * k >= wc) break;  // WPL = 4 also serves 65..96 words
-            const uint32_t wend = wc - 32u * k < 32u ? wc - 32u * k : 32u;
-            for (uint32_t sl = 0; sl < wend; sl++) {
-                const uint32_t m0 = __shfl_sync(FULL, M.m0[k], sl), m1 = __shfl_sync(FULL, M.m1[k], sl);
-                const uint32_t w = 32u * k + sl;
-                n += __popc(m0 & sm_dyn[o0 + w]) + __popc(m1 & sm_dyn[o1 + w]);
-            }
-        }
-        out.tested += valid;
-        if (LEV == l) {
-            if (valid && n >= (uint32_t)R) {
-                out.leaves++;
-                if (n <= (uint32_t)BINOM_TBL) out.sum.add(s_btR[n]);
-                else binom_add_r<R>(out.sum, n, err);
-            }
-        } else if constexpr (LEV < 8) {
-            const uint32_t qe2 = dp - 1 - (uint32_t)(l - LEV - 1);  // room for the rest of Q
-            uint32_t bal = __ballot_sync(FULL, valid && n >= (uint32_t)R);
-            while (bal) {
-                const int sl = __ffs(bal) - 1;
-                bal &= bal - 1;
-                const uint32_t qc = qb + sl;
-                if (qc + 1 > qe2) continue;
-                Pfx<WPL> X;
-#pragma unroll
-                for (int k = 0; k < WPL; k++) {
-                    const uint32_t w = lane + 32u * k;
-                    X.m0[k] = w < wc ? (M.m0[k] & sm_dyn[qc * wcp + w]) : 0u;
-                    X.m1[k] = w < wc ? (M.m1[k] & sm_dyn[(dp + qc) * wcp + w]) : 0u;
-                }
-                const PosOut c = pos_scan<R, WPL, LEV + 1>(dp, wc, wcp, X, qc + 1, qe2, l, err);
-                if (out.sum.add(c.sum)) atomicOr(err, CERR_OVERFLOW);
-                out.tested += c.tested;
-                out.leaves += c.leaves;
-            }
-        }
-    }
-    return out;
-}
-
-// A position-side unit: first position q1 and a chunk of 32 second positions.
-template <int R, int WPL>
-__device__ void pos_unit_scan(uint32_t dp, uint32_t wc, uint32_t wcp, uint32_t q1, uint32_t chunk,
-                              int l, Acc &acc, unsigned *err) {
-    const int lane = threadIdx.x & 31;
-    Pfx<WPL> M;
-    uint32_t n = 0;
-#pragma unroll
-    for (int k = 0; k < WPL; k++) {
-        const uint32_t w = lane + 32u * k;
-        M.m0[k] = w < wc ? sm_dyn[q1 * wcp + w] : 0u;
-        M.m1[k] = w < wc ? sm_dyn[(dp + q1) * wcp + w] : 0u;
-        n += __popc(M.m0[k]) + __popc(M.m1[k]);
-    }
-    n = __reduce_add_sync(FULL, n);
-    if (n < (uint32_t)R) return;  // no Q through q1 has R candidates
-    const uint32_t qe2 = dp - 1 - (uint32_t)(l - 2);
-    const uint32_t qs = q1 + 1 + 32u * chunk;
-    const uint32_t qe = qs + 31 < qe2 ? qs + 31 : qe2;
-    if (qs > qe) return;
-    const PosOut o = pos_scan<R, WPL, 2>(dp, wc, wcp, M, qs, qe, l, err);
-    if (acc.sum.add(o.sum)) atomicOr(err, CERR_OVERFLOW);
-    acc.tested += o.tested;
-    acc.leaves += o.leaves;
-    acc.words += 2ull * wc * o.tested;
-}
-
-// Second-position chunks of first position q1 (l-subsets need q2 <= dp + 1 - l).
-__device__ __forceinline__ uint32_t pos_chunks(uint32_t dp, uint32_t q1, int l) {
-    return (dp + 1 - (uint32_t)l - q1 + 31) / 32;
-}
-
-// ---- two partners with the masks in global memory (anchors too large to
-// stage): blocks of BLK_I first partners, whose S / T words a warp keeps in
-// its shared region, against 32 second partners (one per lane) whose words
-// are loaded once per block instead of once per first partner.
-
-constexpr int BLK_I = 8;
-constexpr uint32_t BLK_MAX_W = PB_SMEM_WORDS / PB_WARPS / (2 * BLK_I);  // words per mask
-
-// Tally of one block unit.
-struct BlkOut {
-    U128 sum;
-    uint32_t tested = 0, closes = 0, viable = 0;
-};
-
-__device__ __noinline__ BlkOut block_r2(MasksG m, uint32_t *wsm, uint32_t ib, uint32_t nrows,
-                                        uint32_t jc, int l, unsigned *err) {
-    BlkOut out;
-    const int lane = threadIdx.x & 31;
-    const uint32_t W = m.W;
-    // stage S = P & ~D, T = P & D of rows ib .. ib + nrows - 1; viability bits
-    __syncwarp();
-    for (uint32_t t = lane; t < nrows * W; t += 32) {
-        const uint32_t k = t / W, w = t - k * W;
-        const uint32_t p = m.P(w, ib + k), d = m.D(w, ib + k);
-        wsm[(2 * k) * W + w] = p & ~d;
-        wsm[(2 * k + 1) * W + w] = p & d;
-    }
-    __syncwarp();
-    uint32_t va = 0;  // bit 2k: row k's same-sign part viable, bit 2k+1: different-sign
-    for (uint32_t k = 0; k < nrows; k++) {
-        uint32_t n0 = 0, n1 = 0;
-        for (uint32_t w = lane; w < W; w += 32) {
-            n0 += __popc(wsm[(2 * k) * W + w]);
-            n1 += __popc(wsm[(2 * k + 1) * W + w]);
-        }
-        n0 = __reduce_add_sync(FULL, n0);
-        n1 = __reduce_add_sync(FULL, n1);
-        va |= ((int)n0 >= l ? 1u : 0u) << (2 * k);
-        va |= ((int)n1 >= l ? 1u : 0u) << (2 * k + 1);
-    }
-    if (!va) return out;
-    const uint32_t j = ib + 1 + jc * 32 + lane;
-    if (j >= m.nc) return out;
-    uint32_t x[BLK_I][4];
-#pragma unroll
-    for (int k = 0; k < BLK_I; k++) x[k][0] = x[k][1] = x[k][2] = x[k][3] = 0;
-    for (uint32_t w = 0; w < W; w++) {
-        const uint32_t p = m.P(w, j), d = m.D(w, j);
-        const uint32_t sj = p & ~d, tj = p & d;
-#pragma unroll
-        for (int k = 0; k < BLK_I; k++) {
-            if ((uint32_t)k >= nrows) break;
-            const uint32_t a0 = wsm[(2 * k) * W + w], a1 = wsm[(2 * k + 1) * W + w];
-            x[k][0] += __popc(a0 & sj);
-            x[k][1] += __popc(a0 & tj);
-            x[k][2] += __popc(a1 & sj);
-            x[k][3] += __popc(a1 & tj);
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < BLK_I; k++) {
-        if ((uint32_t)k >= nrows || j <= ib + k) break;  // pairs i < j only
-        out.tested++;
-        if ((va >> (2 * k)) & 1u) {
-            out.closes++;
-            out.viable += close_x(x[k][0], x[k][1], l, out.sum, err);
-        }
-        if ((va >> (2 * k + 1)) & 1u) {
-            out.closes++;
-            out.viable += close_x(x[k][2], x[k][3], l, out.sum, err);
-        }
-    }
-    return out;
-}
-
-// Units of a two-partner item with global masks: blocks of BLK_I rows and
-// chunks of 32 second partners after the block's first row.
-__device__ __forceinline__ void block_units(const MasksG &m, const Item &it, int l, Acc &acc,
-                                            unsigned *err, uint32_t *s_unit, uint32_t *s_total,
-                                            uint32_t *s_rowpre) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t nc = m.nc;
-    uint32_t *wsm = sm_dyn + (size_t)warp * (2 * BLK_I) * m.W;
-    const bool split = it.u1 != 0;
-    const uint32_t nblk = split ? 1u : (it.i1 - it.i0 + BLK_I - 1) / BLK_I;
-    if (tid == 0) {
-        *s_unit = 0;
-        if (split) {
-            *s_total = it.u1 - it.u0;
-        } else {
-            uint32_t acc_u = 0;
-            for (uint32_t b = 0; b < nblk; b++) {
-                s_rowpre[b] = acc_u;
-                acc_u += (nc - 1 - (it.i0 + b * BLK_I) + 31) / 32;
-            }
-            s_rowpre[nblk] = acc_u;
-            *s_total = acc_u;
-        }
-    }
-    __syncthreads();
-    const uint32_t total = *s_total;
-    for (;;) {
-        uint32_t u = 0;
-        if (lane == 0) u = atomicAdd(s_unit, 1u);
-        u = __shfl_sync(FULL, u, 0);
-        if (u >= total) break;
-        BlkOut o;
-        if (split) {
-            o = block_r2(m, wsm, it.i0, 1, it.u0 + u, l, err);
-        } else {
-            uint32_t lo = 0, hi = nblk;  // largest b with rowpre[b] <= u
-            while (hi - lo > 1) {
-                uint32_t mid = (lo + hi) >> 1;
-                if (s_rowpre[mid] <= u) lo = mid; else hi = mid;
-            }
-            const uint32_t ib = it.i0 + lo * BLK_I;
-            const uint32_t nrows = it.i1 - ib < (uint32_t)BLK_I ? it.i1 - ib : (uint32_t)BLK_I;
-            o = block_r2(m, wsm, ib, nrows, u - s_rowpre[lo], l, err);
-        }
-        if (acc.sum.add(o.sum)) atomicOr(err, CERR_OVERFLOW);
-        acc.tested += o.tested;
-        acc.leaves += o.viable;
-        acc.words += (unsigned long long)(o.closes + o.viable) * m.W;
-    }
-}
-
-// Candidate-side work units of one item (rows i of first partners, chunks of
-// 32 second partners), taken by the CTA's warps from a shared counter.
-template <int R, class MK>
-__device__ __forceinline__ void cand_units(const MK &m, const Item &it, uint32_t *scratch,
-                                           uint32_t wmax, int l, Acc &acc, unsigned *err,
-                                           uint32_t *s_unit, uint32_t *s_total,
-                                           uint32_t *s_rowpre) {
-    const int tid = threadIdx.x, lane = tid & 31;
-    const uint32_t nc = m.nc;
-    const uint32_t W = m.W;
-    // unit layout
-    const bool split = it.u1 != 0;
-    if (tid == 0) {
-        (*s_unit) = 0;
-        if (split) {
-            (*s_total) = it.u1 - it.u0;
-        } else {
-            uint32_t acc = 0;
-            for (uint32_t i = it.i0; i < it.i1; i++) {
-                s_rowpre[i - it.i0] = acc;
-                acc += (nc - 1 - i + 31) / 32;
-            }
-            s_rowpre[it.i1 - it.i0] = acc;
-            (*s_total) = acc;
-        }
-    }
-    __syncthreads();
-    const uint32_t total = (*s_total);
-    for (;;) {
-        uint32_t u = 0;
-        if (lane == 0) u = atomicAdd(s_unit, 1u);
-        u = __shfl_sync(FULL, u, 0);
-        if (u >= total) break;
-        uint32_t i, jc;
-        if (split) {
-            i = it.i0;
-            jc = it.u0 + u;
-        } else {
-            uint32_t lo = 0, hi = it.i1 - it.i0;  // largest k with rowpre[k] <= u
-            while (hi - lo > 1) {
-                uint32_t mid = (lo + hi) >> 1;
-                if (s_rowpre[mid] <= u) lo = mid; else hi = mid;
-            }
-            i = it.i0 + lo;
-            jc = u - s_rowpre[lo];
-        }
-        if constexpr (R == 1) {
-            if (W <= 1) parts_r1<1>(m, jc, l, acc, err);
-            else if (W <= 2) parts_r1<2>(m, jc, l, acc, err);
-            else if (W <= 4) parts_r1<4>(m, jc, l, acc, err);
-            else if (W <= 8) parts_r1<8>(m, jc, l, acc, err);
-            else wide_r1(m, jc, l, acc, err);
-        } else if constexpr (R == 2) {
-            if (W <= 1) parts_r2<1>(m, i, jc, l, acc, err);
-            else if (W <= 2) parts_r2<2>(m, i, jc, l, acc, err);
-            else if (W <= 4) parts_r2<4>(m, i, jc, l, acc, err);
-            else if (W <= 8) parts_r2<8>(m, i, jc, l, acc, err);
-            else wide_r2(m, i, jc, l, acc, err);
-        } else if constexpr (R == 3) {
-            if (W <= 1) parts_r3<1>(m, i, jc, l, acc, err);
-            else if (W <= 2) parts_r3<2>(m, i, jc, l, acc, err);
-            else if (W <= 4) parts_r3<4>(m, i, jc, l, acc, err);
-            else if (W <= (uint32_t)SLOT_W) wide_r3<true>(m, scratch, wmax, i, jc, l, acc, err);
-            else wide_r3<false>(m, scratch, wmax, i, jc, l, acc, err);
-        } else {
-            if (W <= 1) unit_narrow<R, 1>(m, i, jc, l, acc, err);
-            else if (W <= 2) unit_narrow<R, 2>(m, i, jc, l, acc, err);
-            else if (W <= 4) unit_narrow<R, 4>(m, i, jc, l, acc, err);
-            else if (W <= 8) unit_narrow<R, 8>(m, i, jc, l, acc, err);
-            else unit_wide<R>(m, scratch, wmax, i, jc, l, acc, err);
-        }
-    }
-}
-
-template <int R>
-__global__ void __launch_bounds__(PB_THREADS, 2) k_tuples(TupleArgs a) {
-    __shared__ int s_item;
-    __shared__ uint32_t s_unit, s_total;
-    __shared__ uint32_t s_rowpre[ROWS_MAX + 1];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    unsigned *err = &a.cnt->err;
-    for (int x = tid; x <= BINOM_TBL; x += PB_THREADS) {
-        unsigned long long v = 0;
-        if (x >= a.l) {
-            v = 1;
-            for (int i = 1; i <= a.l; i++) v = v * (unsigned long long)(x - a.l + i) / (unsigned long long)i;
-        }
-        s_bt[x] = v;
-        unsigned long long vr = 0;
-        if (x >= R) {
-            vr = 1;
-            for (int i = 1; i <= R; i++) vr = vr * (unsigned long long)(x - R + i) / (unsigned long long)i;
-        }
-        s_btR[x] = vr;
-    }
-    __syncthreads();
-    uint32_t *scratch =
-        a.wide_scratch ? a.wide_scratch + ((size_t)blockIdx.x * PB_WARPS + warp) * SCRATCH_SLOTS * a.wmax
-                       : nullptr;
-    for (;;) {
-        if (tid == 0) s_item = (int)atomicAdd(&a.cnt->head_b, 1u);
-        __syncthreads();
-        const int item = s_item;
-        if (item >= (int)a.cnt->n_items) break;
-        const Item it = a.items[a.iorder[item]];
-        const uint32_t r = it.anchor;
-        const uint32_t nc = a.ncand[r];
-        const uint32_t W = (a.dprime[r] + 31) / 32;
-        const uint32_t rsv = a.rsv_c[r];
-        const uint32_t *region = a.pool + a.pool_off[r];
-        Acc acc;
-        if (it.u1 == POS_ITEM) {
-            // position side: CM0 / CM1 (2 * dp rows of wc words, stride wcp) in shared memory
-            const uint32_t dp = a.dprime[r];
-            const uint32_t wc = (nc + 31) / 32, wcp = wc | 1u;
-            for (uint32_t t = tid; t < 2 * dp * wcp; t += PB_THREADS) sm_dyn[t] = 0;
-            __syncthreads();
-            for (uint32_t c = tid; c < nc; c += PB_THREADS) {
-                const uint32_t cb = 1u << (c & 31), cw = c >> 5;
-                for (uint32_t w = 0; w < W; w++) {
-                    uint32_t pw = region[(size_t)w * rsv + c];
-                    const uint32_t dw = region[(size_t)(W + w) * rsv + c];
-                    while (pw) {
-                        const int b = __ffs(pw) - 1;
-                        pw &= pw - 1;
-                        const uint32_t q = 32 * w + b;
-                        const uint32_t part = (dw >> b) & 1u;
-                        atomicOr(&sm_dyn[(part * dp + q) * wcp + cw], cb);
-                    }
-                }
-            }
-            // units: first position q1 and a chunk of 32 second positions
-            if (tid == 0) {
-                uint32_t acc_u = 0;
-                for (uint32_t q = it.i0; q < it.i1; q++) {
-                    s_rowpre[q - it.i0] = acc_u;
-                    acc_u += pos_chunks(dp, q, a.l);
-                }
-                s_rowpre[it.i1 - it.i0] = acc_u;
-                s_total = acc_u;
-                s_unit = 0;
-            }
-            __syncthreads();
-            const uint32_t total = s_total;
-            for (;;) {
-                uint32_t u = 0;
-                if (lane == 0) u = atomicAdd(&s_unit, 1u);
-                u = __shfl_sync(FULL, u, 0);
-                if (u >= total) break;
-                uint32_t lo = 0, hi = it.i1 - it.i0;
-                while (hi - lo > 1) {
-                    uint32_t mid = (lo + hi) >> 1;
-                    if (s_rowpre[mid] <= u) lo = mid; else hi = mid;
-                }
-                const uint32_t q1 = it.i0 + lo;
-                const uint32_t chunk = u - s_rowpre[lo];
-                if (wc <= 32) pos_unit_scan<R, 1>(dp, wc, wcp, q1, chunk, a.l, acc, err);
-                else if (wc <= 64) pos_unit_scan<R, 2>(dp, wc, wcp, q1, chunk, a.l, acc, err);
-                else pos_unit_scan<R, 4>(dp, wc, wcp, q1, chunk, a.l, acc, err);
-            }
-        } else if (2ull * W * nc <= (unsigned long long)PB_SMEM_WORDS) {
-            // candidate side, masks staged in shared memory
-            for (uint32_t t = tid; t < 2 * W * nc; t += PB_THREADS) {
-                uint32_t wd = t / nc, c = t % nc;
-                sm_dyn[t] = region[(size_t)wd * rsv + c];
-            }
-            MasksS ms;
-            ms.W = W;
-            ms.nc = nc;
-            ms.stride = nc;
-            cand_units<R>(ms, it, scratch, a.wmax, a.l, acc, err, &s_unit, &s_total, s_rowpre);
-        } else {
-            // candidate side, masks read from the pool
-            MasksG mg;
-            mg.base = region;
-            mg.stride = rsv;
-            mg.W = W;
-            mg.nc = nc;
-            bool blocked = false;
-            if constexpr (R == 2) {
-                if (W > 8 && W <= BLK_MAX_W) {
-                    block_units(mg, it, a.l, acc, err, &s_unit, &s_total, s_rowpre);
-                    blocked = true;
-                }
-            }
-            if (!blocked)
-                cand_units<R>(mg, it, scratch, a.wmax, a.l, acc, err, &s_unit, &s_total, s_rowpre);
-        }
-        U128 ws = warp_sum_u128(acc.sum, err);
-        if (lane == 0 && (ws.lo | ws.hi)) {
-            // a batch's union total is not a count (its graphs' totals are)
-            atomic_add_u128(a.cnt->total, ws.lo, ws.hi, a.per_graph ? nullptr : err);
-            if (a.per_anchor) atomic_add_u128(a.per_anchor + 2 * (size_t)r, ws.lo, ws.hi, err);
-            if (a.per_graph) {
-                int lo = 0, hi = a.n_graphs;  // largest g with graph_x0[g] <= r
-                while (hi - lo > 1) {
-                    int mid = (lo + hi) >> 1;
-                    if (a.graph_x0[mid] <= (int64_t)r) lo = mid; else hi = mid;
-                }
-                atomic_add_u128(a.per_graph + 2 * (size_t)lo, ws.lo, ws.hi, err);
-            }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            acc.tested += __shfl_xor_sync(FULL, acc.tested, o);
-            acc.leaves += __shfl_xor_sync(FULL, acc.leaves, o);
-            acc.words += __shfl_xor_sync(FULL, acc.words, o);
-        }
-        if (lane == 0 && acc.tested) {
-            atomicAdd(&a.cnt->tested, acc.tested);
-            atomicAdd(&a.cnt->leaves, acc.leaves);
-            atomicAdd(&a.cnt->popc_words, acc.words);
-        }
-        __syncthreads();
-    }
-}
+#include "tuples.cuh"
 
 }  // namespace
 
@@ -2535,10 +1153,10 @@ __global__ void __launch_bounds__(PB_THREADS, 2) k_tuples(TupleArgs a) {
 
 namespace {
 
-// Relative cost of one position-side prefix node (per candidate word per
-// lane) against one candidate-side tuple word; measured on GB300.
+// Relative cost of one prefix node of the column walk (per row word per lane)
+// against one mask word of the row enumeration; measured on GB300.
 constexpr unsigned long long kPosNodeCost = 3;
-// Default tuple work items per resident warp of a full launch.
+// Default tuple work items per half of a resident CTA of a full launch.
 constexpr unsigned long long kSplitPerWarp = 4;
 // Two-partner anchors with at least this many mask words and candidates take
 // the tensor-core pair step.
@@ -2568,7 +1186,7 @@ unsigned long long binom64_limit(int l) {
 template <int R>
 void set_tuple_attr() {
     SBC_CUDA(cudaFuncSetAttribute(k_tuples<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)PB_SMEM));
+                                  (int)TU_SMEM));
 }
 
 // Opt every large-shared-memory kernel in, and load the binomial limits,
@@ -2603,7 +1221,6 @@ void ensure_kernel_attrs() {
     SBC_CUDA(cudaFuncSetAttribute(k_twohop_large<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PL_SMEM));
     SBC_CUDA(cudaFuncSetAttribute(k_twohop_large<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PL_SMEM));
     tc_ensure_attrs();
-    set_tuple_attr<1>();
     set_tuple_attr<2>();
     set_tuple_attr<3>();
     set_tuple_attr<4>();
@@ -2615,7 +1232,7 @@ void ensure_kernel_attrs() {
 
 template <int R>
 void launch_tuples(int grid, cudaStream_t s, const TupleArgs &a) {
-    k_tuples<R><<<grid, PB_THREADS, PB_SMEM, s>>>(a);
+    k_tuples<R><<<grid, TU_THREADS, TU_SMEM, s>>>(a);
     SBC_LAUNCHED();
 }
 
@@ -2656,10 +1273,11 @@ struct CountRun {
     int R = 0;
     cudaStream_t s = nullptr;
     DevBuf<Counters> cnt;
-    DevBuf<uint32_t> A_bit, dprime, rsv_c, skey, sval, tk, tv, ncand, npaper, pool, ikey, ival, t1b,
-        t2b, scratch;
+    DevBuf<uint32_t> A_bit, dprime, rsv_c, skey, sval, tk, tv, ncand, npaper, nrow, pool,
+        claims, scratch, warp_list;
+    DevBuf<RowInfo> rinfo;
     DevBuf<unsigned long long> e_use, e_all, bucket, per;
-    DevBuf<int64_t> pool_off, dtot, item_off, cum_dev;
+    DevBuf<int64_t> pool_off, cum_dev;
     DevBuf<Item> items;
     DevBuf<uint32_t> tc_list;
     DevBuf<unsigned char> zbuf;     // Z arena of the tensor-core pair step
@@ -2668,7 +1286,6 @@ struct CountRun {
     TupleArgs tu;
     int ga = 0, gs = 0, gt = 0;
     int64_t n_items = 0;
-    unsigned h_items = 0;
     Counters hc;
     CountResult res;
 
@@ -2683,6 +1300,7 @@ struct CountRun {
         if (groups.empty()) return;
         zero_pool(0);
         launch_twohop((unsigned)groups[0].first, (unsigned)groups[0].second);
+        if (claims.ptr) SBC_CUDA(cudaMemsetAsync(claims.ptr, 0, claims.bytes(), s));
         if (gt > 0) launch_tuple_kernel();
         launch_tc(0);
     }
@@ -2753,11 +1371,14 @@ struct CountRun {
         return (int64_t)(fr / 4 / 4);
     }
 
-    // The 2-hop kernels build candidate masks with atomicOr into a pool that
-    // is zero on entry (the CTA kernel also clears what it stages or redoes).
+    // The warp tier of the 2-hop step builds its rows with atomicOr into words
+    // that are zero on entry; the CTA tier clears or writes every word it uses.
     void zero_pool(size_t grp) {
-        const int64_t words = cum[groups[grp].second] - cum[groups[grp].first];
-        if (words > 0) SBC_CUDA(cudaMemsetAsync(pool.ptr, 0, (size_t)words * 4, s));
+        const int64_t a = groups[grp].first, b = groups[grp].second;
+        const int64_t from = std::min(std::max<int64_t>(a, hc.n_big), b);
+        const int64_t words = cum[b] - cum[from];
+        if (words > 0)
+            SBC_CUDA(cudaMemsetAsync(pool.ptr + (cum[from] - cum[a]), 0, (size_t)words * 4, s));
     }
 
     void launch_twohop(unsigned a, unsigned b) {
@@ -2786,7 +1407,6 @@ struct CountRun {
 
     void launch_tuple_kernel() {
         switch (R) {
-            case 1: launch_tuples<1>(gt, s, tu); break;
             case 2: launch_tuples<2>(gt, s, tu); break;
             case 3: launch_tuples<3>(gt, s, tu); break;
             case 4: launch_tuples<4>(gt, s, tu); break;
@@ -2814,7 +1434,7 @@ struct CountRun {
     // Tensor-core plan of group `grp` from the n anchors k_anchor_cost listed.
     void plan_tc(size_t grp, unsigned n) {
         DevBuf<TcInput> tin(n, s);
-        k_tc_gather<<<grid_for(n, 256), 256, 0, s>>>(tc_list.ptr, n, ncand.ptr, dprime.ptr,
+        k_tc_gather<<<grid_for(n, 256), 256, 0, s>>>(tc_list.ptr, n, nrow.ptr, rinfo.ptr, dprime.ptr,
                                                     rsv_c.ptr, pool_off.ptr, tin.ptr);
         SBC_LAUNCHED();
         g_launches++;
@@ -2863,11 +1483,12 @@ struct CountRun {
         tk.alloc(nX, s);
         tv.alloc(nX, s);
         ncand.alloc(nX, s);
+        nrow.alloc(nX, s);
+        rinfo.alloc(nX, s);
         npaper.alloc(spec.paper ? nX : 0, s);
         e_use.alloc(nX, s);
         e_all.alloc(nX, s);
         pool_off.alloc(nX + 1, s);
-        dtot.alloc(1, s);
         k_plan<<<grid_for(nX * 32, B), B, 0, s>>>(o->A_off.ptr, o->A_ent.ptr, o->A_pos.ptr,
                                                   o->B_off.ptr, nX, R, l, spec.shard, spec.nshard,
                                                   spec.paper ? 1 : 0, A_bit.ptr, dprime.ptr,
@@ -2878,6 +1499,7 @@ struct CountRun {
         g_launches++;
         radix_sort_pairs(skey.ptr, sval.ptr, tk.ptr, tv.ptr, nX, 32, s);
         SBC_CUDA(cudaMemsetAsync(ncand.ptr, 0, (size_t)nX * 4, s));
+        SBC_CUDA(cudaMemsetAsync(nrow.ptr, 0, (size_t)nX * 4, s));
         if (spec.paper) SBC_CUDA(cudaMemsetAsync(npaper.ptr, 0, (size_t)nX * 4, s));
         SBC_CUDA(cudaMemcpyAsync(&hc, cnt.ptr, sizeof(Counters), cudaMemcpyDeviceToHost, s));
         SBC_CUDA(cudaStreamSynchronize(s));
@@ -2923,6 +1545,9 @@ struct CountRun {
         ta.pool = pool.ptr;
         ta.ncand = ncand.ptr;
         ta.npaper = spec.paper ? npaper.ptr : nullptr;
+        ta.nrow = nrow.ptr;
+        ta.rinfo = rinfo.ptr;
+        ta.single = R == 1;
         ta.cnt = cnt.ptr;
         ta.l = l;
         ta.check = spec.check ? 1 : 0;
@@ -2945,24 +1570,29 @@ struct CountRun {
             const void *fn = spec.paper ? (const void *)k_twohop_small<true> : (const void *)k_twohop_small<false>;
             gs = sms * blocks_per_sm(fn, PS_THREADS, PS_SMEM);
         }
-        const int gb = sms * blocks_per_sm((const void *)k_tuples<1>, PB_THREADS, PB_SMEM);
+        const int gb = sms;  // one tuple CTA per SM (its shared memory)
         const uint32_t wmax = (uint32_t)((o->max_deg_x + 31) / 32);
         per.alloc(spec.per_anchor ? 2 * nX : 0, s);
         if (per.ptr) SBC_CUDA(cudaMemsetAsync(per.ptr, 0, per.bytes(), s));
         if (spec.per_graph) SBC_CUDA(cudaMemsetAsync(spec.per_graph, 0, 16 * (size_t)spec.n_graphs, s));
-        // warp scratch of the wide paths (more words than the register paths hold)
-        const uint32_t wide_from = R == 3 ? (uint32_t)SLOT_W : R <= 2 ? 0xFFFFFFFFu : 8u;
-        scratch.alloc(wmax > wide_from ? (size_t)gb * PB_WARPS * SCRATCH_SLOTS * wmax : 0, s);
-        tu.ncand = ncand.ptr;
+        // prefix masks of the widest anchors, where they do not fit the warp's shared area
+        scratch.alloc(R > 2 && (uint64_t)(R - 1) * wmax > TU_LIST_W
+                          ? (size_t)gb * TU_WARPS * SCRATCH_SLOTS * wmax : 0, s);
+        Totals tot;
+        tot.total = cnt.ptr->total;
+        tot.per_anchor = per.ptr;
+        tot.per_graph = spec.per_graph;
+        tot.graph_x0 = spec.graph_x0;
+        tot.n_graphs = spec.n_graphs;
+        tot.err = &cnt.ptr->err;
+        ta.tot = tot;
+        tu.nrow = nrow.ptr;
         tu.dprime = dprime.ptr;
         tu.rsv_c = rsv_c.ptr;
         tu.pool_off = pool_off.ptr;
         tu.pool = pool.ptr;
         tu.cnt = cnt.ptr;
-        tu.per_anchor = per.ptr;
-        tu.per_graph = spec.per_graph;
-        tu.graph_x0 = spec.graph_x0;
-        tu.n_graphs = spec.n_graphs;
+        tu.tot = tot;
         tu.wide_scratch = scratch.ptr;
         tu.wmax = wmax;
         tu.l = l;
@@ -2970,21 +1600,21 @@ struct CountRun {
         ItemArgs ia;
         ia.ncand = ncand.ptr;
         ia.npaper = spec.paper ? npaper.ptr : nullptr;
+        ia.nrow = nrow.ptr;
         ia.dprime = dprime.ptr;
+        ia.rinfo = rinfo.ptr;
         ia.order = sval.ptr;
         ia.R = R;
         ia.l = l;
         ia.method = spec.method;
-        ia.pos_unit = spec.pos_unit;
+        ia.pos_unit = (float)spec.pos_unit;
+        ia.items_per_launch = 2.0f * (float)gb *
+            (float)(spec.split_per_warp > 0 ? (unsigned long long)spec.split_per_warp : kSplitPerWarp);
         ia.cnt = cnt.ptr;
         ia.tc_on = spec.tc_min_w >= 0 && R == 2 && !thread_arena_active();
         ia.tc_min_w = spec.tc_min_w > 0 ? (uint32_t)spec.tc_min_w : kTcMinWords;
         ia.tc_min_nc = tc_min_candidates();
-        if (ia.tc_on) {
-            tc_list.alloc(nX, s);
-            tc_ensure_attrs();
-        }
-        ia.tc_list = tc_list.ptr;
+        if (ia.tc_on) tc_ensure_attrs();
         tc_plans.clear();
         tc_plans.resize(groups.size());
         n_items = 0;
@@ -2994,9 +1624,8 @@ struct CountRun {
             k_group_offsets<<<grid_for(na, B), B, 0, s>>>(sval.ptr, cum_dev.ptr, a, b, pool_off.ptr);
             SBC_LAUNCHED();
             g_launches++;
-            SBC_CUDA(cudaMemsetAsync(&cnt.ptr->head_large, 0, 3 * sizeof(unsigned), s));
-            SBC_CUDA(cudaMemsetAsync(&cnt.ptr->cost_total, 0, sizeof(unsigned long long), s));
-            SBC_CUDA(cudaMemsetAsync(&cnt.ptr->n_tc, 0, sizeof(unsigned), s));
+            SBC_CUDA(cudaMemsetAsync(&cnt.ptr->head_large, 0, 4 * sizeof(unsigned), s));
+            SBC_CUDA(cudaMemsetAsync(&cnt.ptr->cost_total, 0, 9 * sizeof(unsigned), s));
             SBC_CUDA(cudaMemsetAsync(&cnt.ptr->tw_fin_max, 0, 2 * sizeof(unsigned long long), s));
             cudaEvent_t t0 = timing ? new_event(ev_twohop) : nullptr;
             cudaEvent_t t1 = timing ? new_event(ev_twohop) : nullptr;
@@ -3007,72 +1636,51 @@ struct CountRun {
                 launch_twohop((unsigned)a, (unsigned)b);
             }
             if (t1) SBC_CUDA(cudaEventRecord(t1, s));
-            // tuple phase planning (needs the candidate counts)
+            // tuple phase planning (needs the row counts)
             ia.begin = a;
             ia.nX = na;
-            ia.item_cost = 0;
-            ia.item_off = nullptr;
-            ia.item_cnt = nullptr;
             ia.items = nullptr;
-            ia.ikey = ia.ival = nullptr;
+            ia.warp_list = ia.tc_list = nullptr;
             k_anchor_cost<<<grid_for(na, B), B, 0, s>>>(ia);
+            SBC_LAUNCHED();
+            g_launches++;
+            if (R == 1) continue;  // the 2-hop kernels added every sum
+            k_items<false><<<grid_for(na, B), B, 0, s>>>(ia);
             SBC_LAUNCHED();
             g_launches++;
             SBC_CUDA(cudaMemcpyAsync(&hc, cnt.ptr, sizeof(Counters), cudaMemcpyDeviceToHost, s));
             SBC_CUDA(cudaStreamSynchronize(s));
             tw_tail_ms = std::max(tw_tail_ms, group_tail_ms());
-            if (hc.n_tc > 0) plan_tc(gi, hc.n_tc);
-            const unsigned long long spw =
-                spec.split_per_warp > 0 ? (unsigned long long)spec.split_per_warp : kSplitPerWarp;
-            unsigned long long ic = hc.cost_total / ((unsigned long long)gb * PB_WARPS * spw);
-            if (ic < (1ull << 12)) ic = 1ull << 12;
-            if (ic > (1ull << 30)) ic = 1ull << 30;
-            ia.item_cost = ic;
-            item_off.alloc(na + 1, s);
-            ia.item_cnt = item_off.ptr;
-            int64_t ng = 0;
-            if (hc.cost_total > 0 || R == 1) {
-                k_items<false><<<grid_for(na, B), B, 0, s>>>(ia);
-                SBC_LAUNCHED();
-                scan_exclusive_i64(item_off.ptr, item_off.ptr, na + 1, dtot.ptr, s);
-                g_launches++;
-                SBC_CUDA(cudaMemcpyAsync(&ng, dtot.ptr, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-                SBC_CUDA(cudaStreamSynchronize(s));
-            }
-            if (ng > 0xFFFFFFF0ll) fail(SBC_E_UNSUPPORTED, "too many work items");
-            if (ng == 0) {
-                run_tc_timed(gi, timing);
-                continue;
-            }
-            items.alloc(ng, s);
-            ikey.alloc(ng, s);
-            ival.alloc(ng, s);
-            t1b.alloc(ng, s);
-            t2b.alloc(ng, s);
-            ia.item_off = item_off.ptr;
+            if (hc.n_items == 0 && hc.n_warp == 0 && hc.n_tc == 0) continue;
+            items.alloc(hc.n_items, s);
+            warp_list.alloc(hc.n_warp, s);
+            claims.alloc(hc.n_claims, s);
+            tc_list.alloc(hc.n_tc, s);
             ia.items = items.ptr;
-            ia.ikey = ikey.ptr;
-            ia.ival = ival.ptr;
+            ia.warp_list = warp_list.ptr;
+            ia.tc_list = tc_list.ptr;
             k_items<true><<<grid_for(na, B), B, 0, s>>>(ia);
             SBC_LAUNCHED();
             g_launches++;
-            radix_sort_pairs(ikey.ptr, ival.ptr, t1b.ptr, t2b.ptr, ng, 32, s);
-            h_items = (unsigned)ng;
-            SBC_CUDA(cudaMemcpyAsync(&cnt.ptr->n_items, &h_items, sizeof(unsigned), cudaMemcpyHostToDevice, s));
             tu.items = items.ptr;
-            tu.iorder = ival.ptr;
-            gt = gb;
-            if ((int64_t)gt > ng) gt = (int)ng;
-            cudaEvent_t t2 = timing ? new_event(ev_tuples) : nullptr;
-            cudaEvent_t t3 = timing ? new_event(ev_tuples) : nullptr;
-            if (t2) SBC_CUDA(cudaEventRecord(t2, s));
-            {
-                NvtxRange nr("sbc/tuples");
-                launch_tuple_kernel();
+            tu.warp_list = warp_list.ptr;
+            tu.claims = claims.ptr;
+            const int64_t work = (int64_t)hc.n_items + ((int64_t)hc.n_warp + TU_WARPS - 1) / TU_WARPS;
+            gt = (int)std::min<int64_t>(gb, work);
+            if (gt > 0) {
+                if (claims.ptr) SBC_CUDA(cudaMemsetAsync(claims.ptr, 0, claims.bytes(), s));
+                cudaEvent_t t2 = timing ? new_event(ev_tuples) : nullptr;
+                cudaEvent_t t3 = timing ? new_event(ev_tuples) : nullptr;
+                if (t2) SBC_CUDA(cudaEventRecord(t2, s));
+                {
+                    NvtxRange nr("sbc/tuples");
+                    launch_tuple_kernel();
+                }
+                if (t3) SBC_CUDA(cudaEventRecord(t3, s));
             }
-            if (t3) SBC_CUDA(cudaEventRecord(t3, s));
+            if (hc.n_tc > 0) plan_tc(gi, hc.n_tc);  // on the host, next to the tuple kernel
             run_tc_timed(gi, timing);
-            n_items += ng;
+            n_items += hc.n_items + hc.n_warp;
         }
         if (tm) tm->mark(4, s);
         collect();
@@ -3085,10 +1693,6 @@ struct CountRun {
         skey.release();
         tk.release();
         tv.release();
-        item_off.release();
-        ikey.release();
-        t1b.release();
-        t2b.release();
     }
 
     // Read the counters after an execution (synchronises the stream).

@@ -263,20 +263,23 @@ void apply_tune(CountSpec &spec, const sbc_tune_t *t);
 // (tc_pairs.cu). One anchor of a chunk:
 struct TcAnchor {
     uint32_t r;          // anchor rank
-    uint32_t nc, W, rsv; // candidates, mask words, candidate stride of its pool region
+    uint32_t nr, W, rsv; // rows, mask words, row stride of its pool region
     uint32_t RB, KB;     // Z row blocks of 128 (even), position blocks of 128
+    uint32_t longest, pad;  // most positions of a row: bounds every Gram entry
     int64_t pool_off;    // its pool region (words)
     int64_t zblk0;       // first Z block (16 KB each) in the chunk's arena
     int64_t tile0;       // first output tile in the chunk
 };
 struct TcInput {
-    uint32_t r, nc, W, rsv;
+    uint32_t r, nr, W, rsv, longest;
     int64_t pool_off;
 };
 struct TcChunk {
     std::vector<TcAnchor> host;
     DevBuf<TcAnchor> dev;
+    DevBuf<uint32_t> job;  // anchor of every job's first tile
     int64_t n_blocks = 0, n_tiles = 0;
+    int job_tiles = 1;     // tiles per job
 };
 struct TcPlan {
     std::vector<TcChunk> chunks;
@@ -287,6 +290,8 @@ struct TcArgs {
     const TcAnchor *anc = nullptr;
     int n_anc = 0;
     int64_t n_blocks = 0, n_tiles = 0;
+    uint32_t *job = nullptr;
+    int job_tiles = 1;
     const uint32_t *pool = nullptr;
     unsigned char *z = nullptr;
     int l = 0;

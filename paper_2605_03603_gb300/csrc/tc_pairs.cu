@@ -2,16 +2,15 @@
 // the loop over (p-1)-subsets A of C with p - 1 = 2, and the type count of
 // Section 4.2) for anchors whose candidate masks are wide.
 //
-// For an anchor u with candidates 0..nc-1 and useful positions 0..d'-1, let
-// S_c = P_c AND NOT D_c (common neighbours where sign(u,v) = sign(c,v)) and
-// T_c = P_c AND D_c (where they differ), as 0/1 vectors over the positions.
-// For a pair of candidates i < j the four type classes of Section 4.2 are
-// (s,s), (s,d), (d,s), (d,d), with sizes <S_i,S_j>, <S_i,T_j>, <T_i,S_j>,
-// <T_i,T_j>. Stacking the rows Z = [S_0; T_0; S_1; T_1; ...] (row 2c + 0 is
-// S_c, row 2c + 1 is T_c) gives all of them at once as G = Z Z^T, and the
-// anchor adds, over row pairs (a, b) with floor(a/2) < floor(b/2),
-// binom(G[a][b], l). This is a dense contraction over the positions, so it
-// runs on the tensor cores:
+// An anchor's rows are the parts S_c = P_c AND NOT D_c (common neighbours where
+// sign(u,v) = sign(c,v)) and T_c = P_c AND D_c (where they differ) of its
+// candidates that hold at least l positions, as 0/1 vectors over its useful
+// positions. For a pair of candidates i < j the four type classes of Section
+// 4.2 are (s,s), (s,d), (d,s), (d,d), with sizes <S_i,S_j>, <S_i,T_j>,
+// <T_i,S_j>, <T_i,T_j>; the two parts of one candidate are disjoint (product 0,
+// which adds nothing). With Z the rows stacked, the anchor therefore adds, over
+// row pairs a < b, binom(G[a][b], l) with G = Z Z^T. This is a dense
+// contraction over the positions, so it runs on the tensor cores:
 //
 // * k_zexpand writes Z as fp8 e4m3 bytes (1.0 or 0) in 16 KB blocks of 128
 //   rows x 128 positions, each block already in the shared-memory layout of
@@ -19,7 +18,7 @@
 //   chunk c ^ (r & 7)), so a block moves to shared memory with one plain
 //   bulk copy.
 // * k_tcpairs is a persistent kernel over output tiles of 128 x 256 rows of
-//   G (only tiles that hold a pair a < b in candidate order). Per CTA: one
+//   G (only tiles that hold a pair a < b). Per CTA: one
 //   producer warp issues the bulk copies into a 4-stage ring, one warp issues
 //   tcgen05.mma (kind::f8f6f4, M = 128, N = 256, K = 32 per instruction)
 //   into one of two TMEM accumulators, and eight epilogue warps read the
@@ -207,25 +206,30 @@ __device__ __noinline__ U128 tc_binom_big(unsigned long long x, int l, unsigned 
 // Expand the chunk's candidate masks into Z blocks (see the file comment).
 __global__ void __launch_bounds__(512) k_zexpand(TcArgs a) {
     const int r = threadIdx.x & 127, wi = threadIdx.x >> 7;
-    // the blocks of a CTA increase, so its anchor index only moves forward
-    int ai = -1;
-    int64_t next0 = 0;
+    // a CTA expands consecutive blocks: one search for its first anchor, then a
+    // walk over the few anchors of its range (with strided blocks every CTA
+    // walked the records of all anchors, a dependent load each)
+    const int64_t per = (a.n_blocks + gridDim.x - 1) / gridDim.x;
+    const int64_t b0 = blockIdx.x * per, b1 = b0 + per < a.n_blocks ? b0 + per : a.n_blocks;
+    if (b0 >= b1) return;
+    int ai = 0, hi = a.n_anc;  // largest ai with zblk0 <= b0
+    while (hi - ai > 1) {
+        const int mid = (ai + hi) >> 1;
+        if (a.anc[mid].zblk0 <= b0) ai = mid; else hi = mid;
+    }
+    ai--;
+    int64_t next0 = b0;
     TcAnchor A;
-    for (int64_t blk = blockIdx.x; blk < a.n_blocks; blk += gridDim.x) {
+    for (int64_t blk = b0; blk < b1; blk++) {
         while (blk >= next0) {
             A = a.anc[++ai];
             next0 = ai + 1 < a.n_anc ? a.anc[ai + 1].zblk0 : a.n_blocks;
         }
         const int64_t local = blk - A.zblk0;
         const uint32_t rb = (uint32_t)(local / A.KB), kb = (uint32_t)(local % A.KB);
-        const uint32_t row = rb * 128 + r, c = row >> 1, w = kb * 4 + wi;
+        const uint32_t row = rb * 128 + r, w = kb * 4 + wi;
         uint32_t bits = 0;
-        if (c < A.nc && w < A.W) {
-            const uint32_t *region = a.pool + A.pool_off;
-            const uint32_t P = region[(size_t)w * A.rsv + c];
-            const uint32_t D = region[(size_t)(A.W + w) * A.rsv + c];
-            bits = (row & 1) ? (P & D) : (P & ~D);
-        }
+        if (row < A.nr && w < A.W) bits = a.pool[A.pool_off + (int64_t)w * A.rsv + row];
         // 32 positions -> 32 bytes of 0x38 (e4m3 1.0) or 0: each nibble is
         // spread to the low bit of 4 bytes and scaled
         uint32_t o[8];
@@ -241,27 +245,52 @@ __global__ void __launch_bounds__(512) k_zexpand(TcArgs a) {
 
 namespace {
 
-// Walks the tiles of one CTA (t = blockIdx.x, + gridDim.x, ...): tile t of
-// the chunk, its anchor and block coordinates (I rows of 128, J columns of
-// 256; column J holds the rows I = 0 .. 2J + 1, the tiles with a pair a < b).
-// Anchor and column only move forward, so every step is a few compares
-// (the anchor record is loaded once per anchor, not searched per tile).
+// Walks the tiles of one CTA: jobs of a.job_tiles consecutive tiles, job
+// blockIdx.x, + gridDim.x, ... Tile t of the chunk, its anchor and block
+// coordinates (I rows of 128, J columns of 256; column J holds the rows
+// I = 0 .. 2J + 1, the tiles with a pair a < b). A job starts at the anchor
+// that k_tcjobs noted for it and walks forward inside the job only: with single
+// strided tiles every role of every CTA walked all anchors of the chunk
+// (medium graph, (3,3): 25 ns per tile of the whole GPU against 10 ns).
 struct TileCursor {
-    int ai = -1;
-    int64_t next0 = 0;  // first tile of the next anchor
+    int64_t t = 0, end = 0, job, next0 = 0;  // next0: first tile of the next anchor
+    int ai = 0;
     TcAnchor A;
     uint32_t I = 0, J = 0;
-    __device__ __forceinline__ void seek(const TcArgs &a, int64_t t) {
-        while (t >= next0) {
-            A = a.anc[++ai];
-            next0 = ai + 1 < a.n_anc ? a.anc[ai + 1].tile0 : a.n_tiles;
+    __device__ __forceinline__ TileCursor() : job((int64_t)blockIdx.x - gridDim.x) {}
+    // Moves to the CTA's next tile; false when there is none.
+    __device__ __forceinline__ bool next(const TcArgs &a) {
+        if (++t >= end) {
+            job += gridDim.x;
+            t = job * a.job_tiles;
+            if (t >= a.n_tiles) return false;
+            end = t + a.job_tiles < a.n_tiles ? t + a.job_tiles : a.n_tiles;
+            ai = (int)a.job[job] - 1;
+            next0 = t;
+        }
+        if (t >= next0) {
+            do {
+                ai++;
+                next0 = ai + 1 < a.n_anc ? a.anc[ai + 1].tile0 : a.n_tiles;
+            } while (t >= next0);
+            A = a.anc[ai];
             J = 0;
         }
+        // columns before J hold J (J + 1) tiles
         const uint64_t local = (uint64_t)(t - A.tile0);
         while ((uint64_t)(J + 1) * (J + 2) <= local) J++;
         I = (uint32_t)(local - (uint64_t)J * (J + 1));
+        return true;
     }
 };
+
+// Anchor of every job's first tile (thread per anchor).
+__global__ void k_tcjobs(TcArgs a) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.n_anc; i += gridDim.x * blockDim.x) {
+        const int64_t t0 = a.anc[i].tile0, t1 = i + 1 < a.n_anc ? a.anc[i + 1].tile0 : a.n_tiles;
+        for (int64_t j = (t0 + a.job_tiles - 1) / a.job_tiles; j * a.job_tiles < t1; j++) a.job[j] = (uint32_t)i;
+    }
+}
 
 }  // namespace
 
@@ -277,8 +306,8 @@ __device__ __forceinline__ unsigned long long binom_u64c(unsigned long long x) {
 }
 
 // Largest multiple of 32 (at most 2048) with 32 * binom(x, L) < 2^32: for
-// anchors of at most this many useful positions every Gram entry indexes a
-// 32-bit table and 32 of its binomials sum in 32 bits.
+// anchors whose longest row has at most this many positions every Gram entry
+// indexes a 32-bit table and 32 of its binomials sum in 32 bits.
 template <int L>
 __host__ __device__ constexpr uint32_t tc_fast_max() {
     uint32_t best = 0;
@@ -343,8 +372,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tcpairs(TcArgs a) {
             int issued[TC_STAGES] = {0, 0, 0, 0};
             uint32_t issued_par[TC_STAGES] = {0, 0, 0, 0};
             TileCursor tr;
-            for (int64_t t = blockIdx.x; t < a.n_tiles && !s_abort; t += gridDim.x) {
-                tr.seek(a, t);
+            while (!s_abort && tr.next(a)) {
                 const TcAnchor &A = tr.A;
                 const unsigned char *zA = a.z + (A.zblk0 + (int64_t)tr.I * A.KB) * TC_BLOCK;
                 const unsigned char *zB0 = a.z + (A.zblk0 + (int64_t)(2 * tr.J) * A.KB) * TC_BLOCK;
@@ -380,8 +408,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tcpairs(TcArgs a) {
             uint32_t stage = 0, round = 0, it = 0;
             const uint32_t sbase = smem_u32(smem);
             TileCursor tr;
-            for (int64_t t = blockIdx.x; t < a.n_tiles && !s_abort; t += gridDim.x, it++) {
-                tr.seek(a, t);
+            for (; !s_abort && tr.next(a); it++) {
                 const TcAnchor &A = tr.A;
                 const uint32_t buf = it & 1;
                 if (!mbar_wait(&acc_empty[buf], ((it >> 1) & 1) ^ 1, &s_abort, a.err)) break;
@@ -447,8 +474,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tcpairs(TcArgs a) {
             if (x <= a.big64) sum.add(binom_u64c<L>(x));
             else if (sum.add(tc_binom_big(x, L, a.err))) atomicOr(a.err, kErrOverflow);
         };
-        for (int64_t t = blockIdx.x; t < a.n_tiles; t += gridDim.x, it++) {
-            tr.seek(a, t);
+        for (; tr.next(a); it++) {
             const uint32_t buf = it & 1;
             if (tr.ai != sum_ai) {
                 if (sum_ai >= 0) flush();
@@ -461,13 +487,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tcpairs(TcArgs a) {
             if (!ok) break;
             tc_fence_after();
             const uint32_t row = tr.I * 128 + g * 32 + lane;  // row of G
-            const uint32_t ca = row >> 1;                       // its candidate
-            // columns of this tile (0..255) whose candidate exceeds the row's:
-            // all of them off the diagonal, from c0 on it
-            const uint32_t c0 = ca + 1 > tr.J * 128 ? (ca + 1 - tr.J * 128) * 2 : 0u;
+            // columns of this tile (0..255) after the row: all of them off the
+            // diagonal, from c0 on it
+            const uint32_t c0 = row + 1 > tr.J * 256 ? row + 1 - tr.J * 256 : 0u;
             const uint32_t cl0 = __shfl_sync(0xffffffffu, c0, 0);  // smallest in the warp
-            // entries are at most the anchor's useful positions (<= 32 W)
-            const bool fast = 32ull * tr.A.W <= FAST;
+            // entries are at most the longest row
+            const bool fast = tr.A.longest <= FAST;
             for (uint32_t cb = half * 128; cb < half * 128 + 128; cb += 32) {
                 if (cb + 32 <= cl0) continue;  // no lane keeps a column here (warp-uniform)
                 uint32_t v[32];
@@ -545,7 +570,7 @@ TcPlan tc_plan(const std::vector<TcInput> &in, int64_t budget_bytes) {
     // heaviest per-tile work first, so that the strided tile assignment of
     // the persistent kernel ends with short tiles
     std::sort(v.begin(), v.end(), [](const TcInput &x, const TcInput &y) {
-        return x.W != y.W ? x.W > y.W : x.nc > y.nc;
+        return x.W != y.W ? x.W > y.W : x.nr > y.nr;
     });
     TcChunk cur;
     int64_t blocks = 0, tiles = 0;
@@ -553,6 +578,9 @@ TcPlan tc_plan(const std::vector<TcInput> &in, int64_t budget_bytes) {
         if (cur.host.empty()) return;
         cur.n_blocks = blocks;
         cur.n_tiles = tiles;
+        // 16 tiles amortise a job's start; fewer when the chunk could not give
+        // every SM several jobs
+        cur.job_tiles = (int)std::max<int64_t>(1, std::min<int64_t>(16, tiles / (152 * 8)));
         plan.max_blocks = std::max(plan.max_blocks, blocks);
         plan.chunks.push_back(std::move(cur));
         cur = TcChunk();
@@ -561,10 +589,12 @@ TcPlan tc_plan(const std::vector<TcInput> &in, int64_t budget_bytes) {
     for (const TcInput &x : v) {
         TcAnchor A;
         A.r = x.r;
-        A.nc = x.nc;
+        A.nr = x.nr;
+        A.longest = x.longest;
+        A.pad = 0;
         A.W = x.W;
         A.rsv = x.rsv;
-        A.RB = 2 * ((x.nc + 127) / 128);
+        A.RB = 2 * ((x.nr + 255) / 256);
         A.KB = (x.W + 3) / 4;
         A.pool_off = x.pool_off;
         const int64_t nb = (int64_t)A.RB * A.KB;
@@ -588,6 +618,7 @@ void tc_upload(TcPlan &plan, cudaStream_t s) {
         c.dev.alloc(c.host.size(), s);
         SBC_CUDA(cudaMemcpyAsync(c.dev.ptr, c.host.data(), sizeof(TcAnchor) * c.host.size(),
                                  cudaMemcpyHostToDevice, s));
+        c.job.alloc((size_t)((c.n_tiles + c.job_tiles - 1) / c.job_tiles), s);
     }
 }
 
@@ -617,10 +648,14 @@ void tc_launch(const TcPlan &plan, TcArgs base, unsigned char *z, cudaStream_t s
         a.n_blocks = c.n_blocks;
         a.n_tiles = c.n_tiles;
         a.z = z;
+        a.job = c.job.ptr;
+        a.job_tiles = c.job_tiles;
+        k_tcjobs<<<grid_for(a.n_anc, 128), 128, 0, s>>>(a);
+        SBC_LAUNCHED();
         int ge = (int)std::min<int64_t>(c.n_blocks, (int64_t)sms * 8);
         k_zexpand<<<ge, 512, 0, s>>>(a);
         SBC_LAUNCHED();
-        int gt = (int)std::min<int64_t>(c.n_tiles, (int64_t)sms);
+        int gt = (int)std::min<int64_t>((c.n_tiles + c.job_tiles - 1) / c.job_tiles, (int64_t)sms);
         switch (a.l) {
             case 2: k_tcpairs<2><<<gt, TC_THREADS, TC_SMEM, s>>>(a); break;
             case 3: k_tcpairs<3><<<gt, TC_THREADS, TC_SMEM, s>>>(a); break;
@@ -631,7 +666,7 @@ void tc_launch(const TcPlan &plan, TcArgs base, unsigned char *z, cudaStream_t s
             default: k_tcpairs<8><<<gt, TC_THREADS, TC_SMEM, s>>>(a); break;
         }
         SBC_LAUNCHED();
-        g_launches += 2;
+        g_launches += 3;
     }
 }
 
