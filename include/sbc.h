@@ -212,7 +212,7 @@ typedef struct {
     uint64_t tc_kblocks;    /* K steps of 128 positions over those tiles: the step made
                                tc_kblocks x 128 x 256 x 128 multiply-adds */
     /* CTA-wide 2-hop kernel (anchors with more than the warp tier's wedges), by
-     * strategy: [0] one hash window, [1] wedges bucketed once by hash class,
+     * strategy: [0] one hash window, or counters indexed by rank, [1] wedges bucketed once by hash class,
      * [2] the 2-hop re-read once per hash class (fallback), [3] bucketed, then
      * scattered a second time at exact class offsets (a class overflowed its
      * capacity) */

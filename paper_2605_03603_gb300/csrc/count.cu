@@ -418,6 +418,8 @@ struct TwohopArgs {
     RowInfo *rinfo;
     Counters *cnt;
     Totals tot;
+    uint32_t n_ranks;               // anchors of the side
+    int direct;                     // direct counters allowed (not when a test forces the hash strategies)
     int single;                     // one partner: the counters give the sum, no rows are written
     unsigned long long *bucket;     // per-CTA bucket slots of the large-anchor kernel
     unsigned long long bucket_slot; // entries per slot
@@ -752,6 +754,278 @@ __device__ __forceinline__ void visit_block(int64_t ebase, int d, bool useful_on
     }
 }
 
+// ---- direct counters. A partner's rank follows the anchor's, and anchors with
+// many wedges have high degrees, so high ranks: their partners' ranks span a
+// short range (on the 2M-edge graph 76 % of the wedges of anchors above 3,584
+// span at most 48k ranks). Such an anchor counts its partners in a table
+// indexed by rank - no keys, no probes, one shared-memory add without a return
+// value per wedge - in windows of consecutive ranks, each a pass over the
+// 2-hop. Counters hold the same-sign and different-sign counts of a partner in
+// 8 + 8 bits (at most 255 useful positions) or 16 + 16 bits. After a window's
+// counts, a bitmap of the parts with at least l positions and its prefix counts
+// number the rows, and the counters' memory stages the mask words of the
+// window's rows, a range of positions at a time.
+// Bound by the shared-memory atomics and the L2 gathers of B_ent. The 2-hop
+// kernels of the (3,3) count took 13.7 -> 6.4 ms on the 2M-edge graph, 74 -> 32
+// ms on a 12M-edge hub graph and 15.6 -> 1.4 ms on a dense 3000 x 800 graph
+// (hash strategies -> direct counters where the rule takes them).
+constexpr uint32_t DT_WORDS = 20480;            // counter words, then staged mask words
+constexpr uint32_t DT_CELLS8 = 2 * DT_WORDS;    // ranks per window with 8 + 8 bit counters
+constexpr uint32_t DT_CELLS16 = DT_WORDS;
+constexpr uint32_t DT_BM = DT_CELLS8 / 16;      // bitmap words (two bits per rank)
+constexpr size_t DT_OFF_BM = (size_t)DT_WORDS * 4;
+constexpr size_t DT_OFF_PRE = DT_OFF_BM + (size_t)DT_BM * 4;
+constexpr size_t DT_OFF_POFF = DT_OFF_PRE + (size_t)DT_BM * 4;
+constexpr size_t DT_OFF_PPRE = DT_OFF_POFF + (size_t)PL_PCH * 4;
+constexpr size_t DT_OFF_PINFO = DT_OFF_PPRE + (size_t)(PL_PCH + 4) * 4;
+static_assert(DT_OFF_PINFO + (size_t)PL_PCH * 4 <= PL_SMEM, "direct counters' shared layout");
+
+// Direct counters or the hash strategies. Lists of at least 8 partners on
+// average (in shorter ones, of the widest hubs, few partners share all the
+// counters). Costs in SM cycles measured on the 2M-edge graph: a window about
+// 3,000 (clear, scan, barriers) and 0.7 per wedge for its two passes; the hash
+// strategies about 8 per wedge.
+__device__ __forceinline__ bool direct_takes(unsigned long long e, uint32_t dp, uint32_t range) {
+    if (dp > 65535u || e < 8ull * dp) return false;
+    const uint32_t cells = dp <= 255u ? DT_CELLS8 : DT_CELLS16;
+    const float nwin = (float)((range + cells - 1) / cells);
+    return nwin * (3000.0f + 0.7f * (float)e) < 8.0f * (float)e;
+}
+
+// Visit the anchor's 2-hop entries at the useful positions whose bit index lies
+// in [blo, bhi), with the whole CTA: positions staged PL_PCH at a time, the
+// non-empty ones compacted; the entries of a batch are split evenly over the
+// warps, every lane finds its first list by a search and walks forward from
+// it, four entries in flight. fn(entry, sign of the position | bit index).
+template <typename F>
+__device__ __forceinline__ void visit_lists(int64_t ebase, int d, uint32_t blo, uint32_t bhi,
+                                            const TwohopArgs &a, uint32_t *poff, uint32_t *ppre,
+                                            uint32_t *pinfo, unsigned long long *warp_tot,
+                                            unsigned long long *s_total, F fn) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int c0 = 0; c0 < d; c0 += PL_PCH) {
+        uint32_t len = 0, info = 0, st = 0;
+        if (c0 + tid < d) {
+            const int64_t e = ebase + c0 + tid;
+            const uint32_t bit = a.A_bit[e];
+            if (bit >= blo && bit < bhi) {  // (EMPTY is above every bhi)
+                const uint32_t av = a.A_ent[e];
+                const uint32_t y = av & VMASK;
+                st = (uint32_t)(a.B_off[y] + (int64_t)a.A_pos[e] + 1);
+                len = (uint32_t)a.B_off[y + 1] - st;
+                info = (av & 0x80000000u) | bit;
+            }
+        }
+        const unsigned long long packed = len ? ((1ull << 32) | len) : 0ull;
+        const unsigned long long ex = block_excl_scan_u64(packed, warp_tot, s_total);
+        if (len) {
+            const uint32_t slot = (uint32_t)(ex >> 32);
+            ppre[slot] = (uint32_t)ex;
+            poff[slot] = st - (uint32_t)ex;
+            pinfo[slot] = info;
+        }
+        const uint32_t npos = (uint32_t)(*s_total >> 32);
+        const uint32_t total = (uint32_t)*s_total;
+        if (tid == 0) ppre[npos] = total;
+        __syncthreads();
+        const uint32_t per = ((total + PL_THREADS - 1) / PL_THREADS) * 32;
+        const uint32_t t1 = (uint32_t)(warp + 1) * per < total ? (uint32_t)(warp + 1) * per : total;
+        uint32_t t = (uint32_t)warp * per + lane;
+        if (t < t1) {
+            uint32_t p = 0, hi = npos;  // largest p with ppre[p] <= t
+            while (hi - p > 1) {
+                const uint32_t mid = (p + hi) >> 1;
+                if (ppre[mid] <= t) p = mid; else hi = mid;
+            }
+            uint32_t nxt = ppre[p + 1], off = poff[p], inf = pinfo[p];
+            while (t < t1) {
+                uint32_t ent[4], pin[4];
+#pragma unroll
+                for (int k = 0; k < 4; k++) {
+                    const uint32_t tt = t + 32 * k;
+                    if (tt < t1) {
+                        while (tt >= nxt) {
+                            p++;
+                            nxt = ppre[p + 1];
+                            off = poff[p];
+                            inf = pinfo[p];
+                        }
+                        ent[k] = a.B_ent[off + tt];
+                        pin[k] = inf;
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < 4; k++)
+                    if (t + 32 * k < t1) fn(ent[k], pin[k]);
+                t += 128;
+            }
+        }
+        __syncthreads();
+    }
+}
+
+struct DirectOut {
+    U128 sum;        // one partner: this thread's share
+    RowInfo rst;     // this thread's share
+    uint32_t nc = 0, nr = 0, passes = 0;
+    bool failed = false;
+};
+
+template <bool C8>
+__device__ __noinline__ DirectOut direct_anchor(const TwohopArgs &a, uint32_t r, uint32_t range,
+                                                unsigned char *smem, unsigned long long *warp_tot,
+                                                unsigned long long *s_total, unsigned *s_nrw,
+                                                unsigned *s_ncw) {
+    uint32_t *tbl = (uint32_t *)smem;
+    uint32_t *bm = (uint32_t *)(smem + DT_OFF_BM), *pre = (uint32_t *)(smem + DT_OFF_PRE);
+    uint32_t *poff = (uint32_t *)(smem + DT_OFF_POFF), *ppre = (uint32_t *)(smem + DT_OFF_PPRE);
+    uint32_t *pinfo = (uint32_t *)(smem + DT_OFF_PINFO);
+    constexpr uint32_t CELLS = C8 ? DT_CELLS8 : DT_CELLS16;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int l = a.l;
+    const int64_t ebase = a.A_off[r];
+    const int d = (int)(a.A_off[r + 1] - ebase);
+    const uint32_t dp = a.dprime[r], W = (dp + 31) / 32, rsv = a.rsv_c[r];
+    uint32_t *region = a.pool + a.pool_off[r];
+    DirectOut out;
+    if (tid == 0) *s_nrw = *s_ncw = 0;
+    for (uint32_t w0 = 0; w0 < range; w0 += CELLS) {
+        const uint32_t base = r + 1 + w0, nw = range - w0 < CELLS ? range - w0 : CELLS;
+        const uint32_t nbm = (nw + 15) / 16;
+        // counts
+        for (uint32_t i = tid; i < nbm * (C8 ? 2u : 4u); i += PL_THREADS)
+            reinterpret_cast<uint4 *>(tbl)[i] = make_uint4(0, 0, 0, 0);
+        __syncthreads();
+        const uint32_t nr0 = *s_nrw;
+        visit_lists(ebase, d, 0, dp, a, poff, ppre, pinfo, warp_tot, s_total, [&](uint32_t ent, uint32_t inf) {
+            const uint32_t idx = (ent & VMASK) - base;
+            if (idx < nw) {
+                const uint32_t sdiff = (ent ^ inf) >> 31;
+                if constexpr (C8) atomicAdd(&tbl[idx >> 1], 1u << ((idx & 1u) * 16u + sdiff * 8u));
+                else atomicAdd(&tbl[idx], sdiff ? 65536u : 1u);
+            }
+        });
+        out.passes++;
+        long long check = 0;  // self-check: bits written minus bits counted
+        // rows: two bits per rank (same-sign part, different-sign part)
+        for (uint32_t j0 = 0; j0 < nbm; j0 += PL_THREADS) {
+            const uint32_t j = j0 + tid;
+            uint32_t bits = 0;
+            if (j < nbm) {
+                if constexpr (C8) {
+                    const uint32_t lim = (uint32_t)l * 0x01010101u;
+#pragma unroll
+                    for (int h = 0; h < 2; h++) {
+                        const uint4 v = reinterpret_cast<const uint4 *>(tbl)[2 * j + h];
+                        const uint32_t x[4] = {v.x, v.y, v.z, v.w};
+                        if (v.x | v.y | v.z | v.w) {
+#pragma unroll
+                            for (int k = 0; k < 4; k++) {
+                                // bytes >= l to four bits in byte order
+                                const uint32_t m = __vcmpgeu4(x[k], lim) & 0x08040201u;
+                                bits |= (((m * 0x01010101u) >> 24) & 15u) << (16 * h + 4 * k);
+                            }
+                        }
+                    }
+                } else {
+#pragma unroll
+                    for (int h = 0; h < 4; h++) {
+                        const uint4 v = reinterpret_cast<const uint4 *>(tbl)[4 * j + h];
+                        const uint32_t x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                        for (int k = 0; k < 4; k++)
+                            bits |= (((x[k] & 0xFFFFu) >= (uint32_t)l ? 1u : 0u) |
+                                     ((x[k] >> 16) >= (uint32_t)l ? 2u : 0u)) << (8 * h + 2 * k);
+                    }
+                }
+            }
+            const uint32_t cnt = __popc(bits);
+            uint32_t incl = cnt;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(FULL, incl, o);
+                if (lane >= o) incl += t;
+            }
+            const uint32_t tot = __shfl_sync(FULL, incl, 31);
+            if (tot) {
+                const uint32_t ncw = __reduce_add_sync(FULL, (uint32_t)__popc((bits | (bits >> 1)) & 0x55555555u));
+                uint32_t at = 0;
+                if (lane == 0) {
+                    at = atomicAdd(s_nrw, tot);
+                    atomicAdd(s_ncw, ncw);
+                }
+                at = __shfl_sync(FULL, at, 0) + incl - cnt;
+                if (j < nbm) pre[j] = at;
+                uint32_t b = bits;
+                while (b) {
+                    const uint32_t k = __ffs(b) - 1;
+                    b &= b - 1;
+                    const uint32_t x = C8 ? (uint32_t)smem[32 * j + k] : (uint32_t)((uint16_t *)smem)[32 * j + k];
+                    if (a.single) binom_add(out.sum, x, l, &a.cnt->err);
+                    else out.rst.add(x);
+                    check -= x;
+                }
+            }
+            if (j < nbm) bm[j] = bits;
+        }
+        __syncthreads();
+        const uint32_t nrw = *s_nrw - nr0;
+        if (a.single || nrw == 0) {
+            __syncthreads();
+            continue;
+        }
+        if (nr0 + nrw > rsv) {
+            if (tid == 0) atomicOr(&a.cnt->err, CERR_RESERVE);
+            out.failed = true;
+            break;
+        }
+        // mask words, as many at a time as the counters' memory stages
+        uint32_t cw = nrw <= DT_WORDS ? DT_WORDS / nrw : 0u;
+        if (cw > W) cw = W;
+        const bool staged = cw > 0;
+        if (!staged) cw = W;
+        for (uint32_t wa = 0; wa < W; wa += cw) {
+            const uint32_t wn = W - wa < cw ? W - wa : cw;
+            for (uint32_t i = tid; i < wn * nrw; i += PL_THREADS) {
+                if (staged) tbl[i] = 0;
+                else region[(size_t)(i / nrw) * rsv + nr0 + i % nrw] = 0;
+            }
+            __syncthreads();
+            visit_lists(ebase, d, 32 * wa, 32 * (wa + wn) < dp ? 32 * (wa + wn) : dp, a, poff, ppre, pinfo,
+                        warp_tot, s_total, [&](uint32_t ent, uint32_t inf) {
+                            const uint32_t idx = (ent & VMASK) - base;
+                            if (idx >= nw) return;
+                            const uint32_t k = 2 * (idx & 15u) + ((ent ^ inf) >> 31);
+                            const uint32_t bw = bm[idx >> 4];
+                            if (!((bw >> k) & 1u)) return;
+                            const uint32_t row = pre[idx >> 4] + __popc(bw & ((1u << k) - 1u));
+                            const uint32_t bit = inf & VMASK, m = 1u << (bit & 31);
+                            if (staged) atomicOr(&tbl[((bit >> 5) - wa) * nrw + row - nr0], m);
+                            else atomicOr(&region[(size_t)(bit >> 5) * rsv + row], m);
+                        });
+            if (staged) {
+                for (uint32_t i = tid; i < wn * nrw; i += PL_THREADS) {
+                    const uint32_t wd = i / nrw, x = tbl[i];
+                    region[(size_t)(wa + wd) * rsv + nr0 + (i - wd * nrw)] = x;
+                    check += __popc(x);
+                }
+                __syncthreads();
+            }
+        }
+        out.passes++;
+        if (a.check && staged) {
+            // self-check: the window's rows hold as many bits as its counters say
+            block_excl_scan_u64((unsigned long long)check, warp_tot, s_total);
+            if (*s_total != 0 && tid == 0) atomicOr(&a.cnt->err, CERR_MASK);
+            __syncthreads();
+        }
+    }
+    __syncthreads();
+    out.nr = *s_nrw;
+    out.nc = *s_ncw;
+    return out;
+}
+
 __device__ __forceinline__ unsigned long long global_ns() {
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -759,7 +1033,7 @@ __device__ __forceinline__ unsigned long long global_ns() {
 }
 
 template <bool STATS>
-__global__ void __launch_bounds__(PL_THREADS) k_twohop_large(TwohopArgs a) {
+__global__ void __launch_bounds__(PL_THREADS, 2) k_twohop_large(TwohopArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint32_t *keys = (uint32_t *)smem_raw;
     unsigned long long *vals = (unsigned long long *)(smem_raw + PL_OFF_VALS);
@@ -910,8 +1184,24 @@ __global__ void __launch_bounds__(PL_THREADS) k_twohop_large(TwohopArgs a) {
         };
 
         const int lgb = bucket_lg(e_vis);
-        bool bucketed = false;
-        if (e_vis <= (unsigned long long)a.wcap) {
+        bool bucketed = false, direct = false;
+        if constexpr (!STATS) {
+            const uint32_t range = a.n_ranks - 1 - r;
+            direct = a.direct && direct_takes(e_use, a.dprime[r], range);
+            if (direct) {
+                DirectOut o = a.dprime[r] <= 255u
+                    ? direct_anchor<true>(a, r, range, smem_raw, warp_tot, &s_total, &s_nrw, &s_ncw)
+                    : direct_anchor<false>(a, r, range, smem_raw, warp_tot, &s_total, &s_nrw, &s_ncw);
+                nc = o.nc;
+                nr = o.nr;
+                failed = o.failed;
+                rst = o.rst;
+                if (sum.add(o.sum)) atomicOr(&a.cnt->err, CERR_OVERFLOW);
+                reads = e_use * o.passes;
+            }
+        }
+        if (direct) {
+        } else if (e_vis <= (unsigned long long)a.wcap) {
             // one window
             uint32_t hs = (uint32_t)((2 * e_vis + 31) & ~31ull);
             hs = hs < 64 ? 64 : (hs > PL_HS ? PL_HS : hs);
@@ -1035,7 +1325,7 @@ __global__ void __launch_bounds__(PL_THREADS) k_twohop_large(TwohopArgs a) {
                 }
             }
         }
-        if (!bucketed && !failed && e_vis > (unsigned long long)a.wcap) {
+        if (!direct && !bucketed && !failed && e_vis > (unsigned long long)a.wcap) {
             // re-read windows: every pass over the 2-hop keeps one hash class
             const U128 sum0 = sum;
             int lg_nw = 0;
@@ -1548,6 +1838,8 @@ struct CountRun {
         ta.nrow = nrow.ptr;
         ta.rinfo = rinfo.ptr;
         ta.single = R == 1;
+        ta.n_ranks = (uint32_t)nX;
+        ta.direct = hash_slots_cap() == 0 && twohop_window_wedges() == (uint32_t)PL_WCAP;
         ta.cnt = cnt.ptr;
         ta.l = l;
         ta.check = spec.check ? 1 : 0;
