@@ -1731,7 +1731,7 @@ struct CountRun {
         std::vector<TcInput> h(n);
         SBC_CUDA(cudaMemcpyAsync(h.data(), tin.ptr, sizeof(TcInput) * n, cudaMemcpyDeviceToHost, s));
         SBC_CUDA(cudaStreamSynchronize(s));
-        TcPlan plan = tc_plan(h, tc_budget_bytes());
+        TcPlan plan = tc_plan(h, spec.l, tc_budget_bytes());
         tc_upload(plan, s);
         const size_t need = (size_t)plan.max_blocks * (size_t)kTcBlockBytes;
         if (need > zbuf.bytes()) zbuf.alloc(need, s);

@@ -259,16 +259,22 @@ void apply_tune(CountSpec &spec, const sbc_tune_t *t);
 
 // ---------------------------------------------------------------- tensor-core pairs
 
-// Tensor-core form of the two-partner tuple step for wide anchors
-// (tc_pairs.cu). One anchor of a chunk:
+// Tensor-core form of the two-partner tuple step (tc_pairs.cu). One anchor of
+// a chunk:
 struct TcAnchor {
     uint32_t r;          // anchor rank
     uint32_t nr, W, rsv; // rows, mask words, row stride of its pool region
+    uint32_t longest;    // most positions of a row: bounds every Gram entry
     uint32_t RB, KB;     // Z row blocks of 128 (even), position blocks of 128
-    uint32_t longest, pad;  // most positions of a row: bounds every Gram entry
+    uint32_t tiles;      // 128 x 256 output tiles
     int64_t pool_off;    // its pool region (words)
     int64_t zblk0;       // first Z block (16 KB each) in the chunk's arena
-    int64_t tile0;       // first output tile in the chunk
+    int64_t job0;        // first job in the chunk
+};
+// Some consecutive tiles (local .. local + count - 1) of one anchor.
+struct TcJob {
+    int64_t zblk0;
+    uint32_t r, KB, longest, local, count, pad;
 };
 struct TcInput {
     uint32_t r, nr, W, rsv, longest;
@@ -277,9 +283,9 @@ struct TcInput {
 struct TcChunk {
     std::vector<TcAnchor> host;
     DevBuf<TcAnchor> dev;
-    DevBuf<uint32_t> job;  // anchor of every job's first tile
-    int64_t n_blocks = 0, n_tiles = 0;
-    int job_tiles = 1;     // tiles per job
+    DevBuf<TcJob> jobs;
+    int64_t n_blocks = 0, n_tiles = 0, n_jobs = 0;
+    int job_tiles = 1, epi = 0;  // tiles per job; epilogue of its anchors
 };
 struct TcPlan {
     std::vector<TcChunk> chunks;
@@ -289,9 +295,8 @@ struct TcPlan {
 struct TcArgs {
     const TcAnchor *anc = nullptr;
     int n_anc = 0;
-    int64_t n_blocks = 0, n_tiles = 0;
-    uint32_t *job = nullptr;
-    int job_tiles = 1;
+    const TcJob *jobs = nullptr;
+    int64_t n_jobs = 0, n_blocks = 0;
     const uint32_t *pool = nullptr;
     unsigned char *z = nullptr;
     int l = 0;
@@ -302,8 +307,9 @@ struct TcArgs {
     unsigned long long big64 = 0;  // largest x with binom(x, l) by the 64-bit formula
 };
 // Chunks of at most budget_bytes of Z (an anchor larger than that forms a
-// chunk of its own).
-TcPlan tc_plan(const std::vector<TcInput> &in, int64_t budget_bytes);
+// chunk of its own), their anchors sharing one epilogue for other sides of l.
+TcPlan tc_plan(const std::vector<TcInput> &in, int l, int64_t budget_bytes);
+// Device copies of the plan and its job records.
 void tc_upload(TcPlan &plan, cudaStream_t s);
 void tc_ensure_attrs();
 // Expansion + pair kernels of every chunk, in stream order (no host sync).

@@ -12,25 +12,37 @@
 // row pairs a < b, binom(G[a][b], l) with G = Z Z^T. This is a dense
 // contraction over the positions, so it runs on the tensor cores:
 //
-// * k_zexpand writes Z as fp8 e4m3 bytes (1.0 or 0) in 16 KB blocks of 128
-//   rows x 128 positions, each block already in the shared-memory layout of
-//   the MMA (K-major, 128-byte swizzle: 16-byte chunk c of row r stored at
-//   chunk c ^ (r & 7)), so a block moves to shared memory with one plain
-//   bulk copy.
-// * k_tcpairs is a persistent kernel over output tiles of 128 x 256 rows of
-//   G (only tiles that hold a pair a < b). Per CTA: one
-//   producer warp issues the bulk copies into a 4-stage ring, one warp issues
-//   tcgen05.mma (kind::f8f6f4, M = 128, N = 256, K = 32 per instruction)
-//   into one of two TMEM accumulators, and eight epilogue warps read the
-//   accumulator with tcgen05.ld, convert each entry to an integer, and add
-//   binom(G[a][b], l) (32-bit table lookups when the anchor's positions
-//   bound every entry, else a 64-bit table up to 256 and exact 128-bit
-//   arithmetic above). The fp32 accumulator holds these integer sums exactly (each is
-//   at most d' < 2^21 < 2^24).
+// * k_zexpand writes Z as fp8 e4m3 bytes in 16 KB blocks of 128 rows x 128
+//   positions, each block already in the shared-memory layout of the MMA
+//   (K-major, 128-byte swizzle: 16-byte chunk c of row r at chunk c ^ (r & 7)),
+//   so a block moves to shared memory with one plain bulk copy. A set bit is
+//   the byte 0x08 = 2^-6, so a product is 2^-12 and every sum an exact multiple
+//   of it.
+// * k_tcpairs is a persistent kernel over output tiles of 128 x 256 rows of G
+//   (only tiles that hold a pair a < b). Per CTA one thread issues the bulk
+//   copies and one tcgen05.mma (kind::f8f6f4, M = 128, N = 256, K = 32 per
+//   instruction; 512 cycles per 128 positions) into one of two TMEM
+//   accumulators; the fp32 accumulator holds the sums exactly (at most d' <
+//   2^21 < 2^24 units of 2^-12). The tiles of a column of 256 rows follow one
+//   another, so their B blocks stay in shared memory for the run (anchors of at
+//   most 384 positions) and a tile reads only its A block, 16 KB instead of
+//   48 KB per 128 positions. (Expanding the bits in the kernel instead, four
+//   warps per block, was slower: 1,325 cycles per block.)
+//   Sixteen epilogue warps read the accumulator with tcgen05.ld and add
+//   binom(G[a][b], l): the sum of l! binom(x, l) = x (x - 1) .. (x - l + 1) in
+//   packed fp32 multiply-adds, exact below 2^24, 1 to 2 instructions per entry
+//   and no shared-memory lookups; long rows take a table (32-bit, or 64-bit
+//   with exact 128-bit arithmetic above 256). The packed chains are bound by
+//   latency, hence four warps per scheduler.
+//   Work comes in jobs of consecutive tiles of one anchor, whose records every
+//   role prefetches one ahead; the loops of the copying and the issuing thread
+//   run over the blocks of a run of tiles (their instructions, a few cycles
+//   each, were 2,100 cycles per tile when every tile was set up anew), and a
+//   chunk's anchors share one epilogue, so each kernel holds only its own.
 //
 // Every wait on an mbarrier is bounded by a clock limit; a wait that runs out
-// sets the error word, every role stops, copies and MMAs in flight are
-// waited for (again bounded), TMEM is freed and the kernel returns.
+// sets the error word, every role stops, copies and MMAs in flight are waited
+// for (again bounded), TMEM is freed and the kernel returns.
 #include <algorithm>
 #include <vector>
 
@@ -40,12 +52,12 @@ namespace sbc {
 
 namespace {
 
-constexpr int TC_THREADS = 320;  // warp 0 producer, warp 1 MMA, warps 2..9 epilogue
-constexpr int TC_EPI_WARPS = 8;  // two per TMEM lane group, each on half the columns
-constexpr int TC_STAGES = 4;
-constexpr uint32_t TC_BLOCK = 16384;           // one Z block: 128 rows x 128 bytes
-constexpr uint32_t TC_STAGE = 3 * TC_BLOCK;    // A (128 rows) + B (256 rows)
-constexpr size_t TC_SMEM = (size_t)TC_STAGES * TC_STAGE + 1024;  // + alignment slack
+constexpr int TC_EPI_WARPS = 16;   // warps 2..17: four per TMEM lane group, 64 columns each
+constexpr int TC_THREADS = 32 * (2 + TC_EPI_WARPS);  // warp 0 MMA, warp 1 copies
+constexpr uint32_t TC_BLOCK = 16384;           // one operand block: 128 rows x 128 bytes
+constexpr int TC_A = 7;                        // ring of A blocks (128 rows)
+constexpr int TC_B = 3;                        // ring of B block pairs (256 rows)
+constexpr size_t TC_SMEM = (size_t)(TC_A + 2 * TC_B) * TC_BLOCK + 1024;  // + alignment slack
 constexpr int TC_TMEM_COLS = 512;              // two 128 x 256 fp32 accumulators
 constexpr int TC_BINOM = 256;
 constexpr long long TC_WAIT_CYCLES = 4000000000ll;  // about 2 s at the SM clock
@@ -112,23 +124,21 @@ __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t by
         : "memory");
 }
 
-// Shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups
-// 1024 bytes apart.
-__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
-    uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)1 << 16;             // leading byte offset (unused for this layout)
-    d |= (uint64_t)(1024 >> 4) << 32;   // stride byte offset
-    d |= (uint64_t)1 << 46;             // descriptor version
-    d |= (uint64_t)2 << 61;             // 128-byte swizzle
-    return d;
-}
+// Shared-memory matrix descriptor (K-major, 128-byte swizzle, 8-row groups 1024
+// bytes apart): the upper word is the stride byte offset, the version and the
+// swizzle mode, the lower word the address in 16-byte units and the (unused)
+// leading byte offset. Four MMAs cover a 128-position block, 32 bytes each.
+constexpr uint32_t TC_DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) { return (saddr >> 4) | (1u << 16); }
 
-__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t accum) {
+__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t accum) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-        "l"(a), "l"(b), "r"(TC_IDESC), "r"(accum));
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "mov.b64 da, {%1, %3};\n\t"
+        "mov.b64 db, {%2, %3};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], da, db, %4, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_lo), "r"(b_lo), "r"(TC_DESC_HI), "r"(TC_IDESC), "r"(accum));
 }
 __device__ __forceinline__ void tc_commit(uint64_t *bar) {
     asm volatile(
@@ -143,7 +153,8 @@ __device__ __forceinline__ void tc_fence_after() {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// 32 consecutive fp32 columns of this thread's TMEM lane.
+// 32 consecutive fp32 columns of this thread's TMEM lane: the load is issued,
+// and its registers may be read after tmem_wait on them.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
@@ -156,7 +167,112 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
           "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]),
           "=r"(v[31])
         : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+// Waits for every load this warp issued; the operands keep uses of v after it.
+__device__ __forceinline__ void tmem_wait(uint32_t (&v)[32]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]),
+                   "+r"(v[7]), "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]),
+                   "+r"(v[13]), "+r"(v[14]), "+r"(v[15]), "+r"(v[16]), "+r"(v[17]), "+r"(v[18]),
+                   "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]), "+r"(v[24]),
+                   "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]),
+                   "+r"(v[31])
+                 :
+                 : "memory");
+}
+
+// Packed pairs of fp32 (two lanes of one 64-bit register).
+__device__ __forceinline__ uint64_t f2_pack(uint32_t a, uint32_t b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(a), "r"(b));
+    return r;
+}
+__device__ __forceinline__ void f2_unpack(uint64_t v, uint32_t &a, uint32_t &b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=r"(a), "=r"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t f2_both(float x) {
+    return f2_pack(__float_as_uint(x), __float_as_uint(x));
+}
+
+// Longest row up to which the packed epilogue is exact. FLOAT: 16 values of
+// x (x - 1) .. (x - l + 1) per fp32 lane sum below 2^24. INT: one value stays
+// below 2^23, so that value + 2^23 carries it in its low bits; 128 of them sum
+// below 2^32.
+template <int L, bool INT>
+__host__ __device__ constexpr uint32_t tc_poly_max() {
+    if (L < 2 || L > 4) return 0;
+    uint32_t best = 0;
+    for (uint32_t x = L; x <= 2048; x++) {
+        unsigned long long f = 1;
+        for (int i = 0; i < L; i++) f *= x - i;
+        if (INT ? f >= (1ull << 23) : 16 * f >= (1ull << 24)) break;
+        best = x;
+    }
+    return best;
+}
+
+// Accumulator entries are multiples of this unit; 2^23 units as a float.
+constexpr float TC_UNIT = 1.0f / 4096.0f;
+constexpr uint32_t TC_BASE = 0x4B000000u - (12u << 23);
+
+// Sum of x (x - 1) .. (x - L + 1) over the 32 entries (integers in units of
+// TC_UNIT, so the product carries TC_UNIT^L); with MASK only over the entries
+// j >= first.
+template <int L, bool INT, bool MASK>
+__device__ __forceinline__ uint32_t poly_sum(const uint32_t (&v)[32], int first) {
+    uint64_t acc = f2_both(0.0f);
+    constexpr float U = TC_UNIT, UL = L == 2 ? U * U : L == 3 ? U * U * U : U * U * U * U;
+    const uint64_t base = f2_both(8388608.0f * UL), m1 = f2_both(-U), m3 = f2_both(-3.0f * U),
+                   p2 = f2_both(2.0f * U * U);
+    uint32_t isum = 0;
+#pragma unroll
+    for (int j = 0; j < 32; j += 2) {
+        uint64_t x;
+        if constexpr (MASK) x = f2_pack(j >= first ? v[j] : 0u, j + 1 >= first ? v[j + 1] : 0u);
+        else x = f2_pack(v[j], v[j + 1]);
+        // the last factor is multiplied into the accumulator
+        uint64_t a, b;
+        if constexpr (L == 2) {
+            a = x;
+            b = f2_add(x, m1);
+        } else if constexpr (L == 3) {
+            a = f2_fma(x, f2_add(x, m3), p2);
+            b = x;
+        } else {
+            a = f2_mul(x, f2_add(x, m3));
+            b = f2_add(a, p2);
+        }
+        if constexpr (INT) {
+            uint32_t r0, r1;
+            f2_unpack(f2_fma(a, b, base), r0, r1);
+            isum += r0 + r1;
+        } else {
+            acc = f2_fma(a, b, acc);
+        }
+    }
+    if constexpr (INT) {
+        // a power of two times the integer: only the exponent field differs
+        constexpr uint32_t EXP = 0x4B000000u - (12u * L << 23);
+        return isum - 32u * EXP;
+    }
+    uint32_t r0, r1;
+    f2_unpack(acc, r0, r1);
+    return (uint32_t)(__uint_as_float(r0) * (1.0f / UL)) + (uint32_t)(__uint_as_float(r1) * (1.0f / UL));
 }
 
 // binom(x, l) exactly for x > TC_BINOM (128-bit multiplicative formula; the
@@ -203,12 +319,13 @@ __device__ __noinline__ U128 tc_binom_big(unsigned long long x, int l, unsigned 
 
 }  // namespace
 
-// Expand the chunk's candidate masks into Z blocks (see the file comment).
+// Expand the chunk's rows into Z blocks (see the file comment). A CTA expands
+// consecutive blocks: one search for its first anchor, then a walk over the few
+// anchors of its range (with strided blocks every CTA walked the records of all
+// anchors, a dependent load each). Eight lanes write one row's 128 bytes, so a
+// warp's store covers four whole lines (one row per lane wrote a sixteenth of
+// 32 lines at a time).
 __global__ void __launch_bounds__(512) k_zexpand(TcArgs a) {
-    const int r = threadIdx.x & 127, wi = threadIdx.x >> 7;
-    // a CTA expands consecutive blocks: one search for its first anchor, then a
-    // walk over the few anchors of its range (with strided blocks every CTA
-    // walked the records of all anchors, a dependent load each)
     const int64_t per = (a.n_blocks + gridDim.x - 1) / gridDim.x;
     const int64_t b0 = blockIdx.x * per, b1 = b0 + per < a.n_blocks ? b0 + per : a.n_blocks;
     if (b0 >= b1) return;
@@ -217,80 +334,86 @@ __global__ void __launch_bounds__(512) k_zexpand(TcArgs a) {
         const int mid = (ai + hi) >> 1;
         if (a.anc[mid].zblk0 <= b0) ai = mid; else hi = mid;
     }
-    ai--;
-    int64_t next0 = b0;
-    TcAnchor A;
+    TcAnchor A = a.anc[ai];
+    const uint32_t c = threadIdx.x & 7;  // 16-byte chunk: positions 16 c .. 16 c + 15
+    uint32_t rb = (uint32_t)((b0 - A.zblk0) / A.KB), kb = (uint32_t)((b0 - A.zblk0) % A.KB);
     for (int64_t blk = b0; blk < b1; blk++) {
-        while (blk >= next0) {
-            A = a.anc[++ai];
-            next0 = ai + 1 < a.n_anc ? a.anc[ai + 1].zblk0 : a.n_blocks;
-        }
-        const int64_t local = blk - A.zblk0;
-        const uint32_t rb = (uint32_t)(local / A.KB), kb = (uint32_t)(local % A.KB);
-        const uint32_t row = rb * 128 + r, w = kb * 4 + wi;
-        uint32_t bits = 0;
-        if (row < A.nr && w < A.W) bits = a.pool[A.pool_off + (int64_t)w * A.rsv + row];
-        // 32 positions -> 32 bytes of 0x38 (e4m3 1.0) or 0: each nibble is
-        // spread to the low bit of 4 bytes and scaled
-        uint32_t o[8];
+        const uint32_t w = 4 * kb + (c >> 1);
 #pragma unroll
-        for (int k = 0; k < 8; k++)
-            o[k] = ((((bits >> (4 * k)) & 0xFu) * 0x00204081u) & 0x01010101u) * 0x38u;
-        unsigned char *dst = a.z + blk * (int64_t)TC_BLOCK + r * 128;
-        const int ch0 = 2 * wi, ch1 = 2 * wi + 1;
-        *reinterpret_cast<uint4 *>(dst + ((ch0 ^ (r & 7)) << 4)) = make_uint4(o[0], o[1], o[2], o[3]);
-        *reinterpret_cast<uint4 *>(dst + ((ch1 ^ (r & 7)) << 4)) = make_uint4(o[4], o[5], o[6], o[7]);
+        for (int h = 0; h < 2; h++) {
+            const uint32_t r = (threadIdx.x >> 3) + 64 * h, row = rb * 128 + r;
+            uint32_t bits = 0;
+            if (row < A.nr && w < A.W) bits = a.pool[A.pool_off + (int64_t)w * A.rsv + row] >> ((c & 1) * 16);
+            // each nibble is spread to bit 3 of 4 bytes
+            uint32_t o[4];
+#pragma unroll
+            for (int k = 0; k < 4; k++) o[k] = (((bits >> (4 * k)) & 0xFu) * 0x01020408u) & 0x08080808u;
+            *reinterpret_cast<uint4 *>(a.z + blk * (int64_t)TC_BLOCK + r * 128 + ((c ^ (r & 7)) << 4)) =
+                make_uint4(o[0], o[1], o[2], o[3]);
+        }
+        if (++kb == A.KB) {
+            kb = 0;
+            if (++rb == A.RB && blk + 1 < b1) {
+                rb = 0;
+                A = a.anc[++ai];
+            }
+        }
     }
 }
 
 namespace {
 
-// Walks the tiles of one CTA: jobs of a.job_tiles consecutive tiles, job
-// blockIdx.x, + gridDim.x, ... Tile t of the chunk, its anchor and block
-// coordinates (I rows of 128, J columns of 256; column J holds the rows
-// I = 0 .. 2J + 1, the tiles with a pair a < b). A job starts at the anchor
-// that k_tcjobs noted for it and walks forward inside the job only: with single
-// strided tiles every role of every CTA walked all anchors of the chunk
-// (medium graph, (3,3): 25 ns per tile of the whole GPU against 10 ns).
-struct TileCursor {
-    int64_t t = 0, end = 0, job, next0 = 0;  // next0: first tile of the next anchor
-    int ai = 0;
-    TcAnchor A;
-    uint32_t I = 0, J = 0;
-    __device__ __forceinline__ TileCursor() : job((int64_t)blockIdx.x - gridDim.x) {}
-    // Moves to the CTA's next tile; false when there is none.
+// Jobs of every anchor (thread per anchor).
+__global__ void k_tcjobs(const TcAnchor *anc, int n_anc, int job_tiles, TcJob *jobs) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_anc; i += gridDim.x * blockDim.x) {
+        const TcAnchor A = anc[i];
+        TcJob j;
+        j.zblk0 = A.zblk0;
+        j.r = A.r;
+        j.KB = A.KB;
+        j.longest = A.longest;
+        for (uint32_t t = 0; t < A.tiles; t += job_tiles) {
+            j.local = t;
+            j.count = A.tiles - t < (uint32_t)job_tiles ? A.tiles - t : (uint32_t)job_tiles;
+            jobs[A.job0 + t / job_tiles] = j;
+        }
+    }
+}
+
+// Walks the runs of one CTA: jobs blockIdx.x, + gridDim.x, ..., each some
+// consecutive tiles of one anchor. Block coordinates of a tile: I rows of 128,
+// J columns of 256; column J holds the rows I = 0 .. 2J + 1 (the tiles with a
+// pair a < b), so J (J + 1) tiles come before it. A run is the tiles of a job in
+// one column: rows I .. I + n - 1. The next job's record is loaded while this
+// one runs.
+struct RunCursor {
+    TcJob A, ahead;
+    int64_t job;       // of `ahead`
+    uint32_t left = 0; // tiles of this job after the current run
+    uint32_t I = 0, J = 0, n = 0;
+    __device__ __forceinline__ RunCursor(const TcArgs &a) : job(blockIdx.x) {
+        if (job < a.n_jobs) ahead = a.jobs[job];
+    }
     __device__ __forceinline__ bool next(const TcArgs &a) {
-        if (++t >= end) {
+        if (left) {
+            I = 0;
+            J++;
+        } else {
+            if (job >= a.n_jobs) return false;
+            A = ahead;
             job += gridDim.x;
-            t = job * a.job_tiles;
-            if (t >= a.n_tiles) return false;
-            end = t + a.job_tiles < a.n_tiles ? t + a.job_tiles : a.n_tiles;
-            ai = (int)a.job[job] - 1;
-            next0 = t;
+            if (job < a.n_jobs) ahead = a.jobs[job];
+            left = A.count;
+            J = (uint32_t)((sqrtf(4.0f * (float)A.local + 1.0f) - 1.0f) * 0.5f);
+            while (J * (J + 1) > A.local) J--;
+            while ((J + 1) * (J + 2) <= A.local) J++;
+            I = A.local - J * (J + 1);
         }
-        if (t >= next0) {
-            do {
-                ai++;
-                next0 = ai + 1 < a.n_anc ? a.anc[ai + 1].tile0 : a.n_tiles;
-            } while (t >= next0);
-            A = a.anc[ai];
-            J = 0;
-        }
-        // columns before J hold J (J + 1) tiles
-        const uint64_t local = (uint64_t)(t - A.tile0);
-        while ((uint64_t)(J + 1) * (J + 2) <= local) J++;
-        I = (uint32_t)(local - (uint64_t)J * (J + 1));
+        n = min(left, 2 * J + 2 - I);
+        left -= n;
         return true;
     }
 };
-
-// Anchor of every job's first tile (thread per anchor).
-__global__ void k_tcjobs(TcArgs a) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.n_anc; i += gridDim.x * blockDim.x) {
-        const int64_t t0 = a.anc[i].tile0, t1 = i + 1 < a.n_anc ? a.anc[i + 1].tile0 : a.n_tiles;
-        for (int64_t j = (t0 + a.job_tiles - 1) / a.job_tiles; j * a.job_tiles < t1; j++) a.job[j] = (uint32_t)i;
-    }
-}
 
 }  // namespace
 
@@ -320,30 +443,40 @@ __host__ __device__ constexpr uint32_t tc_fast_max() {
     return best;
 }
 
-template <int L>
+// Epilogue of a chunk's anchors, by their longest row: packed fp32 sums, packed
+// with integer sums, tables.
+enum : int { EPI_FLOAT = 0, EPI_INT = 1, EPI_TABLE = 2 };
+
+template <int L, int EPI>
 __global__ void __launch_bounds__(TC_THREADS, 1) k_tcpairs(TcArgs a) {
     extern __shared__ __align__(16) unsigned char tc_smem_raw[];
-    __shared__ __align__(8) uint64_t full[TC_STAGES], empty[TC_STAGES], acc_full[2], acc_empty[2],
-        mma_done;
+    __shared__ __align__(8) uint64_t full_a[TC_A], empty_a[TC_A], full_b[TC_B], empty_b[TC_B];
+    __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2], mma_done;
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_abort;
     // binom(x, L) for x <= TC_BINOM, zero below L and at TC_BINOM + 1 (the
-    // clamped index of larger entries, which a slower path adds)
-    __shared__ unsigned long long s_bt[TC_BINOM + 2];
-    // binom(x, L) for x <= FAST in 32 bits (anchors with 32 W <= FAST)
+    // clamped index of larger entries, which a slower path adds), and for x <=
+    // FAST in 32 bits (anchors whose longest row is that short)
     constexpr uint32_t FAST = tc_fast_max<L>();
-    __shared__ uint32_t s_bt32[FAST + 1];
+    __shared__ unsigned long long s_bt[EPI == EPI_TABLE ? TC_BINOM + 2 : 1];
+    __shared__ uint32_t s_bt32[EPI == EPI_TABLE ? FAST + 1 : 1];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     unsigned char *smem =
         (unsigned char *)(((uintptr_t)tc_smem_raw + 1023) & ~(uintptr_t)1023);
-    for (int x = tid; x <= TC_BINOM + 1; x += TC_THREADS)
-        s_bt[x] = (x >= L && x <= TC_BINOM) ? binom_u64c<L>(x) : 0ull;
-    for (int x = tid; x <= (int)FAST; x += TC_THREADS)
-        s_bt32[x] = x >= L ? (uint32_t)binom_u64c<L>(x) : 0u;
+    if constexpr (EPI == EPI_TABLE) {
+        for (int x = tid; x <= TC_BINOM + 1; x += TC_THREADS)
+            s_bt[x] = (x >= L && x <= TC_BINOM) ? binom_u64c<L>(x) : 0ull;
+        for (int x = tid; x <= (int)FAST; x += TC_THREADS)
+            s_bt32[x] = x >= L ? (uint32_t)binom_u64c<L>(x) : 0u;
+    }
     if (tid == 0) {
-        for (int s = 0; s < TC_STAGES; s++) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], 1);
+        for (int s = 0; s < TC_A; s++) {
+            mbar_init(&full_a[s], 1);
+            mbar_init(&empty_a[s], 1);
+        }
+        for (int s = 0; s < TC_B; s++) {
+            mbar_init(&full_b[s], 1);
+            mbar_init(&empty_b[s], 1);
         }
         for (int b = 0; b < 2; b++) {
             mbar_init(&acc_full[b], 1);
@@ -353,7 +486,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tcpairs(TcArgs a) {
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 1) {
+    if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_u32(&s_tmem)),
                      "r"(TC_TMEM_COLS)
@@ -364,76 +497,140 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tcpairs(TcArgs a) {
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = s_tmem;
+    unsigned char *smem_b = smem + (size_t)TC_A * TC_BLOCK;
 
-    if (warp == 0) {
-        // ---- producer: bulk copies of the A block and the two B blocks
+    if (warp == 1) {
+        // ---- copies. A run's A blocks are consecutive in Z. With KB <= TC_B the
+        // run's B pairs come first and stay; else pair kb before A block kb.
         if (lane == 0) {
-            uint32_t stage = 0, round = 0;
-            int issued[TC_STAGES] = {0, 0, 0, 0};
-            uint32_t issued_par[TC_STAGES] = {0, 0, 0, 0};
-            TileCursor tr;
-            while (!s_abort && tr.next(a)) {
-                const TcAnchor &A = tr.A;
-                const unsigned char *zA = a.z + (A.zblk0 + (int64_t)tr.I * A.KB) * TC_BLOCK;
-                const unsigned char *zB0 = a.z + (A.zblk0 + (int64_t)(2 * tr.J) * A.KB) * TC_BLOCK;
-                const unsigned char *zB1 = zB0 + (int64_t)A.KB * TC_BLOCK;
-                for (uint32_t kb = 0; kb < A.KB; kb++) {
-                    if (!mbar_wait(&empty[stage], (round & 1) ^ 1, &s_abort, a.err)) break;
-                    unsigned char *st = smem + (size_t)stage * TC_STAGE;
-                    mbar_expect_tx(&full[stage], TC_STAGE);
-                    bulk_g2s(st, zA + (int64_t)kb * TC_BLOCK, TC_BLOCK, &full[stage]);
-                    bulk_g2s(st + TC_BLOCK, zB0 + (int64_t)kb * TC_BLOCK, TC_BLOCK, &full[stage]);
-                    bulk_g2s(st + 2 * TC_BLOCK, zB1 + (int64_t)kb * TC_BLOCK, TC_BLOCK, &full[stage]);
-                    issued[stage] = 1;
-                    issued_par[stage] = round & 1;
-                    if (++stage == TC_STAGES) {
-                        stage = 0;
-                        round++;
-                    }
+            uint32_t sa = 0, ra = 0, sb = 0, rb = 0;  // ring slots and rounds
+            uint32_t used_a = 0, used_b = 0;          // slots ever filled
+            RunCursor tr(a);
+            auto push_a = [&](const unsigned char *z) -> bool {
+                if (!mbar_wait(&empty_a[sa], (ra & 1) ^ 1, &s_abort, a.err)) return false;
+                mbar_expect_tx(&full_a[sa], TC_BLOCK);
+                bulk_g2s(smem + (size_t)sa * TC_BLOCK, z, TC_BLOCK, &full_a[sa]);
+                used_a |= 1u << sa;
+                if (++sa == TC_A) {
+                    sa = 0;
+                    ra++;
+                }
+                return true;
+            };
+            auto push_b = [&](const unsigned char *z0, const unsigned char *z1) -> bool {
+                if (!mbar_wait(&empty_b[sb], (rb & 1) ^ 1, &s_abort, a.err)) return false;
+                unsigned char *st = smem_b + (size_t)sb * 2 * TC_BLOCK;
+                mbar_expect_tx(&full_b[sb], 2 * TC_BLOCK);
+                bulk_g2s(st, z0, TC_BLOCK, &full_b[sb]);
+                bulk_g2s(st + TC_BLOCK, z1, TC_BLOCK, &full_b[sb]);
+                used_b |= 1u << sb;
+                if (++sb == TC_B) {
+                    sb = 0;
+                    rb++;
+                }
+                return true;
+            };
+            bool ok = true;
+            while (ok && !s_abort && tr.next(a)) {
+                const uint32_t KB = tr.A.KB;
+                const size_t row_bytes = (size_t)KB * TC_BLOCK;  // of one row of blocks
+                const unsigned char *z = a.z + tr.A.zblk0 * (int64_t)TC_BLOCK;
+                const unsigned char *zA = z + tr.I * row_bytes;
+                const unsigned char *zB = z + 2 * tr.J * row_bytes;
+                if (KB <= (uint32_t)TC_B) {
+                    for (uint32_t kb = 0; kb < KB && ok; kb++)
+                        ok = push_b(zB + kb * TC_BLOCK, zB + row_bytes + kb * TC_BLOCK);
+                    const uint32_t blocks = tr.n * KB;
+                    for (uint32_t b = 0; b < blocks && ok; b++, zA += TC_BLOCK) ok = push_a(zA);
+                } else {
+                    for (uint32_t i = 0; i < tr.n && ok; i++)
+                        for (uint32_t kb = 0; kb < KB && ok; kb++, zA += TC_BLOCK)
+                            ok = push_b(zB + (size_t)kb * TC_BLOCK, zB + row_bytes + (size_t)kb * TC_BLOCK) &&
+                                 push_a(zA);
                 }
             }
             if (s_abort) {
                 // let every copy this thread started land before the CTA exits
-                for (int s = 0; s < TC_STAGES; s++)
-                    if (issued[s]) {
+                // (a slot's last round is one less where the ring has not
+                // reached it again)
+                for (int s = 0; s < TC_A; s++)
+                    if ((used_a >> s) & 1u) {
+                        const uint32_t last = (uint32_t)s < sa ? ra : ra - 1;
                         const long long t0 = clock64();
-                        while (!mbar_try(&full[s], issued_par[s]) && clock64() - t0 < TC_WAIT_CYCLES) {
+                        while (!mbar_try(&full_a[s], last & 1) && clock64() - t0 < TC_WAIT_CYCLES) {
+                        }
+                    }
+                for (int s = 0; s < TC_B; s++)
+                    if ((used_b >> s) & 1u) {
+                        const uint32_t last = (uint32_t)s < sb ? rb : rb - 1;
+                        const long long t0 = clock64();
+                        while (!mbar_try(&full_b[s], last & 1) && clock64() - t0 < TC_WAIT_CYCLES) {
                         }
                     }
             }
         }
-    } else if (warp == 1) {
+        __syncwarp();
+    } else if (warp == 0) {
         // ---- MMA issue
         if (lane == 0) {
-            uint32_t stage = 0, round = 0, it = 0;
-            const uint32_t sbase = smem_u32(smem);
-            TileCursor tr;
-            for (; !s_abort && tr.next(a); it++) {
-                const TcAnchor &A = tr.A;
-                const uint32_t buf = it & 1;
-                if (!mbar_wait(&acc_empty[buf], ((it >> 1) & 1) ^ 1, &s_abort, a.err)) break;
+            uint32_t sa = 0, ra = 0, sb = 0, rb = 0, it = 0;
+            const uint32_t alo = desc_lo(smem_u32(smem)), blo = desc_lo(smem_u32(smem_b));
+            RunCursor tr(a);
+            bool ok = true;
+            // one 128-position step: A slot sa against the B pair at blk
+            auto step = [&](uint32_t d_tmem, uint32_t pair, uint32_t accum) -> bool {
+                if (!mbar_wait(&full_a[sa], ra & 1, &s_abort, a.err)) return false;
                 tc_fence_after();
-                const uint32_t d_tmem = tmem + buf * 256;
-                bool ok = true;
-                for (uint32_t kb = 0; kb < A.KB; kb++) {
-                    if (!mbar_wait(&full[stage], round & 1, &s_abort, a.err)) {
+                const uint32_t pa = alo + sa * (TC_BLOCK >> 4), pb = blo + pair * (2 * TC_BLOCK >> 4);
+                tc_mma(d_tmem, pa, pb, accum);
+                tc_mma(d_tmem, pa + 2, pb + 2, 1);
+                tc_mma(d_tmem, pa + 4, pb + 4, 1);
+                tc_mma(d_tmem, pa + 6, pb + 6, 1);
+                tc_commit(&empty_a[sa]);
+                if (++sa == TC_A) {
+                    sa = 0;
+                    ra++;
+                }
+                return true;
+            };
+            while (ok && !s_abort && tr.next(a)) {
+                const uint32_t KB = tr.A.KB;
+                const bool resident = KB <= (uint32_t)TC_B;
+                const uint32_t b0 = sb;  // the run's first pair
+                for (uint32_t i = 0; i < tr.n && ok; i++, it++) {
+                    const uint32_t buf = it & 1;
+                    if (!mbar_wait(&acc_empty[buf], ((it >> 1) & 1) ^ 1, &s_abort, a.err)) {
                         ok = false;
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t sa = sbase + stage * TC_STAGE, sb = sa + TC_BLOCK;
-#pragma unroll
-                    for (int k = 0; k < 4; k++)
-                        tc_mma(d_tmem, sw128_desc(sa + 32 * k), sw128_desc(sb + 32 * k),
-                               (kb | k) != 0 ? 1u : 0u);
-                    tc_commit(&empty[stage]);
-                    if (++stage == TC_STAGES) {
-                        stage = 0;
-                        round++;
+                    uint32_t pair = b0;
+                    for (uint32_t kb = 0; kb < KB && ok; kb++) {
+                        if (!resident || i == 0) {
+                            pair = sb;
+                            if (!mbar_wait(&full_b[sb], rb & 1, &s_abort, a.err)) {
+                                ok = false;
+                                break;
+                            }
+                            if (++sb == TC_B) {
+                                sb = 0;
+                                rb++;
+                            }
+                        }
+                        ok = step(tmem + buf * 256, pair, kb != 0 ? 1u : 0u);
+                        if (!resident) tc_commit(&empty_b[pair]);
+                        if (++pair == TC_B) pair = 0;
+                    }
+                    if (ok) tc_commit(&acc_full[buf]);
+                }
+                if (resident && ok) {
+                    // the run's pairs are free once its MMAs are done
+                    uint32_t pair = b0;
+                    for (uint32_t k = 0; k < KB; k++) {
+                        tc_commit(&empty_b[pair]);
+                        if (++pair == TC_B) pair = 0;
                     }
                 }
-                if (!ok) break;
-                tc_commit(&acc_full[buf]);
             }
             // every MMA this thread issued has completed before TMEM is freed
             tc_commit(&mma_done);
@@ -443,17 +640,24 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tcpairs(TcArgs a) {
         }
         __syncwarp();
     } else {
-        // ---- epilogue: warps 2..9; warp w reads TMEM lanes 32 * (w % 4) ..
-        // (the rows of its lane group) and columns 128 * half .. + 128
-        const uint32_t g = (uint32_t)(warp & 3), half = (uint32_t)(warp - 2) >> 2;
+        // ---- epilogue: warp w reads TMEM lanes 32 * (w % 4) .. (the rows of
+        // its lane group) and 64 of the columns
+        const uint32_t g = (uint32_t)(warp & 3);
+        const uint32_t col0 = 64u * ((uint32_t)(warp - 2) >> 2);
         uint32_t it = 0;
-        TileCursor tr;
+        RunCursor tr(a);
         // the warp's sum over its tiles of one anchor, added to the totals
         // when the anchor changes (one set of atomics per anchor, not per tile)
         U128 sum;
-        int sum_ai = -1;
+        unsigned long long fsum = 0;  // the packed sums' L! binom(x, L)
+        constexpr unsigned long long LFACT = L == 2 ? 2 : L == 3 ? 6 : 24;
+        bool any = false, ok = true;
         uint32_t sum_r = 0;
         auto flush = [&]() {
+            if constexpr (EPI != EPI_TABLE) {
+                sum.add(fsum / LFACT);
+                fsum = 0;
+            }
             const U128 ws = warp_sum_u128(sum, a.err);
             if (lane == 0 && (ws.lo | ws.hi)) {
                 atomic_add_u128(a.total, ws.lo, ws.hi, a.per_graph ? nullptr : a.err);
@@ -474,87 +678,100 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tcpairs(TcArgs a) {
             if (x <= a.big64) sum.add(binom_u64c<L>(x));
             else if (sum.add(tc_binom_big(x, L, a.err))) atomicOr(a.err, kErrOverflow);
         };
-        for (; tr.next(a); it++) {
-            const uint32_t buf = it & 1;
-            if (tr.ai != sum_ai) {
-                if (sum_ai >= 0) flush();
-                sum_ai = tr.ai;
-                sum_r = tr.A.r;
-            }
-            bool ok = true;
-            if (lane == 0) ok = mbar_wait(&acc_full[buf], (it >> 1) & 1, &s_abort, a.err);
-            ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t row = tr.I * 128 + g * 32 + lane;  // row of G
-            // columns of this tile (0..255) after the row: all of them off the
-            // diagonal, from c0 on it
-            const uint32_t c0 = row + 1 > tr.J * 256 ? row + 1 - tr.J * 256 : 0u;
-            const uint32_t cl0 = __shfl_sync(0xffffffffu, c0, 0);  // smallest in the warp
-            // entries are at most the longest row
-            const bool fast = tr.A.longest <= FAST;
-            for (uint32_t cb = half * 128; cb < half * 128 + 128; cb += 32) {
-                if (cb + 32 <= cl0) continue;  // no lane keeps a column here (warp-uniform)
-                uint32_t v[32];
-                tmem_ld32(tmem + ((g * 32) << 16) + buf * 256 + cb, v);
-                if (fast && cb >= c0) {
-                    // The float bits of entry + 2^23 are 0x4B000000 + entry;
-                    // the table's address is offset by that constant (32-bit
-                    // shared-window arithmetic), and the bits are clamped to
-                    // the table's end.
-                    const uint32_t tb = smem_u32(s_bt32) - (0x4B000000u << 2);
-                    uint32_t part32 = 0;
+        // 32 columns from column cb; kept: the columns >= c0 (per lane)
+        auto chunk = [&](const uint32_t (&v)[32], uint32_t cb, uint32_t c0, bool fast) {
+            const bool whole = cb >= c0;
+            if constexpr (EPI != EPI_TABLE) {
+                constexpr bool INT = EPI == EPI_INT;
+                if (__all_sync(0xffffffffu, whole)) fsum += poly_sum<(L <= 4 ? L : 4), INT, false>(v, 0);
+                else fsum += poly_sum<(L <= 4 ? L : 4), INT, true>(v, (int)c0 - (int)cb);
+            } else if (fast) {
+                // The float bits of entry + 2^23 units are TC_BASE + entry; the
+                // table's address is offset by that constant (32-bit
+                // shared-window arithmetic), and the bits are clamped to the
+                // table's end. Dropped columns read entry 0.
+                const uint32_t tb = smem_u32(s_bt32) - (TC_BASE << 2);
+                uint32_t part32 = 0;
 #pragma unroll
-                    for (int j = 0; j < 32; j++) {
-                        const uint32_t bits =
-                            min(__float_as_uint(__uint_as_float(v[j]) + 8388608.0f), 0x4B000000u + FAST);
-                        uint32_t b;
-                        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(b) : "r"(tb + (bits << 2)));
-                        part32 += b;
-                    }
-                    sum.add((unsigned long long)part32);
-                    continue;
+                for (int j = 0; j < 32; j++) {
+                    const uint32_t x = whole || cb + j >= c0 ? v[j] : 0u;
+                    const uint32_t bits =
+                        min(__float_as_uint(__uint_as_float(x) + 8388608.0f * TC_UNIT), TC_BASE + FAST);
+                    uint32_t b;
+                    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(b) : "r"(tb + (bits << 2)));
+                    part32 += b;
                 }
+                sum.add((unsigned long long)part32);
+            } else {
                 unsigned long long part = 0;  // < 32 * binom(256, 8) < 2^64
                 uint32_t mx = 0;
-                if (cb >= c0) {
 #pragma unroll
-                    for (int j = 0; j < 32; j++) {
-                        // the entry is an exact integer below 2^23: adding 2^23
-                        // leaves it in the low mantissa bits
-                        const uint32_t x =
-                            __float_as_uint(__uint_as_float(v[j]) + 8388608.0f) & 0x7FFFFFu;
-                        mx = max(mx, x);
-                        part += s_bt[min(x, (uint32_t)TC_BINOM + 1)];
-                    }
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 32; j++) {
-                        uint32_t x = __float_as_uint(__uint_as_float(v[j]) + 8388608.0f) & 0x7FFFFFu;
-                        x = cb + j >= c0 ? x : 0u;
-                        mx = max(mx, x);
-                        part += s_bt[min(x, (uint32_t)TC_BINOM + 1)];
-                    }
+                for (int j = 0; j < 32; j++) {
+                    // the entry is an exact integer below 2^23 units: adding
+                    // 2^23 of them leaves it in the low mantissa bits
+                    uint32_t x = __float_as_uint(__uint_as_float(v[j]) + 8388608.0f * TC_UNIT) & 0x7FFFFFu;
+                    x = cb + j >= c0 ? x : 0u;
+                    mx = max(mx, x);
+                    part += s_bt[min(x, (uint32_t)TC_BINOM + 1)];
                 }
                 sum.add(part);
                 if (mx > (uint32_t)TC_BINOM) {
 #pragma unroll
                     for (int j = 0; j < 32; j++) {
                         const uint32_t x =
-                            __float_as_uint(__uint_as_float(v[j]) + 8388608.0f) & 0x7FFFFFu;
+                            __float_as_uint(__uint_as_float(v[j]) + 8388608.0f * TC_UNIT) & 0x7FFFFFu;
                         if (x > (uint32_t)TC_BINOM && cb + j >= c0) add_big(x);
                     }
                 }
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&acc_empty[buf]);
+        };
+        while (ok && tr.next(a)) {
+            if (!any || tr.A.r != sum_r) {
+                if (any) flush();
+                any = true;
+                sum_r = tr.A.r;
+            }
+            const bool fast = tr.A.longest <= FAST;
+            for (uint32_t i = 0; i < tr.n; i++, it++) {
+                const uint32_t buf = it & 1;
+                if (lane == 0) ok = mbar_wait(&acc_full[buf], (it >> 1) & 1, &s_abort, a.err);
+                ok = __shfl_sync(0xffffffffu, ok ? 1 : 0, 0) != 0;
+                if (!ok) break;
+                tc_fence_after();
+                // columns of this tile (0..255) after the row: all of them off
+                // the diagonal, from c0 on it
+                const uint32_t row = (tr.I + i) * 128 + g * 32 + lane;  // row of G
+                const uint32_t c0 = row + 1 > tr.J * 256 ? row + 1 - tr.J * 256 : 0u;
+                const uint32_t cl0 = __shfl_sync(0xffffffffu, c0, 0);  // smallest in the warp
+                // 32-column chunks from the first that holds a kept column of
+                // some lane (warp-uniform)
+                const uint32_t begin = max(col0, cl0 & ~31u), end = col0 + 64;
+                const uint32_t tcol = tmem + ((g * 32) << 16) + buf * 256;
+                uint32_t v[32];
+                for (uint32_t cb = begin; cb < end; cb += 32) {
+                    tmem_ld32(tcol + cb, v);
+                    tmem_wait(v);
+                    if (cb + 32 >= end) {
+                        // the last chunk is in registers: the accumulator is
+                        // free for the next tile but one
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&acc_empty[buf]);
+                    }
+                    chunk(v, cb, c0, fast);
+                }
+                if (begin >= end) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&acc_empty[buf]);
+                }
+            }
         }
-        if (sum_ai >= 0) flush();
+        if (any) flush();
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) {
+    if (warp == 0) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                      "r"(TC_TMEM_COLS)
@@ -562,54 +779,88 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_tcpairs(TcArgs a) {
     }
 }
 
+namespace {
+
+// Epilogue of an anchor whose longest row has x positions.
+template <int L>
+constexpr int epi_of(uint32_t x) {
+    return x <= tc_poly_max<L, false>() ? EPI_FLOAT : x <= tc_poly_max<L, true>() ? EPI_INT : EPI_TABLE;
+}
+int epi_of(int l, uint32_t x) {
+    return l == 2 ? epi_of<2>(x) : l == 3 ? epi_of<3>(x) : l == 4 ? epi_of<4>(x) : (int)EPI_TABLE;
+}
+
+const void *tc_kernel(int l, int epi) {
+    switch (l) {
+        case 2: return epi == EPI_FLOAT ? (const void *)k_tcpairs<2, EPI_FLOAT>
+                     : epi == EPI_INT ? (const void *)k_tcpairs<2, EPI_INT> : (const void *)k_tcpairs<2, EPI_TABLE>;
+        case 3: return epi == EPI_FLOAT ? (const void *)k_tcpairs<3, EPI_FLOAT>
+                     : epi == EPI_INT ? (const void *)k_tcpairs<3, EPI_INT> : (const void *)k_tcpairs<3, EPI_TABLE>;
+        case 4: return epi == EPI_FLOAT ? (const void *)k_tcpairs<4, EPI_FLOAT>
+                     : epi == EPI_INT ? (const void *)k_tcpairs<4, EPI_INT> : (const void *)k_tcpairs<4, EPI_TABLE>;
+        case 5: return (const void *)k_tcpairs<5, EPI_TABLE>;
+        case 6: return (const void *)k_tcpairs<6, EPI_TABLE>;
+        case 7: return (const void *)k_tcpairs<7, EPI_TABLE>;
+        default: return (const void *)k_tcpairs<8, EPI_TABLE>;
+    }
+}
+
+}  // namespace
+
 // ------------------------------------------------------------------ host
 
-TcPlan tc_plan(const std::vector<TcInput> &in, int64_t budget_bytes) {
+TcPlan tc_plan(const std::vector<TcInput> &in, int l, int64_t budget_bytes) {
     TcPlan plan;
     std::vector<TcInput> v(in);
-    // heaviest per-tile work first, so that the strided tile assignment of
-    // the persistent kernel ends with short tiles
-    std::sort(v.begin(), v.end(), [](const TcInput &x, const TcInput &y) {
-        return x.W != y.W ? x.W > y.W : x.nr > y.nr;
+    // one epilogue per chunk; in it the heaviest per-tile work first, so that
+    // the strided job assignment of the persistent kernel ends with short tiles
+    std::sort(v.begin(), v.end(), [l](const TcInput &x, const TcInput &y) {
+        const int ex = epi_of(l, x.longest), ey = epi_of(l, y.longest);
+        return ex != ey ? ex > ey : x.W != y.W ? x.W > y.W : x.nr > y.nr;
     });
     TcChunk cur;
-    int64_t blocks = 0, tiles = 0;
     auto flush = [&]() {
         if (cur.host.empty()) return;
-        cur.n_blocks = blocks;
-        cur.n_tiles = tiles;
-        // 16 tiles amortise a job's start; fewer when the chunk could not give
+        // up to 64 tiles amortise a job's start; fewer when that would not give
         // every SM several jobs
-        cur.job_tiles = (int)std::max<int64_t>(1, std::min<int64_t>(16, tiles / (152 * 8)));
-        plan.max_blocks = std::max(plan.max_blocks, blocks);
+        cur.job_tiles = (int)std::max<int64_t>(1, std::min<int64_t>(64, cur.n_tiles / (152 * 16)));
+        for (TcAnchor &A : cur.host) {
+            A.job0 = cur.n_jobs;
+            cur.n_jobs += ((int64_t)A.tiles + cur.job_tiles - 1) / cur.job_tiles;
+        }
+        plan.max_blocks = std::max(plan.max_blocks, cur.n_blocks);
+        plan.tiles += cur.n_tiles;
         plan.chunks.push_back(std::move(cur));
         cur = TcChunk();
-        blocks = tiles = 0;
     };
     for (const TcInput &x : v) {
         TcAnchor A;
         A.r = x.r;
         A.nr = x.nr;
-        A.longest = x.longest;
-        A.pad = 0;
         A.W = x.W;
         A.rsv = x.rsv;
-        A.RB = 2 * ((x.nr + 255) / 256);
-        A.KB = (x.W + 3) / 4;
+        A.longest = x.longest;
         A.pool_off = x.pool_off;
+        const uint64_t h = (x.nr + 255) / 256;
+        A.RB = (uint32_t)(2 * h);
+        A.KB = (x.W + 3) / 4;
+        const uint64_t tiles = h * (h + 1);  // sum over columns J < h of 2J + 2
+        if (tiles > 0xFFFFFFFFull) fail(SBC_E_UNSUPPORTED, "an anchor with %u rows is too large", x.nr);
+        A.tiles = (uint32_t)tiles;
         const int64_t nb = (int64_t)A.RB * A.KB;
-        if (!cur.host.empty() && (blocks + nb) * (int64_t)TC_BLOCK > budget_bytes) flush();
-        A.zblk0 = blocks;
-        A.tile0 = tiles;
-        const uint64_t h = A.RB / 2;
-        tiles += (int64_t)(h * (h + 1));  // sum over J < RB/2 of min(2J + 2, RB)
-        plan.kblocks += h * (h + 1) * A.KB;
-        blocks += nb;
+        const int epi = epi_of(l, x.longest);
+        if (!cur.host.empty() &&
+            (epi != cur.epi || (cur.n_blocks + nb) * (int64_t)TC_BLOCK > budget_bytes)) flush();
+        cur.epi = epi;
+        A.zblk0 = cur.n_blocks;
+        A.job0 = 0;
+        cur.n_blocks += nb;
+        cur.n_tiles += (int64_t)tiles;
+        plan.kblocks += tiles * A.KB;
         cur.host.push_back(A);
         plan.anchors++;
     }
     flush();
-    for (const TcChunk &c : plan.chunks) plan.tiles += c.n_tiles;
     return plan;
 }
 
@@ -618,7 +869,11 @@ void tc_upload(TcPlan &plan, cudaStream_t s) {
         c.dev.alloc(c.host.size(), s);
         SBC_CUDA(cudaMemcpyAsync(c.dev.ptr, c.host.data(), sizeof(TcAnchor) * c.host.size(),
                                  cudaMemcpyHostToDevice, s));
-        c.job.alloc((size_t)((c.n_tiles + c.job_tiles - 1) / c.job_tiles), s);
+        c.jobs.alloc((size_t)c.n_jobs, s);
+        k_tcjobs<<<grid_for((int64_t)c.host.size(), 128), 128, 0, s>>>(c.dev.ptr, (int)c.host.size(),
+                                                                      c.job_tiles, c.jobs.ptr);
+        SBC_LAUNCHED();
+        g_launches++;
     }
 }
 
@@ -630,12 +885,10 @@ void tc_ensure_attrs() {
     SBC_CUDA(cudaGetDevice(&dev));
     if (dev < 0 || dev >= 64) fail(SBC_E_UNSUPPORTED, "device ordinal %d out of range", dev);
     if (done[dev]) return;
-    const void *fns[] = {(const void *)k_tcpairs<2>, (const void *)k_tcpairs<3>,
-                         (const void *)k_tcpairs<4>, (const void *)k_tcpairs<5>,
-                         (const void *)k_tcpairs<6>, (const void *)k_tcpairs<7>,
-                         (const void *)k_tcpairs<8>};
-    for (const void *f : fns)
-        SBC_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TC_SMEM));
+    for (int l = 2; l <= 8; l++)
+        for (int e = l <= 4 ? (int)EPI_FLOAT : (int)EPI_TABLE; e <= EPI_TABLE; e++)
+            SBC_CUDA(cudaFuncSetAttribute(tc_kernel(l, e), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)TC_SMEM));
     done[dev] = true;
 }
 
@@ -645,28 +898,17 @@ void tc_launch(const TcPlan &plan, TcArgs base, unsigned char *z, cudaStream_t s
         TcArgs a = base;
         a.anc = c.dev.ptr;
         a.n_anc = (int)c.host.size();
+        a.jobs = c.jobs.ptr;
+        a.n_jobs = c.n_jobs;
         a.n_blocks = c.n_blocks;
-        a.n_tiles = c.n_tiles;
         a.z = z;
-        a.job = c.job.ptr;
-        a.job_tiles = c.job_tiles;
-        k_tcjobs<<<grid_for(a.n_anc, 128), 128, 0, s>>>(a);
+        k_zexpand<<<(int)std::min<int64_t>(c.n_blocks, (int64_t)sms * 16), 512, 0, s>>>(a);
         SBC_LAUNCHED();
-        int ge = (int)std::min<int64_t>(c.n_blocks, (int64_t)sms * 8);
-        k_zexpand<<<ge, 512, 0, s>>>(a);
+        const int g = (int)std::min<int64_t>(c.n_jobs, (int64_t)sms);
+        void *args[] = {&a};
+        SBC_CUDA(cudaLaunchKernel(tc_kernel(a.l, c.epi), dim3(g), dim3(TC_THREADS), args, TC_SMEM, s));
         SBC_LAUNCHED();
-        int gt = (int)std::min<int64_t>((c.n_tiles + c.job_tiles - 1) / c.job_tiles, (int64_t)sms);
-        switch (a.l) {
-            case 2: k_tcpairs<2><<<gt, TC_THREADS, TC_SMEM, s>>>(a); break;
-            case 3: k_tcpairs<3><<<gt, TC_THREADS, TC_SMEM, s>>>(a); break;
-            case 4: k_tcpairs<4><<<gt, TC_THREADS, TC_SMEM, s>>>(a); break;
-            case 5: k_tcpairs<5><<<gt, TC_THREADS, TC_SMEM, s>>>(a); break;
-            case 6: k_tcpairs<6><<<gt, TC_THREADS, TC_SMEM, s>>>(a); break;
-            case 7: k_tcpairs<7><<<gt, TC_THREADS, TC_SMEM, s>>>(a); break;
-            default: k_tcpairs<8><<<gt, TC_THREADS, TC_SMEM, s>>>(a); break;
-        }
-        SBC_LAUNCHED();
-        g_launches += 3;
+        g_launches += 2;
     }
 }
 
