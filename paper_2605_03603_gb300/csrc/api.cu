@@ -170,7 +170,7 @@ sbc_status sbc_count(const sbc_graph *g, int p, int q, sbc_u128 *out, void *stre
     SBC_API_BEGIN
     if (!g || !out) fail(SBC_E_INVAL, "NULL argument");
     sbc_count_stats st;
-    count_graph(g, p, q, nullptr, &st, (cudaStream_t)stream);
+    count_graph(g, p, q, nullptr, &st, (cudaStream_t)stream, false);
     *out = st.count;
     SBC_API_END
 }
@@ -184,7 +184,7 @@ sbc_status sbc_count_csr(int64_t n_u, int64_t n_v, int64_t nnz, const void *row_
     std::unique_ptr<sbc_graph> g(
         create_graph(n_u, n_v, nnz, row_offsets, cols, signs, flags, (cudaStream_t)stream));
     sbc_count_stats st;
-    count_graph(g.get(), p, q, nullptr, &st, (cudaStream_t)stream);
+    count_graph(g.get(), p, q, nullptr, &st, (cudaStream_t)stream, false);
     *out = st.count;
     SBC_API_END
 }

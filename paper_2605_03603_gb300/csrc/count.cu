@@ -51,15 +51,15 @@ struct Counters {
     unsigned long long tuples_ours[2]; // u128, sum binom(|C'|, R)
     unsigned long long candidates;     // sum |C'| (or |C_paper| in stats mode)
     unsigned long long e_max;          // largest visited-wedge count of a large anchor
+    unsigned long long words_big, words_small;  // pool words of the two 2-hop tiers
     unsigned int n_active;             // anchors with work
     unsigned int n_big;                // anchors for the CTA-wide 2-hop kernel
-    // tuple step of one anchor group: sizes, then the emit pass's cursors
-    float cost_total;                  // cost estimate of the work items
+    // tuple step of one anchor group
+    double cost_total;                 // cost estimate of the work items
     unsigned int n_items;
     unsigned int n_warp;               // anchors counted one per warp
     unsigned int n_tc;                 // anchors for the tensor-core pair step
     unsigned int n_claims;             // anchors shared by several work items
-    unsigned int e_items, e_warp, e_tc, e_claims;
     // ---- per execution
     unsigned long long run_begin;      // marker (unused)
     unsigned long long total[2];       // u128 count
@@ -180,75 +180,305 @@ __device__ __forceinline__ void binom_add(U128 &acc, unsigned x, int l, unsigned
 
 // ------------------------------------------------------------------ plan
 
-// Warp per anchor: useful positions, wedge counts, reservation, sort key.
-__global__ void k_plan(const int64_t *__restrict__ A_off, const uint32_t *__restrict__ A_ent,
-                       const uint32_t *__restrict__ A_pos, const int64_t *__restrict__ B_off,
-                       int64_t nX, int R, int l, int shard, int nshard, int stats,
-                       uint32_t *__restrict__ A_bit, uint32_t *__restrict__ dprime,
-                       unsigned long long *__restrict__ e_use, unsigned long long *__restrict__ e_all,
-                       uint32_t *__restrict__ rsv_c, int64_t *__restrict__ rsv_w,
-                       uint32_t *__restrict__ skey, uint32_t *__restrict__ sval,
-                       Counters *cnt, int small_e) {
-    const int lane = threadIdx.x & 31;
-    int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const uint32_t lt = (1u << lane) - 1u;
-    for (int64_t r = warp; r < nX; r += nwarps) {
-        int64_t e0 = A_off[r], e1 = A_off[r + 1];
+struct PlanArgs {
+    const int64_t *A_off;
+    const uint32_t *A_ent, *A_pos;
+    const int64_t *B_off;
+    int64_t nX;
+    int R, l, shard, nshard, stats, small_e;
+    uint32_t *A_bit, *dprime, *rsv_c;
+    unsigned long long *e_use, *e_all;  // e_all: with stats only
+    uint8_t *key;
+    uint32_t *hist;  // anchors per key
+    Counters *cnt;
+};
+
+// Order key of an anchor, heavy first: 0..127 for the CTA-wide 2-hop tier,
+// 128..254 for the warp tier, each by the visited wedges on a logarithmic scale
+// (four steps per octave), 255 without work. The order only balances the work,
+// so one pass over 256 keys is enough (four radix passes over 32-bit costs were
+// a third of a small count's launches).
+__device__ __forceinline__ uint32_t plan_key(unsigned long long cost, bool big) {
+    const uint32_t x = cost < 0xFFFFFFFFull ? (uint32_t)cost : 0xFFFFFFFFu;
+    const uint32_t e = 31 - __clz(x | 1u);
+    const uint32_t q = 4 * e + (e >= 2 ? (x >> (e - 2)) & 3u : 0u);  // 0..127
+    return big ? 127u - q : 128u + (q < 126u ? 126u - q : 0u);
+}
+
+// Useful positions, wedge counts, reservation and order key of every anchor.
+// Eight lanes per row up to PLAN_GROUP entries, a warp up to PLAN_WARP, else the
+// CTA (a hub's 29,000 positions on one warp were 0.9 ms of a 1 ms plan).
+constexpr int PLAN_THREADS = 256, PLAN_WARPS = PLAN_THREADS / 32, PLAN_ROWS = 4 * PLAN_WARPS;
+constexpr int64_t PLAN_GROUP = 64, PLAN_WARP = 1024;
+
+__global__ void __launch_bounds__(PLAN_THREADS) k_plan(PlanArgs a) {
+    __shared__ uint32_t s_hist[256];
+    __shared__ uint32_t s_cnt[2][4 * PLAN_WARPS];
+    __shared__ unsigned long long s_sum[4][PLAN_WARPS];
+    __shared__ unsigned s_act[2];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    s_hist[tid] = 0;
+    if (tid < 2) s_act[tid] = 0;
+    __syncthreads();
+    unsigned long long words_big = 0, words_small = 0, e_max = 0;
+    unsigned n_act = 0, n_big = 0;
+    // a row's results (one thread)
+    auto finish = [&](int64_t r, int64_t d, uint32_t dp, unsigned long long eu, unsigned long long ea) {
+        const bool mine = a.nshard <= 1 || (r % a.nshard) == a.shard;
+        const unsigned long long least = (unsigned long long)a.R * a.l;
+        const bool active = mine && (a.stats ? d >= a.l && ea >= least : dp >= (uint32_t)a.l && eu >= least);
+        // rows (candidate parts with >= l positions) the masks need room for;
+        // one partner needs none (its 2-hop counters are enough)
+        unsigned long long rc = 0;
+        if (active && a.R > 1) {
+            rc = eu / (unsigned long long)a.l;  // each row owns >= l useful wedges
+            const unsigned long long above = 2 * (unsigned long long)(a.nX - 1 - r);
+            rc = rc < above ? rc : above;
+        }
+        a.dprime[r] = dp;
+        a.e_use[r] = eu;
+        if (a.stats) a.e_all[r] = ea;
+        a.rsv_c[r] = (uint32_t)rc;
+        uint32_t key = 255;
+        if (active) {
+            const unsigned long long cost = a.stats ? ea : eu, words = (dp + 31) / 32 * rc;
+            const bool big = cost > (unsigned long long)a.small_e;
+            key = plan_key(cost, big);
+            n_act++;
+            if (big) {
+                n_big++;
+                words_big += words;
+                e_max = cost > e_max ? cost : e_max;
+            } else {
+                words_small += words;
+            }
+            atomicAdd(&s_hist[key], 1u);
+        }
+        a.key[r] = (uint8_t)key;
+    };
+    auto suffix = [&](int64_t e) -> unsigned long long {
+        const uint32_t y = a.A_ent[e] & VMASK;
+        return (unsigned long long)(a.B_off[y + 1] - a.B_off[y] - (int64_t)a.A_pos[e] - 1);
+    };
+    // The rows of a step are chunks apart: the hubs, which rank next to one
+    // another, go to different CTAs (32 of them on one were 1.1 ms)
+    const int64_t chunks = (a.nX + PLAN_ROWS - 1) / PLAN_ROWS;
+    for (int64_t ch = blockIdx.x; ch < chunks; ch += gridDim.x) {
+        // four rows per warp, eight lanes each
+        const int64_t r = ch + chunks * (4 * warp + (lane >> 3));
+        int64_t e0 = 0, d = 0;
+        if (r < a.nX) {
+            e0 = a.A_off[r];
+            d = a.A_off[r + 1] - e0;
+        }
+        const bool grouped = r < a.nX && d <= PLAN_GROUP;
+        const uint32_t sub = lane & 7, sh = lane & 24;
         uint32_t dp = 0;
         unsigned long long eu = 0, ea = 0;
-        for (int64_t b = e0; b < e1; b += 32) {
-            int64_t e = b + lane;
-            bool in = e < e1;
-            unsigned long long suf = 0;
-            if (in) {
-                uint32_t y = A_ent[e] & VMASK;
-                suf = (unsigned long long)(B_off[y + 1] - B_off[y] - (int64_t)A_pos[e] - 1);
-            }
-            bool useful = in && suf >= (unsigned long long)R;
-            uint32_t bal = __ballot_sync(FULL, useful);
-            if (in) A_bit[e] = useful ? dp + __popc(bal & lt) : EMPTY;
+        const uint32_t steps = __reduce_max_sync(FULL, grouped ? (uint32_t)((d + 7) / 8) : 0u);
+        for (uint32_t t = 0; t < steps; t++) {
+            const int64_t k = 8 * (int64_t)t + sub;
+            const bool in = grouped && k < d;
+            const unsigned long long suf = in ? suffix(e0 + k) : 0ull;
+            const bool useful = in && suf >= (unsigned long long)a.R;
+            const uint32_t bal = (__ballot_sync(FULL, useful) >> sh) & 0xFFu;
+            if (in) a.A_bit[e0 + k] = useful ? dp + __popc(bal & ((1u << sub) - 1u)) : EMPTY;
             dp += __popc(bal);
             eu += useful ? suf : 0ull;
             ea += suf;
         }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
+        for (int o = 4; o > 0; o >>= 1) {
             eu += __shfl_xor_sync(FULL, eu, o);
             ea += __shfl_xor_sync(FULL, ea, o);
         }
-        if (lane == 0) {
-            bool mine = nshard <= 1 || (r % nshard) == shard;
-            int64_t d = e1 - e0;
-            bool act_count = dp >= (uint32_t)l && eu >= (unsigned long long)R * l;
-            bool act_stats = d >= l && ea >= (unsigned long long)R * l;
-            bool active = mine && (stats ? act_stats : act_count);
-            // rows (candidate parts with >= l positions) the masks need room
-            // for; one partner needs none (its 2-hop counters are enough)
-            unsigned long long rc = 0;
-            if (active && R > 1) {
-                rc = eu / (unsigned long long)l;  // each row owns >= l useful wedges
-                unsigned long long above = 2 * (unsigned long long)(nX - 1 - r);
-                rc = rc < above ? rc : above;
+        if (grouped && sub == 0) finish(r, d, dp, eu, ea);
+        // longer rows of the warp's four, one at a time
+        for (uint32_t todo = __ballot_sync(FULL, sub == 0 && r < a.nX && d > PLAN_GROUP && d <= PLAN_WARP); todo;
+             todo &= todo - 1) {
+            const int src = __ffs(todo) - 1;
+            const int64_t rr = __shfl_sync(FULL, r, src), f0 = __shfl_sync(FULL, e0, src),
+                          dd = __shfl_sync(FULL, d, src);
+            uint32_t p = 0;
+            unsigned long long su = 0, sa = 0;
+            for (int64_t k0 = 0; k0 < dd; k0 += 32) {
+                const int64_t k = k0 + lane;
+                const bool in = k < dd;
+                const unsigned long long suf = in ? suffix(f0 + k) : 0ull;
+                const bool useful = in && suf >= (unsigned long long)a.R;
+                const uint32_t bal = __ballot_sync(FULL, useful);
+                if (in) a.A_bit[f0 + k] = useful ? p + __popc(bal & ((1u << lane) - 1u)) : EMPTY;
+                p += __popc(bal);
+                su += useful ? suf : 0ull;
+                sa += suf;
             }
-            uint32_t W = (dp + 31) / 32;
-            dprime[r] = dp;
-            e_use[r] = eu;
-            e_all[r] = ea;
-            rsv_c[r] = (uint32_t)rc;
-            rsv_w[r] = (int64_t)((unsigned long long)W * rc);
-            unsigned long long cost = stats ? ea : eu;
-            skey[r] = active ? 0xFFFFFFFEu - (uint32_t)(cost < 0xFFFFFFFEull ? cost : 0xFFFFFFFEull)
-                             : 0xFFFFFFFFu;
-            sval[r] = (uint32_t)r;
-            if (active) atomicAdd(&cnt->n_active, 1u);
-            if (active && cost > (unsigned long long)small_e) {
-                atomicAdd(&cnt->n_big, 1u);
-                atomicMax(&cnt->e_max, cost);
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                su += __shfl_xor_sync(FULL, su, o);
+                sa += __shfl_xor_sync(FULL, sa, o);
             }
+            if (lane == 0) finish(rr, dd, p, su, sa);
+        }
+        // the longest rows, by the CTA, four entries per thread and step
+        if (!__syncthreads_or(sub == 0 && r < a.nX && d > PLAN_WARP)) continue;
+        for (int64_t rr = ch; rr < a.nX; rr += chunks) {
+            const int64_t f0 = a.A_off[rr], dd = a.A_off[rr + 1] - f0;
+            if (dd <= PLAN_WARP) continue;
+            uint32_t p = 0;
+            unsigned long long su = 0, sa = 0;
+            int flip = 0;
+            for (int64_t k0 = 0; k0 < dd; k0 += 4 * PLAN_THREADS, flip ^= 1) {
+                unsigned long long suf[4];
+                uint32_t bal[4];
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    const int64_t k = k0 + q * PLAN_THREADS + tid;
+                    suf[q] = k < dd ? suffix(f0 + k) : 0ull;
+                }
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    bal[q] = __ballot_sync(FULL, suf[q] >= (unsigned long long)a.R && k0 + q * PLAN_THREADS + tid < dd);
+                    if (lane == 0) s_cnt[flip][q * PLAN_WARPS + warp] = __popc(bal[q]);
+                }
+                __syncthreads();
+                // (the other half of s_cnt is written in the next step)
+                const uint32_t x = s_cnt[flip][lane];
+                uint32_t incl = x;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t t = __shfl_up_sync(FULL, incl, o);
+                    if (lane >= o) incl += t;
+                }
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    const uint32_t pre = __shfl_sync(FULL, incl - x, q * PLAN_WARPS + warp);
+                    const int64_t k = k0 + q * PLAN_THREADS + tid;
+                    if (k < dd) {
+                        const bool useful = (bal[q] >> lane) & 1u;
+                        a.A_bit[f0 + k] = useful ? p + pre + __popc(bal[q] & ((1u << lane) - 1u)) : EMPTY;
+                        su += useful ? suf[q] : 0ull;
+                        sa += suf[q];
+                    }
+                }
+                p += __shfl_sync(FULL, incl, 31);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                su += __shfl_xor_sync(FULL, su, o);
+                sa += __shfl_xor_sync(FULL, sa, o);
+            }
+            __syncthreads();
+            if (lane == 0) {
+                s_sum[0][warp] = su;
+                s_sum[1][warp] = sa;
+            }
+            __syncthreads();
+            if (tid == 0) {
+                su = sa = 0;
+                for (int w = 0; w < PLAN_WARPS; w++) {
+                    su += s_sum[0][w];
+                    sa += s_sum[1][w];
+                }
+                finish(rr, dd, p, su, sa);
+            }
+            __syncthreads();
         }
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) rsv_w[nX] = 0;
+    // the CTA's totals
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        words_big += __shfl_xor_sync(FULL, words_big, o);
+        words_small += __shfl_xor_sync(FULL, words_small, o);
+        const unsigned long long t = __shfl_xor_sync(FULL, e_max, o);
+        e_max = t > e_max ? t : e_max;
+    }
+    n_act = __reduce_add_sync(FULL, n_act);
+    n_big = __reduce_add_sync(FULL, n_big);
+    __syncthreads();
+    if (lane == 0) {
+        s_sum[0][warp] = words_big;
+        s_sum[1][warp] = words_small;
+        s_sum[2][warp] = e_max;
+        if (n_act) atomicAdd(&s_act[0], n_act);
+        if (n_big) atomicAdd(&s_act[1], n_big);
+    }
+    __syncthreads();
+    if (s_hist[tid]) atomicAdd(&a.hist[tid], s_hist[tid]);
+    if (tid == 0 && s_act[0]) {
+        for (int w = 1; w < PLAN_WARPS; w++) {
+            words_big += s_sum[0][w];
+            words_small += s_sum[1][w];
+            e_max = s_sum[2][w] > e_max ? s_sum[2][w] : e_max;
+        }
+        atomicAdd(&a.cnt->n_active, s_act[0]);
+        if (words_small) atomicAdd(&a.cnt->words_small, words_small);
+        if (s_act[1]) {
+            atomicAdd(&a.cnt->n_big, s_act[1]);
+            atomicAdd(&a.cnt->words_big, words_big);
+            atomicMax(&a.cnt->e_max, e_max);
+        }
+    }
+}
+
+// Order of the active anchors by key (in any order within one), and their pool
+// offsets when all fit one group: the CTA-wide tier's regions first, then the
+// warp tier's. cursor: anchors placed per key, then the words placed per tier.
+__global__ void __launch_bounds__(256) k_order(const uint8_t *__restrict__ key, int64_t nX,
+                                               const uint32_t *__restrict__ hist,
+                                               const uint32_t *__restrict__ dprime,
+                                               const uint32_t *__restrict__ rsv_c, uint32_t *cursor,
+                                               unsigned long long *word_cursor, const Counters *cnt,
+                                               uint32_t *order, int64_t *pool_off) {
+    __shared__ uint32_t s_base[256], s_tot[8];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    {
+        const uint32_t x = tid < 255 ? hist[tid] : 0u;
+        uint32_t incl = x;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(FULL, incl, o);
+            if (lane >= o) incl += t;
+        }
+        if (lane == 31) s_tot[warp] = incl;
+        __syncthreads();
+        uint32_t pre = 0;
+        for (int w = 0; w < warp; w++) pre += s_tot[w];
+        s_base[tid] = pre + incl - x;
+        __syncthreads();
+    }
+    const unsigned long long small0 = cnt->words_big;
+    const uint32_t lt = (1u << lane) - 1u;
+    for (int64_t r0 = blockIdx.x * 256ll; r0 < nX; r0 += gridDim.x * 256ll) {
+        const int64_t r = r0 + tid;
+        const uint32_t k = r < nX ? key[r] : 255u;
+        const bool on = k != 255u;
+        const uint32_t peers = __match_any_sync(FULL, k);
+        uint32_t at = 0;
+        if (on && (peers & lt) == 0) at = s_base[k] + atomicAdd(&cursor[k], (uint32_t)__popc(peers));
+        at = __shfl_sync(FULL, at, __ffs(peers) - 1);
+        if (on) order[at + __popc(peers & lt)] = (uint32_t)r;
+        // pool words of the warp's anchors of each tier
+        const bool big = k < 128u;
+        const unsigned long long words = on ? (unsigned long long)((dprime[r] + 31) / 32) * rsv_c[r] : 0ull;
+        unsigned long long wb = big ? words : 0ull, ws = big ? 0ull : words;
+        const unsigned long long mb = wb, ms = ws;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long t = __shfl_up_sync(FULL, wb, o), u = __shfl_up_sync(FULL, ws, o);
+            if (lane >= o) {
+                wb += t;
+                ws += u;
+            }
+        }
+        unsigned long long ob = 0, os = 0;
+        if (lane == 31) {
+            if (wb) ob = atomicAdd(&word_cursor[0], wb);
+            if (ws) os = atomicAdd(&word_cursor[1], ws);
+        }
+        ob = __shfl_sync(FULL, ob, 31);
+        os = __shfl_sync(FULL, os, 31);
+        if (on) pool_off[r] = (int64_t)(big ? ob + wb - mb : small0 + os + ws - ms);
+    }
 }
 
 // ------------------------------------------------------------------ 2-hop
@@ -1045,6 +1275,7 @@ __global__ void __launch_bounds__(PL_THREADS, 2) k_twohop_large(TwohopArgs a) {
     __shared__ unsigned long long s_total;
     __shared__ unsigned s_item, s_ncw, s_nrw, s_paper, s_ovf;
     __shared__ float s_pops;
+    __shared__ uint32_t s_range;
     __shared__ unsigned s_longest;
     __shared__ uint32_t s_bcnt[PL_MAXCLS];
     const int tid = threadIdx.x, lane = tid & 31;
@@ -1186,7 +1417,21 @@ __global__ void __launch_bounds__(PL_THREADS, 2) k_twohop_large(TwohopArgs a) {
         const int lgb = bucket_lg(e_vis);
         bool bucketed = false, direct = false;
         if constexpr (!STATS) {
-            const uint32_t range = a.n_ranks - 1 - r;
+            // ranks above the anchor's (in a batch: of its own graph)
+            if (tid == 0) {
+                uint32_t end = a.n_ranks;
+                if (a.tot.per_graph) {
+                    int lo = 0, hi = a.tot.n_graphs;
+                    while (hi - lo > 1) {
+                        const int mid = (lo + hi) >> 1;
+                        if (a.tot.graph_x0[mid] <= (int64_t)r) lo = mid; else hi = mid;
+                    }
+                    end = (uint32_t)a.tot.graph_x0[lo + 1];
+                }
+                s_range = end - 1 - r;
+            }
+            __syncthreads();
+            const uint32_t range = s_range;
             direct = a.direct && direct_takes(e_use, a.dprime[r], range);
             if (direct) {
                 DirectOut o = a.dprime[r] <= 255u
@@ -1419,12 +1664,12 @@ __global__ void __launch_bounds__(PL_THREADS, 2) k_twohop_large(TwohopArgs a) {
 
 // ------------------------------------------------------------------ groups
 
-// Candidate-mask words of the sorted anchors: gw[i] = words of order[i].
-__global__ void k_gather_words(const uint32_t *order, const int64_t *words_by_rank, int64_t n,
-                               int64_t *gw) {
+// Pool words of the ordered anchors: gw[i] = words of order[i].
+__global__ void k_gather_words(const uint32_t *order, const uint32_t *dprime, const uint32_t *rsv_c,
+                               int64_t n, int64_t *gw) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i <= n;
          i += (int64_t)gridDim.x * blockDim.x)
-        gw[i] = i < n ? words_by_rank[order[i]] : 0;
+        gw[i] = i < n ? (int64_t)((dprime[order[i]] + 31) / 32) * rsv_c[order[i]] : 0;
 }
 
 // Pool offsets of one group of sorted anchors [a, b): offset from cum[a].
@@ -1563,13 +1808,17 @@ struct CountRun {
     int R = 0;
     cudaStream_t s = nullptr;
     DevBuf<Counters> cnt;
-    DevBuf<uint32_t> A_bit, dprime, rsv_c, skey, sval, tk, tv, ncand, npaper, nrow, pool,
-        claims, scratch, warp_list;
-    DevBuf<RowInfo> rinfo;
-    DevBuf<unsigned long long> e_use, e_all, bucket, per;
-    DevBuf<int64_t> pool_off, cum_dev;
+    DevBuf<unsigned char> ws;       // per-anchor and per-entry arrays, one allocation
+    uint32_t *A_bit = nullptr, *dprime = nullptr, *rsv_c = nullptr, *order = nullptr, *ncand = nullptr,
+             *nrow = nullptr, *npaper = nullptr;
+    unsigned long long *e_use = nullptr, *e_all = nullptr;
+    int64_t *pool_off = nullptr;
+    RowInfo *rinfo = nullptr;
+    DevBuf<uint32_t> pool, claims, scratch, warp_list;
+    DevBuf<unsigned long long> bucket, per;
+    DevBuf<int64_t> cum_dev;
     DevBuf<Item> items;
-    DevBuf<uint32_t> tc_list;
+    DevBuf<TcInput> tc_in;
     DevBuf<unsigned char> zbuf;     // Z arena of the tensor-core pair step
     std::vector<TcPlan> tc_plans;   // per anchor group
     TwohopArgs ta;
@@ -1664,11 +1913,14 @@ struct CountRun {
     // The warp tier of the 2-hop step builds its rows with atomicOr into words
     // that are zero on entry; the CTA tier clears or writes every word it uses.
     void zero_pool(size_t grp) {
-        const int64_t a = groups[grp].first, b = groups[grp].second;
-        const int64_t from = std::min(std::max<int64_t>(a, hc.n_big), b);
-        const int64_t words = cum[b] - cum[from];
-        if (words > 0)
-            SBC_CUDA(cudaMemsetAsync(pool.ptr + (cum[from] - cum[a]), 0, (size_t)words * 4, s));
+        int64_t from = words_big, words = words_small;
+        if (!cum.empty()) {
+            const int64_t a = groups[grp].first, b = groups[grp].second;
+            const int64_t f = std::min(std::max<int64_t>(a, hc.n_big), b);
+            from = cum[f] - cum[a];
+            words = cum[b] - cum[f];
+        }
+        if (words > 0) SBC_CUDA(cudaMemsetAsync(pool.ptr + from, 0, (size_t)words * 4, s));
     }
 
     void launch_twohop(unsigned a, unsigned b) {
@@ -1708,7 +1960,8 @@ struct CountRun {
     }
 
     std::vector<std::pair<int64_t, int64_t>> groups;  // ranges of the sorted anchors
-    std::vector<int64_t> cum;  // pool words before each sorted anchor
+    int64_t words_big = 0, words_small = 0;  // pool words of the two 2-hop tiers
+    std::vector<int64_t> cum;  // several groups: pool words before each ordered anchor
     float tw_tail_ms = 0;      // largest finish spread of the CTA-wide 2-hop kernel's CTAs
 
     // Finish spread of the CTA-wide 2-hop launch of the last group (counters in hc).
@@ -1718,20 +1971,9 @@ struct CountRun {
     float ms_twohop = 0, ms_tuples = 0, ms_tc = 0;
     std::vector<cudaEvent_t> ev_tc;
 
-    // Plan (with host reads of sizes) and execute once. Anchors are taken in
-    // heavy-first order in groups whose candidate masks fit the pool budget;
-    // each group runs its 2-hop kernels, item planning and tuple kernel.
-    // Tensor-core plan of group `grp` from the n anchors k_anchor_cost listed.
-    void plan_tc(size_t grp, unsigned n) {
-        DevBuf<TcInput> tin(n, s);
-        k_tc_gather<<<grid_for(n, 256), 256, 0, s>>>(tc_list.ptr, n, nrow.ptr, rinfo.ptr, dprime.ptr,
-                                                    rsv_c.ptr, pool_off.ptr, tin.ptr);
-        SBC_LAUNCHED();
-        g_launches++;
-        std::vector<TcInput> h(n);
-        SBC_CUDA(cudaMemcpyAsync(h.data(), tin.ptr, sizeof(TcInput) * n, cudaMemcpyDeviceToHost, s));
-        SBC_CUDA(cudaStreamSynchronize(s));
-        TcPlan plan = tc_plan(h, spec.l, tc_budget_bytes());
+    // Tensor-core plan of group `grp`.
+    void plan_tc(size_t grp, const std::vector<TcInput> &in) {
+        TcPlan plan = tc_plan(in, spec.l, tc_budget_bytes());
         tc_upload(plan, s);
         const size_t need = (size_t)plan.max_blocks * (size_t)kTcBlockBytes;
         if (need > zbuf.bytes()) zbuf.alloc(need, s);
@@ -1752,6 +1994,9 @@ struct CountRun {
     }
     uint64_t tc_anchors = 0, tc_tiles = 0, tc_kblocks = 0;
 
+    // Plan (with host reads of sizes) and execute once. Anchors are taken in
+    // heavy-first order in groups whose rows fit the pool budget; each group runs
+    // its 2-hop kernels, item planning, tuple kernel and tensor-core step.
     void plan_and_run(EventTimer *tm) {
         NvtxRange nr("sbc/count");
         const bool timing = tm != nullptr;
@@ -1763,50 +2008,87 @@ struct CountRun {
         gt = 0;
         const int l = spec.l;
         R = spec.k - 1;
+        // one allocation for the arrays, its head zeroed: counters' histogram
+        // and cursors, ncand, nrow, npaper
         cnt.alloc(1, s);
         SBC_CUDA(cudaMemsetAsync(cnt.ptr, 0, sizeof(Counters), s));
-        A_bit.alloc(nnz, s);
-        dprime.alloc(nX, s);
-        rsv_c.alloc(nX, s);
-        skey.alloc(nX, s);
-        sval.alloc(nX, s);
-        tk.alloc(nX, s);
-        tv.alloc(nX, s);
-        ncand.alloc(nX, s);
-        nrow.alloc(nX, s);
-        rinfo.alloc(nX, s);
-        npaper.alloc(spec.paper ? nX : 0, s);
-        e_use.alloc(nX, s);
-        e_all.alloc(nX, s);
-        pool_off.alloc(nX + 1, s);
-        k_plan<<<grid_for(nX * 32, B), B, 0, s>>>(o->A_off.ptr, o->A_ent.ptr, o->A_pos.ptr,
-                                                  o->B_off.ptr, nX, R, l, spec.shard, spec.nshard,
-                                                  spec.paper ? 1 : 0, A_bit.ptr, dprime.ptr,
-                                                  e_use.ptr, e_all.ptr, rsv_c.ptr, pool_off.ptr,
-                                                  skey.ptr, sval.ptr, cnt.ptr,
-                                                  spec.small_e > 0 ? spec.small_e : SMALL_E_MAX);
+        size_t at = 0;
+        auto carve = [&](size_t bytes) {
+            const size_t p = at;
+            at += (bytes + 255) & ~(size_t)255;
+            return p;
+        };
+        const size_t N = (size_t)nX;
+        const size_t o_words = carve(16), o_hist = carve(1024), o_cursor = carve(1024), o_ncand = carve(4 * N),
+                     o_nrow = carve(4 * N), o_npaper = carve(spec.paper ? 4 * N : 0), zeroed = at,
+                     o_bit = carve(4 * (size_t)nnz), o_dprime = carve(4 * N), o_rsv = carve(4 * N),
+                     o_order = carve(4 * N), o_use = carve(8 * N), o_all = carve(spec.paper ? 8 * N : 0),
+                     o_off = carve(8 * N), o_info = carve(sizeof(RowInfo) * N), o_key = carve(N);
+        ws.alloc(at, s);
+        unsigned char *w = ws.ptr;
+        unsigned long long *word_cursor = (unsigned long long *)(w + o_words);
+        uint32_t *hist = (uint32_t *)(w + o_hist), *cursor = (uint32_t *)(w + o_cursor);
+        ncand = (uint32_t *)(w + o_ncand);
+        nrow = (uint32_t *)(w + o_nrow);
+        npaper = spec.paper ? (uint32_t *)(w + o_npaper) : nullptr;
+        A_bit = (uint32_t *)(w + o_bit);
+        dprime = (uint32_t *)(w + o_dprime);
+        rsv_c = (uint32_t *)(w + o_rsv);
+        order = (uint32_t *)(w + o_order);
+        e_use = (unsigned long long *)(w + o_use);
+        e_all = spec.paper ? (unsigned long long *)(w + o_all) : nullptr;
+        pool_off = (int64_t *)(w + o_off);
+        rinfo = (RowInfo *)(w + o_info);
+        uint8_t *key = w + o_key;
+        SBC_CUDA(cudaMemsetAsync(w, 0, zeroed, s));
+        PlanArgs pa;
+        pa.A_off = o->A_off.ptr;
+        pa.A_ent = o->A_ent.ptr;
+        pa.A_pos = o->A_pos.ptr;
+        pa.B_off = o->B_off.ptr;
+        pa.nX = nX;
+        pa.R = R;
+        pa.l = l;
+        pa.shard = spec.shard;
+        pa.nshard = spec.nshard;
+        pa.stats = spec.paper ? 1 : 0;
+        pa.small_e = spec.small_e > 0 ? spec.small_e : SMALL_E_MAX;
+        pa.A_bit = A_bit;
+        pa.dprime = dprime;
+        pa.rsv_c = rsv_c;
+        pa.e_use = e_use;
+        pa.e_all = e_all;
+        pa.key = key;
+        pa.hist = hist;
+        pa.cnt = cnt.ptr;
+        k_plan<<<grid_for((nX + 3) / 4 * 32, PLAN_THREADS, 152 * 8), PLAN_THREADS, 0, s>>>(pa);
         SBC_LAUNCHED();
-        g_launches++;
-        radix_sort_pairs(skey.ptr, sval.ptr, tk.ptr, tv.ptr, nX, 32, s);
-        SBC_CUDA(cudaMemsetAsync(ncand.ptr, 0, (size_t)nX * 4, s));
-        SBC_CUDA(cudaMemsetAsync(nrow.ptr, 0, (size_t)nX * 4, s));
-        if (spec.paper) SBC_CUDA(cudaMemsetAsync(npaper.ptr, 0, (size_t)nX * 4, s));
+        k_order<<<grid_for(nX, 256, 152 * 8), 256, 0, s>>>(key, nX, hist, dprime, rsv_c, cursor, word_cursor,
+                                                           cnt.ptr, order, pool_off);
+        SBC_LAUNCHED();
+        g_launches += 2;
         SBC_CUDA(cudaMemcpyAsync(&hc, cnt.ptr, sizeof(Counters), cudaMemcpyDeviceToHost, s));
         SBC_CUDA(cudaStreamSynchronize(s));
         const int64_t n_act = hc.n_active;
-        // candidate-mask words in heavy-first order, prefix sums, groups
-        cum.assign(n_act + 1, 0);
-        {
+        words_big = (int64_t)hc.words_big;
+        words_small = (int64_t)hc.words_small;
+        cum.clear();
+        const int64_t budget = pool_budget_words();
+        int64_t most = words_big + words_small;
+        if (n_act > 0 && most <= budget) {
+            groups.emplace_back(0, n_act);
+        } else if (n_act > 0) {
+            // pool words in heavy-first order, prefix sums, groups
+            cum.assign(n_act + 1, 0);
             DevBuf<int64_t> dcum(n_act + 1, s);
-            k_gather_words<<<grid_for(n_act + 1, B), B, 0, s>>>(sval.ptr, pool_off.ptr, n_act, dcum.ptr);
+            k_gather_words<<<grid_for(n_act + 1, B), B, 0, s>>>(order, dprime, rsv_c, n_act, dcum.ptr);
             SBC_LAUNCHED();
             g_launches++;
             scan_exclusive_i64(dcum.ptr, dcum.ptr, n_act + 1, nullptr, s);
             SBC_CUDA(cudaMemcpyAsync(cum.data(), dcum.ptr, 8 * (size_t)(n_act + 1),
                                      cudaMemcpyDeviceToHost, s));
             SBC_CUDA(cudaStreamSynchronize(s));
-            const int64_t budget = pool_budget_words();
-            int64_t most = 1;
+            most = 1;
             for (int64_t a = 0; a < n_act;) {
                 int64_t b = std::upper_bound(cum.begin() + a + 1, cum.end(), cum[a] + budget) -
                             cum.begin() - 1;
@@ -1816,27 +2098,27 @@ struct CountRun {
                 a = b;
             }
             cum_dev = std::move(dcum);
-            pool.alloc((size_t)most, s);
         }
+        pool.alloc((size_t)std::max<int64_t>(most, 1), s);
         const int sms = sm_count();
 
         ta.A_off = o->A_off.ptr;
         ta.A_ent = o->A_ent.ptr;
         ta.A_pos = o->A_pos.ptr;
-        ta.A_bit = A_bit.ptr;
+        ta.A_bit = A_bit;
         ta.B_off = o->B_off.ptr;
         ta.B_ent = o->B_ent.ptr;
-        ta.dprime = dprime.ptr;
-        ta.e_use = e_use.ptr;
-        ta.e_all = e_all.ptr;
-        ta.rsv_c = rsv_c.ptr;
-        ta.pool_off = pool_off.ptr;
-        ta.order = sval.ptr;
+        ta.dprime = dprime;
+        ta.e_use = e_use;
+        ta.e_all = e_all;
+        ta.rsv_c = rsv_c;
+        ta.pool_off = pool_off;
+        ta.order = order;
         ta.pool = pool.ptr;
-        ta.ncand = ncand.ptr;
-        ta.npaper = spec.paper ? npaper.ptr : nullptr;
-        ta.nrow = nrow.ptr;
-        ta.rinfo = rinfo.ptr;
+        ta.ncand = ncand;
+        ta.npaper = npaper;
+        ta.nrow = nrow;
+        ta.rinfo = rinfo;
         ta.single = R == 1;
         ta.n_ranks = (uint32_t)nX;
         ta.direct = hash_slots_cap() == 0 && twohop_window_wedges() == (uint32_t)PL_WCAP;
@@ -1878,10 +2160,10 @@ struct CountRun {
         tot.n_graphs = spec.n_graphs;
         tot.err = &cnt.ptr->err;
         ta.tot = tot;
-        tu.nrow = nrow.ptr;
-        tu.dprime = dprime.ptr;
-        tu.rsv_c = rsv_c.ptr;
-        tu.pool_off = pool_off.ptr;
+        tu.nrow = nrow;
+        tu.dprime = dprime;
+        tu.rsv_c = rsv_c;
+        tu.pool_off = pool_off;
         tu.pool = pool.ptr;
         tu.cnt = cnt.ptr;
         tu.tot = tot;
@@ -1890,12 +2172,14 @@ struct CountRun {
         tu.l = l;
 
         ItemArgs ia;
-        ia.ncand = ncand.ptr;
-        ia.npaper = spec.paper ? npaper.ptr : nullptr;
-        ia.nrow = nrow.ptr;
-        ia.dprime = dprime.ptr;
-        ia.rinfo = rinfo.ptr;
-        ia.order = sval.ptr;
+        ia.ncand = ncand;
+        ia.npaper = npaper;
+        ia.nrow = nrow;
+        ia.dprime = dprime;
+        ia.rsv_c = rsv_c;
+        ia.pool_off = pool_off;
+        ia.rinfo = rinfo;
+        ia.order = order;
         ia.R = R;
         ia.l = l;
         ia.method = spec.method;
@@ -1912,13 +2196,16 @@ struct CountRun {
         n_items = 0;
         for (size_t gi = 0; gi < groups.size(); gi++) {
             const int64_t a = groups[gi].first, b = groups[gi].second, na = b - a;
-            // this group's pool offsets and fresh queue heads
-            k_group_offsets<<<grid_for(na, B), B, 0, s>>>(sval.ptr, cum_dev.ptr, a, b, pool_off.ptr);
-            SBC_LAUNCHED();
-            g_launches++;
-            SBC_CUDA(cudaMemsetAsync(&cnt.ptr->head_large, 0, 4 * sizeof(unsigned), s));
-            SBC_CUDA(cudaMemsetAsync(&cnt.ptr->cost_total, 0, 9 * sizeof(unsigned), s));
-            SBC_CUDA(cudaMemsetAsync(&cnt.ptr->tw_fin_max, 0, 2 * sizeof(unsigned long long), s));
+            if (!cum.empty()) {
+                // this group's pool offsets and fresh queue heads
+                k_group_offsets<<<grid_for(na, B), B, 0, s>>>(order, cum_dev.ptr, a, b, pool_off);
+                SBC_LAUNCHED();
+                g_launches++;
+                SBC_CUDA(cudaMemsetAsync(&cnt.ptr->head_large, 0, 4 * sizeof(unsigned), s));
+                SBC_CUDA(cudaMemsetAsync(&cnt.ptr->cost_total, 0,
+                                         offsetof(Counters, run_begin) - offsetof(Counters, cost_total), s));
+                SBC_CUDA(cudaMemsetAsync(&cnt.ptr->tw_fin_max, 0, 2 * sizeof(unsigned long long), s));
+            }
             cudaEvent_t t0 = timing ? new_event(ev_twohop) : nullptr;
             cudaEvent_t t1 = timing ? new_event(ev_twohop) : nullptr;
             zero_pool(gi);
@@ -1931,36 +2218,47 @@ struct CountRun {
             // tuple phase planning (needs the row counts)
             ia.begin = a;
             ia.nX = na;
-            ia.items = nullptr;
-            ia.warp_list = ia.tc_list = nullptr;
             k_anchor_cost<<<grid_for(na, B), B, 0, s>>>(ia);
             SBC_LAUNCHED();
             g_launches++;
             if (R == 1) continue;  // the 2-hop kernels added every sum
-            k_items<false><<<grid_for(na, B), B, 0, s>>>(ia);
-            SBC_LAUNCHED();
-            g_launches++;
-            SBC_CUDA(cudaMemcpyAsync(&hc, cnt.ptr, sizeof(Counters), cudaMemcpyDeviceToHost, s));
-            SBC_CUDA(cudaStreamSynchronize(s));
-            tw_tail_ms = std::max(tw_tail_ms, group_tail_ms());
-            if (hc.n_items == 0 && hc.n_warp == 0 && hc.n_tc == 0) continue;
-            items.alloc(hc.n_items, s);
-            warp_list.alloc(hc.n_warp, s);
-            claims.alloc(hc.n_claims, s);
-            tc_list.alloc(hc.n_tc, s);
+            // room for the most items there can be (k_items), so that nothing
+            // has to be read back first
+            const size_t split = (size_t)ia.items_per_launch + 64;
+            items.alloc((size_t)na + split, s);
+            warp_list.alloc((size_t)na, s);
+            claims.alloc(split, s);
+            tc_in.alloc(ia.tc_on ? (size_t)na : 0, s);
             ia.items = items.ptr;
             ia.warp_list = warp_list.ptr;
-            ia.tc_list = tc_list.ptr;
-            k_items<true><<<grid_for(na, B), B, 0, s>>>(ia);
+            ia.tc_in = tc_in.ptr;
+            SBC_CUDA(cudaMemsetAsync(claims.ptr, 0, claims.bytes(), s));
+            k_items<<<grid_for(na, B), B, 0, s>>>(ia);
             SBC_LAUNCHED();
             g_launches++;
+            std::vector<TcInput> tci;
+            if (ia.tc_on) {
+                // the listed anchors are planned on the host while the tuple
+                // kernel runs; the first of them come with the counters
+                tci.resize(std::min<size_t>((size_t)na, 2048));
+                SBC_CUDA(cudaMemcpyAsync(tci.data(), tc_in.ptr, sizeof(TcInput) * tci.size(),
+                                         cudaMemcpyDeviceToHost, s));
+                SBC_CUDA(cudaMemcpyAsync(&hc, cnt.ptr, sizeof(Counters), cudaMemcpyDeviceToHost, s));
+                SBC_CUDA(cudaStreamSynchronize(s));
+                const size_t have = tci.size();
+                tci.resize(hc.n_tc);
+                if (tci.size() > have) {
+                    SBC_CUDA(cudaMemcpyAsync(tci.data() + have, tc_in.ptr + have,
+                                             sizeof(TcInput) * (tci.size() - have), cudaMemcpyDeviceToHost, s));
+                    SBC_CUDA(cudaStreamSynchronize(s));
+                }
+            }
             tu.items = items.ptr;
             tu.warp_list = warp_list.ptr;
             tu.claims = claims.ptr;
-            const int64_t work = (int64_t)hc.n_items + ((int64_t)hc.n_warp + TU_WARPS - 1) / TU_WARPS;
-            gt = (int)std::min<int64_t>(gb, work);
+            gt = (int)std::min<int64_t>(gb, na);
+            if (ia.tc_on && hc.n_items == 0 && hc.n_warp == 0) gt = 0;
             if (gt > 0) {
-                if (claims.ptr) SBC_CUDA(cudaMemsetAsync(claims.ptr, 0, claims.bytes(), s));
                 cudaEvent_t t2 = timing ? new_event(ev_tuples) : nullptr;
                 cudaEvent_t t3 = timing ? new_event(ev_tuples) : nullptr;
                 if (t2) SBC_CUDA(cudaEventRecord(t2, s));
@@ -1970,9 +2268,14 @@ struct CountRun {
                 }
                 if (t3) SBC_CUDA(cudaEventRecord(t3, s));
             }
-            if (hc.n_tc > 0) plan_tc(gi, hc.n_tc);  // on the host, next to the tuple kernel
+            if (!tci.empty()) plan_tc(gi, tci);
             run_tc_timed(gi, timing);
-            n_items += hc.n_items + hc.n_warp;
+            if (!cum.empty()) {  // a further group clears the counters
+                SBC_CUDA(cudaMemcpyAsync(&hc, cnt.ptr, sizeof(Counters), cudaMemcpyDeviceToHost, s));
+                SBC_CUDA(cudaStreamSynchronize(s));
+                tw_tail_ms = std::max(tw_tail_ms, group_tail_ms());
+                n_items += hc.n_items + hc.n_warp;
+            }
         }
         if (tm) tm->mark(4, s);
         collect();
@@ -1981,10 +2284,7 @@ struct CountRun {
             ms_tuples = pairs_ms(ev_tuples);
             ms_tc = pairs_ms(ev_tc);
         }
-        // planning scratch a replay does not need
-        skey.release();
-        tk.release();
-        tv.release();
+        if (cum.empty()) res.work_items = (uint64_t)hc.n_items + hc.n_warp;
     }
 
     // Read the counters after an execution (synchronises the stream).
@@ -2007,7 +2307,7 @@ struct CountRun {
         res.anchor_tuples.hi = tt[1];
         res.candidates = hc.candidates;
         res.wedges = hc.wedges;
-        res.work_items = (uint64_t)n_items;
+        if (!cum.empty()) res.work_items = (uint64_t)n_items;
         res.tested = hc.tested;
         res.typed = hc.leaves;
         res.popc_words = hc.popc_words;
@@ -2022,7 +2322,7 @@ struct CountRun {
             res.twohop_share[i] = cyc > 0 ? (float)(hc.tw_cyc[i] / cyc) : 0.f;
         }
         res.twohop_tail_ms = std::max(tw_tail_ms, group_tail_ms());
-        res.pool_bytes = cum.empty() ? 0 : (uint64_t)cum.back() * 4;
+        res.pool_bytes = (uint64_t)(words_big + words_small) * 4;
     }
 };
 
@@ -2144,7 +2444,7 @@ unsigned long long pos_node_cost_setting() {
 }
 
 void count_graph(const sbc_graph *gc, int p, int q, const sbc_count_opts *opts,
-                 sbc_count_stats *stats, cudaStream_t s) {
+                 sbc_count_stats *stats, cudaStream_t s, bool timing) {
     sbc_graph *g = const_cast<sbc_graph *>(gc);
     if (p < 2 || q < 2 || p > 8 || q > 8) fail(SBC_E_INVAL, "p and q must be in [2, 8], got (%d, %d)", p, q);
     int cur = 0;
@@ -2175,7 +2475,7 @@ void count_graph(const sbc_graph *gc, int p, int q, const sbc_count_opts *opts,
     const int64_t nX = side == 0 ? g->n_u : g->n_v;
     if (opts && opts->per_anchor && nX > 0) memset(opts->per_anchor, 0, sizeof(sbc_u128) * (size_t)nX);
     if (g->nnz == 0 || nX == 0) return;
-    EventTimer tm(stats != nullptr && !thread_arena_active());
+    EventTimer tm(timing && stats != nullptr && !thread_arena_active());
     tm.mark(0, s);
     {
         std::lock_guard<std::mutex> lock(g->mu);

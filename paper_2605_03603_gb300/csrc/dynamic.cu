@@ -97,7 +97,7 @@ U128 local_count(const Csr &h, int p, int q, cudaStream_t s) {
     std::unique_ptr<sbc_graph> g(create_graph(h.n_l, h.n_r, (int64_t)h.col.size(), h.off.data(),
                                               h.col.data(), plus.data(), SBC_OFFS_I64, s));
     sbc_count_stats st;
-    count_graph(g.get(), p - 1, q - 1, nullptr, &st, s);
+    count_graph(g.get(), p - 1, q - 1, nullptr, &st, s, false);
     r.lo = st.count.lo;
     r.hi = st.count.hi;
     return r;
@@ -207,7 +207,7 @@ sbc_status sbc_dyn_create(sbc_dyn **out, int64_t n_u, int64_t n_v, int64_t nnz,
     std::unique_ptr<sbc_graph> g(create_graph(n_u, n_v, nnz, row_offsets, cols, signs, SBC_OFFS_I64,
                                               (cudaStream_t)stream));
     sbc_count_stats st;
-    count_graph(g.get(), p, q, nullptr, &st, (cudaStream_t)stream);
+    count_graph(g.get(), p, q, nullptr, &st, (cudaStream_t)stream, false);
     d->count.lo = st.count.lo;
     d->count.hi = st.count.hi;
     *out = d.release();

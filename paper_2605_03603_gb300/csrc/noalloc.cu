@@ -94,7 +94,7 @@ extern "C" sbc_status sbc_count_csr_noalloc(int64_t n_u, int64_t n_v, int64_t nn
         std::unique_ptr<sbc_graph> g(
             sbc::create_graph(n_u, n_v, nnz, row_offsets, cols, signs, flags, s));
         sbc_count_stats st;
-        sbc::count_graph(g.get(), p, q, nullptr, &st, s);
+        sbc::count_graph(g.get(), p, q, nullptr, &st, s, false);
         g.reset();
         *out = st.count;
     } catch (const sbc::SbcError &e) {

@@ -194,9 +194,10 @@ int preferred_side(const sbc_graph *g, int p, int q);
 sbc_graph *create_graph(int64_t n_u, int64_t n_v, int64_t nnz, const void *row_offsets,
                         const int32_t *cols, const void *signs, uint32_t flags, cudaStream_t s);
 
-// Count driver: defined in count.cu.
+// Count driver: defined in count.cu. timing: fill the stats' times (events on
+// the stream).
 void count_graph(const sbc_graph *g, int p, int q, const sbc_count_opts *opts,
-                 sbc_count_stats *stats, cudaStream_t s);
+                 sbc_count_stats *stats, cudaStream_t s, bool timing = true);
 
 // One count over an orientation (count.cu): k = tuple size on the anchor
 // side, l = size on the other side.

@@ -133,7 +133,7 @@ void lane_main(sbc_server *s, Lane *lane) {
             } else {
                 for (size_t i = 0; i < gids.size(); i++) {
                     sbc_count_stats stt;
-                    count_graph(s->graphs[gids[i]], job->p, job->q, nullptr, &stt, lane->stream);
+                    count_graph(s->graphs[gids[i]], job->p, job->q, nullptr, &stt, lane->stream, false);
                     res[i] = stt.count;
                 }
             }

@@ -80,13 +80,15 @@ struct ItemArgs {
     int method;  // 0: cheaper side per anchor, 1: rows, 2: column walk where it fits
     float pos_unit;
     float items_per_launch;  // items that the anchors' total cost is split into
-    Item *items;             // emit pass
-    uint32_t *warp_list;
+    const uint32_t *rsv_c;
+    const int64_t *pool_off;
+    Item *items;             // room for nX + items_per_launch
+    uint32_t *warp_list;     // ... nX
     Counters *cnt;
     // tensor-core pair step (two partners)
     int tc_on;
     uint32_t tc_min_w, tc_min_nc;
-    uint32_t *tc_list;
+    TcInput *tc_in;          // ... nX
 };
 
 // Costs in mask-word operations (one AND + POPC of the row side).
@@ -156,7 +158,7 @@ __device__ __forceinline__ AnchorPlan plan_anchor(const ItemArgs &a, uint32_t r)
 __global__ void k_anchor_cost(ItemArgs a) {
     U128 tp, to;
     unsigned long long cand = 0;
-    float cost = 0;
+    double cost = 0;
     for (int64_t ix = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; ix < a.nX;
          ix += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t r = a.order[a.begin + ix];
@@ -183,7 +185,7 @@ __global__ void k_anchor_cost(ItemArgs a) {
             cand += nc;
         }
         if (nc >= (uint32_t)a.R) to.add(binom_sat(nc, a.R));
-        cost += plan_anchor(a, r).cost;
+        cost += (double)plan_anchor(a, r).cost;
     }
     tp = warp_sum_u128(tp, nullptr);
     to = warp_sum_u128(to, nullptr);
@@ -200,54 +202,39 @@ __global__ void k_anchor_cost(ItemArgs a) {
     }
 }
 
-// Work items of every anchor; EMIT == false counts them. An anchor's items
-// depend on its sizes and the cost total only (a few operations per anchor:
-// how its first rows are shared among its items is settled while they run).
-template <bool EMIT>
+// Work items, warp list and tensor-core list of every anchor. An anchor's items
+// depend on its sizes and the cost total only (a few operations per anchor: how
+// its first rows are shared among its items is settled while they run). The
+// items beyond one per anchor sum to at most items_per_launch.
 __global__ void k_items(ItemArgs a) {
-    const float item_cost = fmaxf(a.cnt->cost_total / a.items_per_launch, 16384.0f);
+    const float item_cost = fmaxf((float)(a.cnt->cost_total / (double)a.items_per_launch), 16384.0f);
     for (int64_t ix = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; ix < a.nX;
          ix += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t r = a.order[a.begin + ix];
         const AnchorPlan p = plan_anchor(a, r);
         if (p.tc) {
-            const unsigned k = atomicAdd(EMIT ? &a.cnt->e_tc : &a.cnt->n_tc, 1u);
-            if (EMIT) a.tc_list[k] = r;
+            TcInput t;
+            t.r = r;
+            t.nr = a.nrow[r];
+            t.W = (a.dprime[r] + 31) / 32;
+            t.rsv = a.rsv_c[r];
+            t.longest = a.rinfo[r].longest;
+            t.pool_off = a.pool_off[r];
+            a.tc_in[atomicAdd(&a.cnt->n_tc, 1u)] = t;
         } else if (p.warp) {
-            const unsigned k = atomicAdd(EMIT ? &a.cnt->e_warp : &a.cnt->n_warp, 1u);
-            if (EMIT) a.warp_list[k] = r;
+            a.warp_list[atomicAdd(&a.cnt->n_warp, 1u)] = r;
         } else if (p.rows || p.cols) {
             const uint32_t total = (uint32_t)fminf(fmaxf(p.cost / item_cost, 1.0f), 1024.0f);
-            const unsigned k0 = atomicAdd(EMIT ? &a.cnt->e_items : &a.cnt->n_items, total);
-            unsigned claim = NO_CLAIM;
-            if (total > 1) claim = atomicAdd(EMIT ? &a.cnt->e_claims : &a.cnt->n_claims, 1u);
-            if (EMIT) {
-                for (uint32_t i = 0; i < total; i++) {
-                    Item it;
-                    it.anchor = r;
-                    it.claim = claim;
-                    it.cols = p.cols;
-                    a.items[k0 + i] = it;
-                }
+            const unsigned k0 = atomicAdd(&a.cnt->n_items, total);
+            const unsigned claim = total > 1 ? atomicAdd(&a.cnt->n_claims, 1u) : NO_CLAIM;
+            for (uint32_t i = 0; i < total; i++) {
+                Item it;
+                it.anchor = r;
+                it.claim = claim;
+                it.cols = p.cols;
+                a.items[k0 + i] = it;
             }
         }
-    }
-}
-
-// Inputs of the tensor-core plan: the listed anchors' sizes and pool offsets.
-__global__ void k_tc_gather(const uint32_t *list, unsigned n, const uint32_t *nrow,
-                            const RowInfo *rinfo, const uint32_t *dprime, const uint32_t *rsv_c, const int64_t *pool_off,
-                            TcInput *out) {
-    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const uint32_t r = list[i];
-        TcInput t;
-        t.r = r;
-        t.nr = nrow[r];
-        t.W = (dprime[r] + 31) / 32;
-        t.rsv = rsv_c[r];
-        t.longest = rinfo[r].longest;
-        t.pool_off = pool_off[r];
-        out[i] = t;
     }
 }
 
