@@ -53,7 +53,8 @@ struct Counters {
     unsigned long long e_max;          // largest visited-wedge count of a large anchor
     unsigned long long words_big, words_small;  // pool words of the two 2-hop tiers
     unsigned int n_active;             // anchors with work
-    unsigned int n_big;                // anchors for the CTA-wide 2-hop kernel
+    unsigned int n_direct;             // anchors for the direct 2-hop kernel,
+    unsigned int n_big;                // ... for it and the CTA-wide hash kernel
     // tuple step of one anchor group
     double cost_total;                 // cost estimate of the work items
     unsigned int n_items;
@@ -74,7 +75,8 @@ struct Counters {
     unsigned long long tw_anchors[4];
     unsigned long long tw_fin_max, tw_fin_min_n;  // CTA finish times (global ns; min kept as ~t)
     unsigned long long tw_split;       // hash classes hashed in sub-class windows
-    unsigned int head_large;           // 2-hop queue heads
+    unsigned int head_direct;          // 2-hop queue heads
+    unsigned int head_large;
     unsigned int head_small;
     unsigned int head_b;               // tuple queue heads: work items,
     unsigned int head_w;               // ... small anchors
@@ -178,6 +180,47 @@ __device__ __forceinline__ void binom_add(U128 &acc, unsigned x, int l, unsigned
     acc.add(v);
 }
 
+// ---- direct 2-hop counters. A partner's rank follows the anchor's, and anchors with
+// many wedges have high degrees, so high ranks: their partners' ranks span a
+// short range (on the 2M-edge graph 76 % of the wedges of anchors above 3,584
+// span at most 48k ranks). Such an anchor counts its partners in a table
+// indexed by rank - no keys, no probes, one shared-memory add without a return
+// value per wedge - in windows of consecutive ranks, each a pass over the
+// 2-hop. Counters hold the same-sign and different-sign counts of a partner in
+// 8 + 8 bits (at most 255 useful positions) or 16 + 16 bits. After a window's
+// counts, a bitmap of the parts with at least l positions and its prefix counts
+// number the rows, and the counters' memory stages the mask words of the
+// window's rows, a range of positions at a time.
+// Bound by the shared-memory atomics and the L2 gathers of B_ent. The 2-hop
+// kernels of the (3,3) count took 13.7 -> 4.9 ms on the 2M-edge graph, 74 -> 23
+// ms on a 12M-edge hub graph and 15.6 -> 1.0 ms on a dense 3000 x 800 graph
+// (hash strategies -> direct counters where the rule takes them).
+constexpr int DT_THREADS = 512;
+constexpr int DT_WARPS = DT_THREADS / 32;
+constexpr int DT_PCH = DT_THREADS;               // positions staged at once
+constexpr uint32_t DT_WORDS = 20480;            // counter words, then staged mask words
+constexpr uint32_t DT_CELLS8 = 2 * DT_WORDS;    // ranks per window with 8 + 8 bit counters
+constexpr uint32_t DT_CELLS16 = DT_WORDS;
+constexpr uint32_t DT_BM = DT_CELLS8 / 16;      // bitmap words (two bits per rank)
+constexpr size_t DT_OFF_BM = (size_t)DT_WORDS * 4;
+constexpr size_t DT_OFF_PRE = DT_OFF_BM + (size_t)DT_BM * 4;
+constexpr size_t DT_OFF_POFF = DT_OFF_PRE + (size_t)DT_BM * 4;
+constexpr size_t DT_OFF_PPRE = DT_OFF_POFF + (size_t)DT_PCH * 4;
+constexpr size_t DT_OFF_PINFO = DT_OFF_PPRE + (size_t)(DT_PCH + 4) * 4;
+constexpr size_t DT_SMEM = DT_OFF_PINFO + (size_t)DT_PCH * 4;
+
+// Direct counters or the hash strategies. Lists of at least 8 partners on
+// average (in shorter ones, of the widest hubs, few partners share all the
+// counters). Costs in SM cycles measured on the 2M-edge graph: a window about
+// 3,000 (clear, scan, barriers) and 0.7 per wedge for its two passes; the hash
+// strategies about 8 per wedge.
+__device__ __forceinline__ bool direct_takes(unsigned long long e, uint32_t dp, uint32_t range) {
+    if (dp > 65535u || e < 8ull * dp) return false;
+    const uint32_t cells = dp <= 255u ? DT_CELLS8 : DT_CELLS16;
+    const float nwin = (float)((range + cells - 1) / cells);
+    return nwin * (3000.0f + 0.7f * (float)e) < 8.0f * (float)e;
+}
+
 // ------------------------------------------------------------------ plan
 
 struct PlanArgs {
@@ -186,6 +229,9 @@ struct PlanArgs {
     const int64_t *B_off;
     int64_t nX;
     int R, l, shard, nshard, stats, small_e;
+    int direct;                // direct counters allowed (not when a test forces the hash strategies)
+    const int64_t *graph_x0;   // batches: first rank per graph (n_graphs + 1), else null
+    int n_graphs;
     uint32_t *A_bit, *dprime, *rsv_c;
     unsigned long long *e_use, *e_all;  // e_all: with stats only
     uint8_t *key;
@@ -193,16 +239,33 @@ struct PlanArgs {
     Counters *cnt;
 };
 
-// Order key of an anchor, heavy first: 0..127 for the CTA-wide 2-hop tier,
-// 128..254 for the warp tier, each by the visited wedges on a logarithmic scale
-// (four steps per octave), 255 without work. The order only balances the work,
+// One past the last rank that anchor r's partners can have: the side's, in a
+// batch its own graph's.
+__device__ __forceinline__ uint32_t rank_end(const int64_t *graph_x0, int n_graphs, uint32_t n_ranks, uint32_t r) {
+    if (!graph_x0) return n_ranks;
+    int lo = 0, hi = n_graphs;
+    while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (graph_x0[mid] <= (int64_t)r) lo = mid; else hi = mid;
+    }
+    return (uint32_t)graph_x0[lo + 1];
+}
+
+// Order key of an anchor, heavy first: 0..63 for the direct 2-hop tier, 64..127
+// for the CTA-wide hash tier (two steps per octave of visited wedges), 128..254
+// for the warp tier (four), 255 without work. The order only balances the work,
 // so one pass over 256 keys is enough (four radix passes over 32-bit costs were
 // a third of a small count's launches).
-__device__ __forceinline__ uint32_t plan_key(unsigned long long cost, bool big) {
+enum : int { TIER_DIRECT = 0, TIER_LARGE = 1, TIER_SMALL = 2 };
+__device__ __forceinline__ uint32_t plan_key(unsigned long long cost, int tier) {
     const uint32_t x = cost < 0xFFFFFFFFull ? (uint32_t)cost : 0xFFFFFFFFu;
     const uint32_t e = 31 - __clz(x | 1u);
-    const uint32_t q = 4 * e + (e >= 2 ? (x >> (e - 2)) & 3u : 0u);  // 0..127
-    return big ? 127u - q : 128u + (q < 126u ? 126u - q : 0u);
+    if (tier == TIER_SMALL) {
+        const uint32_t q = 4 * e + (e >= 2 ? (x >> (e - 2)) & 3u : 0u);
+        return 128u + (q < 126u ? 126u - q : 0u);
+    }
+    const uint32_t q = 2 * e + (e >= 1 ? (x >> (e - 1)) & 1u : 0u);  // 0..63
+    return (tier == TIER_DIRECT ? 63u : 127u) - q;
 }
 
 // Useful positions, wedge counts, reservation and order key of every anchor.
@@ -215,13 +278,13 @@ __global__ void __launch_bounds__(PLAN_THREADS) k_plan(PlanArgs a) {
     __shared__ uint32_t s_hist[256];
     __shared__ uint32_t s_cnt[2][4 * PLAN_WARPS];
     __shared__ unsigned long long s_sum[4][PLAN_WARPS];
-    __shared__ unsigned s_act[2];
+    __shared__ unsigned s_act[3];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     s_hist[tid] = 0;
-    if (tid < 2) s_act[tid] = 0;
+    if (tid < 3) s_act[tid] = 0;
     __syncthreads();
     unsigned long long words_big = 0, words_small = 0, e_max = 0;
-    unsigned n_act = 0, n_big = 0;
+    unsigned n_act = 0, n_big = 0, n_direct = 0;
     // a row's results (one thread)
     auto finish = [&](int64_t r, int64_t d, uint32_t dp, unsigned long long eu, unsigned long long ea) {
         const bool mine = a.nshard <= 1 || (r % a.nshard) == a.shard;
@@ -243,8 +306,12 @@ __global__ void __launch_bounds__(PLAN_THREADS) k_plan(PlanArgs a) {
         if (active) {
             const unsigned long long cost = a.stats ? ea : eu, words = (dp + 31) / 32 * rc;
             const bool big = cost > (unsigned long long)a.small_e;
-            key = plan_key(cost, big);
+            const bool direct = big && a.direct && !a.stats &&
+                                direct_takes(eu, dp, rank_end(a.graph_x0, a.n_graphs, (uint32_t)a.nX, (uint32_t)r) -
+                                                         1 - (uint32_t)r);
+            key = plan_key(cost, direct ? TIER_DIRECT : big ? TIER_LARGE : TIER_SMALL);
             n_act++;
+            n_direct += direct;
             if (big) {
                 n_big++;
                 words_big += words;
@@ -394,6 +461,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) k_plan(PlanArgs a) {
     }
     n_act = __reduce_add_sync(FULL, n_act);
     n_big = __reduce_add_sync(FULL, n_big);
+    n_direct = __reduce_add_sync(FULL, n_direct);
     __syncthreads();
     if (lane == 0) {
         s_sum[0][warp] = words_big;
@@ -401,6 +469,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) k_plan(PlanArgs a) {
         s_sum[2][warp] = e_max;
         if (n_act) atomicAdd(&s_act[0], n_act);
         if (n_big) atomicAdd(&s_act[1], n_big);
+        if (n_direct) atomicAdd(&s_act[2], n_direct);
     }
     __syncthreads();
     if (s_hist[tid]) atomicAdd(&a.hist[tid], s_hist[tid]);
@@ -414,6 +483,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) k_plan(PlanArgs a) {
         if (words_small) atomicAdd(&a.cnt->words_small, words_small);
         if (s_act[1]) {
             atomicAdd(&a.cnt->n_big, s_act[1]);
+            if (s_act[2]) atomicAdd(&a.cnt->n_direct, s_act[2]);
             atomicAdd(&a.cnt->words_big, words_big);
             atomicMax(&a.cnt->e_max, e_max);
         }
@@ -649,11 +719,11 @@ struct TwohopArgs {
     Counters *cnt;
     Totals tot;
     uint32_t n_ranks;               // anchors of the side
-    int direct;                     // direct counters allowed (not when a test forces the hash strategies)
     int single;                     // one partner: the counters give the sum, no rows are written
     unsigned long long *bucket;     // per-CTA bucket slots of the large-anchor kernel
     unsigned long long bucket_slot; // entries per slot
-    unsigned large_begin, large_end;  // order[] ranges of the two kernels
+    unsigned direct_begin, direct_end;  // order[] ranges of the three kernels
+    unsigned large_begin, large_end;
     unsigned small_begin, small_end;
     int l;
     int check;                      // run the candidate-mask self-check
@@ -727,8 +797,14 @@ __device__ __forceinline__ void visit_warp(int64_t ebase, int d, bool useful_onl
     }
 }
 
+// The 2-hop kernels of one launch_twohop overlap: a kernel lets the next one start
+// once all its CTAs run, and ends only after the one before it.
+__device__ __forceinline__ void twohop_let_next_start() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void twohop_wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 template <bool STATS>
-__global__ void __launch_bounds__(PS_THREADS) k_twohop_small(TwohopArgs a) {
+__global__ void __launch_bounds__(PS_THREADS) k_twohop_small(const __grid_constant__ TwohopArgs a) {
+    twohop_let_next_start();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t *keys = (uint32_t *)(smem_raw + (size_t)warp * PS_HS * 4);
@@ -852,6 +928,7 @@ __global__ void __launch_bounds__(PS_THREADS) k_twohop_small(TwohopArgs a) {
         if (leaves) atomicAdd(&a.cnt->leaves, leaves);
     }
     if (lane == 0 && wedges) atomicAdd(&a.cnt->wedges, wedges);
+    twohop_wait_previous();
 }
 
 // ---- large anchors: one CTA per anchor, wedges flattened over the CTA
@@ -984,113 +1061,78 @@ __device__ __forceinline__ void visit_block(int64_t ebase, int d, bool useful_on
     }
 }
 
-// ---- direct counters. A partner's rank follows the anchor's, and anchors with
-// many wedges have high degrees, so high ranks: their partners' ranks span a
-// short range (on the 2M-edge graph 76 % of the wedges of anchors above 3,584
-// span at most 48k ranks). Such an anchor counts its partners in a table
-// indexed by rank - no keys, no probes, one shared-memory add without a return
-// value per wedge - in windows of consecutive ranks, each a pass over the
-// 2-hop. Counters hold the same-sign and different-sign counts of a partner in
-// 8 + 8 bits (at most 255 useful positions) or 16 + 16 bits. After a window's
-// counts, a bitmap of the parts with at least l positions and its prefix counts
-// number the rows, and the counters' memory stages the mask words of the
-// window's rows, a range of positions at a time.
-// Bound by the shared-memory atomics and the L2 gathers of B_ent. The 2-hop
-// kernels of the (3,3) count took 13.7 -> 6.4 ms on the 2M-edge graph, 74 -> 32
-// ms on a 12M-edge hub graph and 15.6 -> 1.4 ms on a dense 3000 x 800 graph
-// (hash strategies -> direct counters where the rule takes them).
-constexpr uint32_t DT_WORDS = 20480;            // counter words, then staged mask words
-constexpr uint32_t DT_CELLS8 = 2 * DT_WORDS;    // ranks per window with 8 + 8 bit counters
-constexpr uint32_t DT_CELLS16 = DT_WORDS;
-constexpr uint32_t DT_BM = DT_CELLS8 / 16;      // bitmap words (two bits per rank)
-constexpr size_t DT_OFF_BM = (size_t)DT_WORDS * 4;
-constexpr size_t DT_OFF_PRE = DT_OFF_BM + (size_t)DT_BM * 4;
-constexpr size_t DT_OFF_POFF = DT_OFF_PRE + (size_t)DT_BM * 4;
-constexpr size_t DT_OFF_PPRE = DT_OFF_POFF + (size_t)PL_PCH * 4;
-constexpr size_t DT_OFF_PINFO = DT_OFF_PPRE + (size_t)(PL_PCH + 4) * 4;
-static_assert(DT_OFF_PINFO + (size_t)PL_PCH * 4 <= PL_SMEM, "direct counters' shared layout");
+// ---- direct counters (see their description above the plan)
 
-// Direct counters or the hash strategies. Lists of at least 8 partners on
-// average (in shorter ones, of the widest hubs, few partners share all the
-// counters). Costs in SM cycles measured on the 2M-edge graph: a window about
-// 3,000 (clear, scan, barriers) and 0.7 per wedge for its two passes; the hash
-// strategies about 8 per wedge.
-__device__ __forceinline__ bool direct_takes(unsigned long long e, uint32_t dp, uint32_t range) {
-    if (dp > 65535u || e < 8ull * dp) return false;
-    const uint32_t cells = dp <= 255u ? DT_CELLS8 : DT_CELLS16;
-    const float nwin = (float)((range + cells - 1) / cells);
-    return nwin * (3000.0f + 0.7f * (float)e) < 8.0f * (float)e;
+// Positions staged in shared memory: list p's entries t in [ppre[p], ppre[p + 1])
+// are B_ent[poff[p] + t], pinfo[p] holds the sign of the position and its bit
+// index.
+struct Lists {
+    uint32_t *poff, *ppre, *pinfo;
+    uint32_t *wtot;  // DT_WARPS + 1 words: scan scratch
+};
+
+// Exclusive scan of one 32-bit value per thread over the CTA; *total: the sum.
+__device__ __forceinline__ uint32_t block_excl_scan_u32(uint32_t v, uint32_t *wtot, uint32_t *total) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(FULL, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) wtot[warp] = incl;
+    __syncthreads();
+    const uint32_t x = lane < DT_WARPS ? wtot[lane] : 0u;
+    uint32_t xi = x;
+#pragma unroll
+    for (int o = 1; o < DT_WARPS; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(FULL, xi, o);
+        if (lane >= o) xi += t;
+    }
+    *total = __shfl_sync(FULL, xi, DT_WARPS - 1);
+    return __shfl_sync(FULL, xi - x, warp) + incl - v;
 }
 
-// Visit the anchor's 2-hop entries at the useful positions whose bit index lies
-// in [blo, bhi), with the whole CTA: positions staged PL_PCH at a time, the
-// non-empty ones compacted; the entries of a batch are split evenly over the
-// warps, every lane finds its first list by a search and walks forward from
-// it, four entries in flight. fn(entry, sign of the position | bit index).
+// Walk the entries of the staged lists [plo, phi) with the whole CTA: split
+// evenly over the warps; every lane finds its first list by a search and walks
+// forward from it, four entries in flight. fn(entry, sign | bit index).
 template <typename F>
-__device__ __forceinline__ void visit_lists(int64_t ebase, int d, uint32_t blo, uint32_t bhi,
-                                            const TwohopArgs &a, uint32_t *poff, uint32_t *ppre,
-                                            uint32_t *pinfo, unsigned long long *warp_tot,
-                                            unsigned long long *s_total, F fn) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int c0 = 0; c0 < d; c0 += PL_PCH) {
-        uint32_t len = 0, info = 0, st = 0;
-        if (c0 + tid < d) {
-            const int64_t e = ebase + c0 + tid;
-            const uint32_t bit = a.A_bit[e];
-            if (bit >= blo && bit < bhi) {  // (EMPTY is above every bhi)
-                const uint32_t av = a.A_ent[e];
-                const uint32_t y = av & VMASK;
-                st = (uint32_t)(a.B_off[y] + (int64_t)a.A_pos[e] + 1);
-                len = (uint32_t)a.B_off[y + 1] - st;
-                info = (av & 0x80000000u) | bit;
-            }
-        }
-        const unsigned long long packed = len ? ((1ull << 32) | len) : 0ull;
-        const unsigned long long ex = block_excl_scan_u64(packed, warp_tot, s_total);
-        if (len) {
-            const uint32_t slot = (uint32_t)(ex >> 32);
-            ppre[slot] = (uint32_t)ex;
-            poff[slot] = st - (uint32_t)ex;
-            pinfo[slot] = info;
-        }
-        const uint32_t npos = (uint32_t)(*s_total >> 32);
-        const uint32_t total = (uint32_t)*s_total;
-        if (tid == 0) ppre[npos] = total;
-        __syncthreads();
-        const uint32_t per = ((total + PL_THREADS - 1) / PL_THREADS) * 32;
-        const uint32_t t1 = (uint32_t)(warp + 1) * per < total ? (uint32_t)(warp + 1) * per : total;
-        uint32_t t = (uint32_t)warp * per + lane;
-        if (t < t1) {
-            uint32_t p = 0, hi = npos;  // largest p with ppre[p] <= t
-            while (hi - p > 1) {
-                const uint32_t mid = (p + hi) >> 1;
-                if (ppre[mid] <= t) p = mid; else hi = mid;
-            }
-            uint32_t nxt = ppre[p + 1], off = poff[p], inf = pinfo[p];
-            while (t < t1) {
-                uint32_t ent[4], pin[4];
+__device__ __forceinline__ void walk_lists(const Lists &L, uint32_t plo, uint32_t phi,
+                                           const uint32_t *__restrict__ B_ent, F fn) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t tb = L.ppre[plo], te = L.ppre[phi];
+    const uint32_t per = ((te - tb + DT_THREADS - 1) / DT_THREADS) * 32;
+    const uint32_t t1 = min(te, tb + (uint32_t)(warp + 1) * per);
+    uint32_t t = tb + (uint32_t)warp * per + lane;
+    if (t >= t1) return;
+    uint32_t p = plo, hi = phi;  // largest p with ppre[p] <= t
+    while (hi - p > 1) {
+        const uint32_t mid = (p + hi) >> 1;
+        if (L.ppre[mid] <= t) p = mid; else hi = mid;
+    }
+    uint32_t nxt = L.ppre[p + 1], off = L.poff[p], inf = L.pinfo[p];
+    while (t < t1) {
+        uint32_t ent[4], pin[4];
 #pragma unroll
-                for (int k = 0; k < 4; k++) {
-                    const uint32_t tt = t + 32 * k;
-                    if (tt < t1) {
-                        while (tt >= nxt) {
-                            p++;
-                            nxt = ppre[p + 1];
-                            off = poff[p];
-                            inf = pinfo[p];
-                        }
-                        ent[k] = a.B_ent[off + tt];
-                        pin[k] = inf;
-                    }
+        for (int k = 0; k < 4; k++) {
+            const uint32_t tt = t + 32 * k;
+            if (tt < t1) {
+                if (tt >= nxt) {
+                    do {
+                        p++;
+                        nxt = L.ppre[p + 1];
+                    } while (tt >= nxt);
+                    off = L.poff[p];
+                    inf = L.pinfo[p];
                 }
-#pragma unroll
-                for (int k = 0; k < 4; k++)
-                    if (t + 32 * k < t1) fn(ent[k], pin[k]);
-                t += 128;
+                ent[k] = B_ent[off + tt];
+                pin[k] = inf;
             }
         }
-        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+            if (t + 32 * k < t1) fn(ent[k], pin[k]);
+        t += 128;
     }
 }
 
@@ -1101,15 +1143,27 @@ struct DirectOut {
     bool failed = false;
 };
 
+// Position of the part `sdiff` of rank idx in its bitmap word: the words of 16
+// ranks' counters are compared four counters at a time, byte (or half) b of
+// counter word w to bit 8 b + w (8-bit counters: two ranks per word) or
+// 16 b + w (16-bit counters: one).
 template <bool C8>
-__device__ __noinline__ DirectOut direct_anchor(const TwohopArgs &a, uint32_t r, uint32_t range,
+__device__ __forceinline__ uint32_t part_bit(uint32_t idx, uint32_t sdiff) {
+    if constexpr (C8) return ((idx & 1u) << 4) + (sdiff << 3) + ((idx >> 1) & 7u);
+    else return (sdiff << 4) + (idx & 15u);
+}
+
+template <bool C8>
+__device__ __forceinline__ DirectOut direct_anchor(const TwohopArgs &a, uint32_t r, uint32_t range,
                                                 unsigned char *smem, unsigned long long *warp_tot,
-                                                unsigned long long *s_total, unsigned *s_nrw,
-                                                unsigned *s_ncw) {
+                                                unsigned *s_nrw, unsigned *s_ncw) {
     uint32_t *tbl = (uint32_t *)smem;
     uint32_t *bm = (uint32_t *)(smem + DT_OFF_BM), *pre = (uint32_t *)(smem + DT_OFF_PRE);
-    uint32_t *poff = (uint32_t *)(smem + DT_OFF_POFF), *ppre = (uint32_t *)(smem + DT_OFF_PPRE);
-    uint32_t *pinfo = (uint32_t *)(smem + DT_OFF_PINFO);
+    Lists L;
+    L.poff = (uint32_t *)(smem + DT_OFF_POFF);
+    L.ppre = (uint32_t *)(smem + DT_OFF_PPRE);
+    L.pinfo = (uint32_t *)(smem + DT_OFF_PINFO);
+    L.wtot = (uint32_t *)warp_tot;
     constexpr uint32_t CELLS = C8 ? DT_CELLS8 : DT_CELLS16;
     const int tid = threadIdx.x, lane = tid & 31;
     const int l = a.l;
@@ -1117,17 +1171,92 @@ __device__ __noinline__ DirectOut direct_anchor(const TwohopArgs &a, uint32_t r,
     const int d = (int)(a.A_off[r + 1] - ebase);
     const uint32_t dp = a.dprime[r], W = (dp + 31) / 32, rsv = a.rsv_c[r];
     uint32_t *region = a.pool + a.pool_off[r];
+    const uint32_t *__restrict__ B_ent = a.B_ent;
     DirectOut out;
     if (tid == 0) *s_nrw = *s_ncw = 0;
+    // With at most DT_PCH positions every position has its thread: the useful
+    // ones, numbered by their bit index, are staged once per window, cut to the
+    // window's ranks (lists ascend by rank, so a search finds the cut).
+    const bool one = d <= DT_PCH;
+    uint32_t st = 0, en = 0, info = EMPTY;
+    if (one && tid < d) {
+        const int64_t e = ebase + tid;
+        const uint32_t bit = a.A_bit[e];
+        if (bit != EMPTY) {
+            const uint32_t av = a.A_ent[e], y = av & VMASK;
+            st = (uint32_t)(a.B_off[y] + (int64_t)a.A_pos[e] + 1);
+            en = (uint32_t)a.B_off[y + 1];
+            info = (av & 0x80000000u) | bit;
+        }
+    }
+    // Positions c0 .. c0 + DT_PCH - 1 with bits in [blo, bhi), compacted.
+    auto stage_batch = [&](int c0, uint32_t blo, uint32_t bhi) -> uint32_t {
+        uint32_t len = 0, s0 = 0, inf = 0;
+        if (c0 + tid < d) {
+            const int64_t e = ebase + c0 + tid;
+            const uint32_t bit = a.A_bit[e];
+            if (bit >= blo && bit < bhi) {  // (EMPTY is above every bhi)
+                const uint32_t av = a.A_ent[e], y = av & VMASK;
+                s0 = (uint32_t)(a.B_off[y] + (int64_t)a.A_pos[e] + 1);
+                len = (uint32_t)a.B_off[y + 1] - s0;
+                inf = (av & 0x80000000u) | bit;
+            }
+        }
+        uint32_t npos = 0, total = 0;
+        const uint32_t slot = block_excl_scan_u32(len ? 1u : 0u, L.wtot, &npos);
+        __syncthreads();
+        const uint32_t ex = block_excl_scan_u32(len, L.wtot, &total);
+        if (len) {
+            L.ppre[slot] = ex;
+            L.poff[slot] = s0 - ex;
+            L.pinfo[slot] = inf;
+        }
+        if (tid == 0) L.ppre[npos] = total;
+        __syncthreads();
+        return npos;
+    };
+    // All entries at the bits [blo, bhi) (of the window staged last).
+    auto visit = [&](uint32_t blo, uint32_t bhi, auto &&fn) {
+        if (one) {
+            walk_lists(L, blo, bhi, B_ent, fn);
+            __syncthreads();
+            return;
+        }
+        for (int c0 = 0; c0 < d; c0 += DT_PCH) {
+            const uint32_t npos = stage_batch(c0, blo, bhi);
+            if (npos) walk_lists(L, 0, npos, B_ent, fn);
+            __syncthreads();
+        }
+    };
     for (uint32_t w0 = 0; w0 < range; w0 += CELLS) {
         const uint32_t base = r + 1 + w0, nw = range - w0 < CELLS ? range - w0 : CELLS;
         const uint32_t nbm = (nw + 15) / 16;
         // counts
-        for (uint32_t i = tid; i < nbm * (C8 ? 2u : 4u); i += PL_THREADS)
+        for (uint32_t i = tid; i < nbm * (C8 ? 2u : 4u); i += DT_THREADS)
             reinterpret_cast<uint4 *>(tbl)[i] = make_uint4(0, 0, 0, 0);
+        if (one) {
+            uint32_t cut = en;
+            if (w0 + CELLS < range && info != EMPTY) {  // first entry past the window
+                uint32_t lo = st;
+                while (lo < cut) {
+                    const uint32_t mid = (lo + cut) >> 1;
+                    if ((B_ent[mid] & VMASK) < base + nw) lo = mid + 1; else cut = mid;
+                }
+            }
+            uint32_t total = 0;
+            const uint32_t ex = block_excl_scan_u32(cut - st, L.wtot, &total);
+            if (info != EMPTY) {
+                const uint32_t slot = info & VMASK;
+                L.ppre[slot] = ex;
+                L.poff[slot] = st - ex;
+                L.pinfo[slot] = info;
+            }
+            if (tid == 0) L.ppre[dp] = total;
+            st = cut;
+        }
         __syncthreads();
         const uint32_t nr0 = *s_nrw;
-        visit_lists(ebase, d, 0, dp, a, poff, ppre, pinfo, warp_tot, s_total, [&](uint32_t ent, uint32_t inf) {
+        visit(0, dp, [&](uint32_t ent, uint32_t inf) {
             const uint32_t idx = (ent & VMASK) - base;
             if (idx < nw) {
                 const uint32_t sdiff = (ent ^ inf) >> 31;
@@ -1137,67 +1266,76 @@ __device__ __noinline__ DirectOut direct_anchor(const TwohopArgs &a, uint32_t r,
         });
         out.passes++;
         long long check = 0;  // self-check: bits written minus bits counted
-        // rows: two bits per rank (same-sign part, different-sign part)
-        for (uint32_t j0 = 0; j0 < nbm; j0 += PL_THREADS) {
+        // rows: a bit per rank and part (part_bit)
+        uint32_t all = 0;     // OR (8-bit) or maximum (16-bit) of the counters: bounds the longest row
+        for (uint32_t j0 = 0; j0 < nbm; j0 += DT_THREADS) {
             const uint32_t j = j0 + tid;
             uint32_t bits = 0;
             if (j < nbm) {
                 if constexpr (C8) {
-                    const uint32_t lim = (uint32_t)l * 0x01010101u;
+                    // per byte: bit 7 of (low 7 bits + 128 - l) | byte is set
+                    // when the byte is at least l (l <= 8)
+                    const uint32_t add = (128u - (uint32_t)l) * 0x01010101u;
 #pragma unroll
                     for (int h = 0; h < 2; h++) {
                         const uint4 v = reinterpret_cast<const uint4 *>(tbl)[2 * j + h];
                         const uint32_t x[4] = {v.x, v.y, v.z, v.w};
-                        if (v.x | v.y | v.z | v.w) {
 #pragma unroll
-                            for (int k = 0; k < 4; k++) {
-                                // bytes >= l to four bits in byte order
-                                const uint32_t m = __vcmpgeu4(x[k], lim) & 0x08040201u;
-                                bits |= (((m * 0x01010101u) >> 24) & 15u) << (16 * h + 4 * k);
-                            }
+                        for (int k = 0; k < 4; k++) {
+                            const uint32_t m = (((x[k] & 0x7F7F7F7Fu) + add) | x[k]) & 0x80808080u;
+                            bits |= m >> (7 - (4 * h + k));
+                            all |= x[k];
                         }
                     }
                 } else {
+                    const uint32_t add = (32768u - (uint32_t)l) * 0x00010001u;
 #pragma unroll
                     for (int h = 0; h < 4; h++) {
                         const uint4 v = reinterpret_cast<const uint4 *>(tbl)[4 * j + h];
                         const uint32_t x[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-                        for (int k = 0; k < 4; k++)
-                            bits |= (((x[k] & 0xFFFFu) >= (uint32_t)l ? 1u : 0u) |
-                                     ((x[k] >> 16) >= (uint32_t)l ? 2u : 0u)) << (8 * h + 2 * k);
+                        for (int k = 0; k < 4; k++) {
+                            const uint32_t m = (((x[k] & 0x7FFF7FFFu) + add) | x[k]) & 0x80008000u;
+                            bits |= m >> (15 - (4 * h + k));
+                            all = __vmaxu2(all, x[k]);
+                        }
                     }
                 }
             }
             const uint32_t cnt = __popc(bits);
             uint32_t incl = cnt;
+            if (__any_sync(FULL, bits != 0)) {
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t t = __shfl_up_sync(FULL, incl, o);
-                if (lane >= o) incl += t;
-            }
-            const uint32_t tot = __shfl_sync(FULL, incl, 31);
-            if (tot) {
-                const uint32_t ncw = __reduce_add_sync(FULL, (uint32_t)__popc((bits | (bits >> 1)) & 0x55555555u));
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t t = __shfl_up_sync(FULL, incl, o);
+                    if (lane >= o) incl += t;
+                }
+                const uint32_t both = C8 ? (bits | (bits >> 8)) & 0x00FF00FFu : (bits | (bits >> 16)) & 0xFFFFu;
+                const uint32_t ncw = __reduce_add_sync(FULL, (uint32_t)__popc(both));
                 uint32_t at = 0;
-                if (lane == 0) {
-                    at = atomicAdd(s_nrw, tot);
+                if (lane == 31) {
+                    at = atomicAdd(s_nrw, incl);
                     atomicAdd(s_ncw, ncw);
                 }
-                at = __shfl_sync(FULL, at, 0) + incl - cnt;
+                at = __shfl_sync(FULL, at, 31) + incl - cnt;
                 if (j < nbm) pre[j] = at;
-                uint32_t b = bits;
-                while (b) {
-                    const uint32_t k = __ffs(b) - 1;
-                    b &= b - 1;
-                    const uint32_t x = C8 ? (uint32_t)smem[32 * j + k] : (uint32_t)((uint16_t *)smem)[32 * j + k];
-                    if (a.single) binom_add(out.sum, x, l, &a.cnt->err);
-                    else out.rst.add(x);
-                    check -= x;
+                if (a.single || a.check) {
+                    uint32_t b = bits;
+                    while (b) {
+                        const uint32_t k = __ffs(b) - 1;
+                        b &= b - 1;
+                        const uint32_t x = C8 ? (uint32_t)smem[32 * j + 4 * (k & 7u) + (k >> 3)]
+                                              : (uint32_t)((uint16_t *)smem)[32 * j + 2 * (k & 15u) + (k >> 4)];
+                        if (a.single) binom_add(out.sum, x, l, &a.cnt->err);
+                        check -= x;
+                    }
                 }
             }
             if (j < nbm) bm[j] = bits;
         }
+        if constexpr (C8) all |= all >> 16;
+        out.rst.longest = max(out.rst.longest, C8 ? max(all & 0xFFu, (all >> 8) & 0xFFu)
+                                                  : max(all & 0xFFFFu, all >> 16));
         __syncthreads();
         const uint32_t nrw = *s_nrw - nr0;
         if (a.single || nrw == 0) {
@@ -1214,39 +1352,55 @@ __device__ __noinline__ DirectOut direct_anchor(const TwohopArgs &a, uint32_t r,
         if (cw > W) cw = W;
         const bool staged = cw > 0;
         if (!staged) cw = W;
+        uint32_t hits = 0;
         for (uint32_t wa = 0; wa < W; wa += cw) {
             const uint32_t wn = W - wa < cw ? W - wa : cw;
-            for (uint32_t i = tid; i < wn * nrw; i += PL_THREADS) {
-                if (staged) tbl[i] = 0;
-                else region[(size_t)(i / nrw) * rsv + nr0 + i % nrw] = 0;
+            if (staged) {
+                for (uint32_t i = tid; i < (wn * nrw + 3) / 4; i += DT_THREADS)
+                    reinterpret_cast<uint4 *>(tbl)[i] = make_uint4(0, 0, 0, 0);
+            } else {
+                for (uint32_t i = tid; i < wn * nrw; i += DT_THREADS)
+                    region[(size_t)(i / nrw) * rsv + nr0 + i % nrw] = 0;
             }
             __syncthreads();
-            visit_lists(ebase, d, 32 * wa, 32 * (wa + wn) < dp ? 32 * (wa + wn) : dp, a, poff, ppre, pinfo,
-                        warp_tot, s_total, [&](uint32_t ent, uint32_t inf) {
-                            const uint32_t idx = (ent & VMASK) - base;
-                            if (idx >= nw) return;
-                            const uint32_t k = 2 * (idx & 15u) + ((ent ^ inf) >> 31);
-                            const uint32_t bw = bm[idx >> 4];
-                            if (!((bw >> k) & 1u)) return;
-                            const uint32_t row = pre[idx >> 4] + __popc(bw & ((1u << k) - 1u));
-                            const uint32_t bit = inf & VMASK, m = 1u << (bit & 31);
-                            if (staged) atomicOr(&tbl[((bit >> 5) - wa) * nrw + row - nr0], m);
-                            else atomicOr(&region[(size_t)(bit >> 5) * rsv + row], m);
-                        });
+            visit(32 * wa, 32 * (wa + wn) < dp ? 32 * (wa + wn) : dp, [&](uint32_t ent, uint32_t inf) {
+                const uint32_t idx = (ent & VMASK) - base;
+                if (idx >= nw) return;
+                const uint32_t k = part_bit<C8>(idx, (ent ^ inf) >> 31);
+                const uint32_t bw = bm[idx >> 4];
+                if (!((bw >> k) & 1u)) return;
+                hits++;
+                const uint32_t row = pre[idx >> 4] + __popc(bw & ((1u << k) - 1u));
+                const uint32_t bit = inf & VMASK, m = 1u << (bit & 31);
+                if (staged) atomicOr(&tbl[((bit >> 5) - wa) * nrw + row - nr0], m);
+                else atomicOr(&region[(size_t)(bit >> 5) * rsv + row], m);
+            });
             if (staged) {
-                for (uint32_t i = tid; i < wn * nrw; i += PL_THREADS) {
-                    const uint32_t wd = i / nrw, x = tbl[i];
-                    region[(size_t)(wa + wd) * rsv + nr0 + (i - wd * nrw)] = x;
-                    check += __popc(x);
+                if (nrw >= 64) {
+                    for (uint32_t wd = 0; wd < wn; wd++)
+                        for (uint32_t i = tid; i < nrw; i += DT_THREADS)
+                            region[(size_t)(wa + wd) * rsv + nr0 + i] = tbl[wd * nrw + i];
+                } else {
+                    for (uint32_t i = tid; i < wn * nrw; i += DT_THREADS) {
+                        const uint32_t wd = i / nrw;
+                        region[(size_t)(wa + wd) * rsv + nr0 + (i - wd * nrw)] = tbl[i];
+                    }
                 }
+                if (a.check)
+                    for (uint32_t i = tid; i < wn * nrw; i += DT_THREADS) check += __popc(tbl[i]);
                 __syncthreads();
             }
         }
+        out.rst.pops += (float)hits;
         out.passes++;
         if (a.check && staged) {
             // self-check: the window's rows hold as many bits as its counters say
-            block_excl_scan_u64((unsigned long long)check, warp_tot, s_total);
-            if (*s_total != 0 && tid == 0) atomicOr(&a.cnt->err, CERR_MASK);
+            unsigned long long *scr = (unsigned long long *)(smem + DT_OFF_BM);  // (free now)
+            if (tid == 0) *scr = 0;
+            __syncthreads();
+            atomicAdd(scr, (unsigned long long)check);
+            __syncthreads();
+            if (tid == 0 && *scr != 0) atomicOr(&a.cnt->err, CERR_MASK);
             __syncthreads();
         }
     }
@@ -1262,8 +1416,96 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 
+// Direct counters, one CTA per anchor.
+__global__ void __launch_bounds__(DT_THREADS, 2) k_twohop_direct(const __grid_constant__ TwohopArgs a) {
+    twohop_let_next_start();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ unsigned long long warp_tot[DT_WARPS];
+    __shared__ unsigned s_item, s_nrw, s_ncw, s_longest;
+    __shared__ uint32_t s_rank, s_range;
+    __shared__ float s_pops;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const bool split_totals = a.tot.per_anchor || a.tot.per_graph;
+    unsigned long long wedges = 0, tested = 0, leaves = 0, reads = 0, cycles = 0, anchors = 0;
+    U128 sum;  // one partner: this thread's share of the sums
+    // the next item is claimed, and its anchor looked up, while this one runs
+    if (tid == 0) {
+        s_item = a.direct_begin + atomicAdd(&a.cnt->head_direct, 1u);
+        s_rank = s_item < a.direct_end ? a.order[s_item] : 0u;
+    }
+    for (;;) {
+        __syncthreads();
+        if (s_item >= a.direct_end) break;
+        const uint32_t r = s_rank;
+        const long long c0 = clock64();
+        unsigned next = 0;
+        uint32_t next_rank = 0;
+        if (tid == 0) {
+            next = a.direct_begin + atomicAdd(&a.cnt->head_direct, 1u);
+            if (next < a.direct_end) next_rank = a.order[next];
+            s_range = rank_end(a.tot.per_graph ? a.tot.graph_x0 : nullptr, a.tot.n_graphs, a.n_ranks, r) - 1 - r;
+            s_pops = 0.f;
+            s_longest = 0;
+        }
+        __syncthreads();
+        DirectOut o = a.dprime[r] <= 255u ? direct_anchor<true>(a, r, s_range, smem_raw, warp_tot, &s_nrw, &s_ncw)
+                                          : direct_anchor<false>(a, r, s_range, smem_raw, warp_tot, &s_nrw, &s_ncw);
+        if (o.failed) o.nc = o.nr = 0;
+        if (a.single) {
+            if (sum.add(o.sum)) atomicOr(&a.cnt->err, CERR_OVERFLOW);
+            if (split_totals) {
+                const U128 ws = warp_sum_u128(sum, &a.cnt->err);
+                if (lane == 0) add_totals(a.tot, r, ws);
+                sum = U128();
+            }
+        } else {
+            o.rst.warp_sum();
+            if (lane == 0) {
+                atomicAdd(&s_pops, o.rst.pops);
+                atomicMax(&s_longest, o.rst.longest);
+            }
+            __syncthreads();
+        }
+        if (tid == 0) {
+            a.ncand[r] = o.nc;
+            a.nrow[r] = o.nr;
+            RowInfo ri;
+            ri.pops = s_pops;
+            ri.longest = s_longest;
+            a.rinfo[r] = ri;
+            if (a.single) {
+                tested += o.nc;
+                leaves += o.nr;
+            }
+            wedges += a.e_use[r];
+            reads += a.e_use[r] * o.passes;
+            cycles += (unsigned long long)(clock64() - c0);
+            anchors++;
+            s_item = next;
+            s_rank = next_rank;
+        }
+    }
+    if (a.single && !split_totals) {
+        const U128 ws = warp_sum_u128(sum, &a.cnt->err);
+        if (lane == 0) add_totals(a.tot, 0, ws);
+    }
+    if (tid == 0) {
+        if (wedges) atomicAdd(&a.cnt->wedges, wedges);
+        if (tested) atomicAdd(&a.cnt->tested, tested);
+        if (leaves) atomicAdd(&a.cnt->leaves, leaves);
+        atomicAdd(&a.cnt->tw_reads, reads);
+        atomicAdd(&a.cnt->tw_cyc[0], cycles);
+        atomicAdd(&a.cnt->tw_anchors[0], anchors);
+        const unsigned long long t = global_ns();
+        atomicMax(&a.cnt->tw_fin_max, t);
+        atomicMax(&a.cnt->tw_fin_min_n, ~t);
+    }
+    twohop_wait_previous();
+}
+
 template <bool STATS>
-__global__ void __launch_bounds__(PL_THREADS, 2) k_twohop_large(TwohopArgs a) {
+__global__ void __launch_bounds__(PL_THREADS, 2) k_twohop_large(const __grid_constant__ TwohopArgs a) {
+    twohop_let_next_start();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     uint32_t *keys = (uint32_t *)smem_raw;
     unsigned long long *vals = (unsigned long long *)(smem_raw + PL_OFF_VALS);
@@ -1275,7 +1517,7 @@ __global__ void __launch_bounds__(PL_THREADS, 2) k_twohop_large(TwohopArgs a) {
     __shared__ unsigned long long s_total;
     __shared__ unsigned s_item, s_ncw, s_nrw, s_paper, s_ovf;
     __shared__ float s_pops;
-    __shared__ uint32_t s_range;
+    __shared__ uint32_t s_rank;
     __shared__ unsigned s_longest;
     __shared__ uint32_t s_bcnt[PL_MAXCLS];
     const int tid = threadIdx.x, lane = tid & 31;
@@ -1329,13 +1571,23 @@ __global__ void __launch_bounds__(PL_THREADS, 2) k_twohop_large(TwohopArgs a) {
         if (row != EMPTY) atomicOr(&bb[(size_t)(bit >> 5) * bstride + row], 1u << (bit & 31));
     };
 
+    // the next item is claimed, and its anchor looked up, while this one runs
+    if (tid == 0) {
+        s_item = a.large_begin + atomicAdd(&a.cnt->head_large, 1u);
+        s_rank = s_item < a.large_end ? a.order[s_item] : 0u;
+    }
     for (;;) {
-        if (tid == 0) s_item = a.large_begin + atomicAdd(&a.cnt->head_large, 1u);
         __syncthreads();
         const unsigned item = s_item;
-        __syncthreads();
         if (item >= a.large_end) break;
-        const uint32_t r = a.order[item];
+        const uint32_t r = s_rank;
+        __syncthreads();
+        unsigned next = 0;
+        uint32_t next_rank = 0;
+        if (tid == 0) {
+            next = a.large_begin + atomicAdd(&a.cnt->head_large, 1u);
+            if (next < a.large_end) next_rank = a.order[next];
+        }
         const int64_t ebase = a.A_off[r];
         const int d = (int)(a.A_off[r + 1] - ebase);
         const uint32_t W = (a.dprime[r] + 31) / 32;
@@ -1415,38 +1667,8 @@ __global__ void __launch_bounds__(PL_THREADS, 2) k_twohop_large(TwohopArgs a) {
         };
 
         const int lgb = bucket_lg(e_vis);
-        bool bucketed = false, direct = false;
-        if constexpr (!STATS) {
-            // ranks above the anchor's (in a batch: of its own graph)
-            if (tid == 0) {
-                uint32_t end = a.n_ranks;
-                if (a.tot.per_graph) {
-                    int lo = 0, hi = a.tot.n_graphs;
-                    while (hi - lo > 1) {
-                        const int mid = (lo + hi) >> 1;
-                        if (a.tot.graph_x0[mid] <= (int64_t)r) lo = mid; else hi = mid;
-                    }
-                    end = (uint32_t)a.tot.graph_x0[lo + 1];
-                }
-                s_range = end - 1 - r;
-            }
-            __syncthreads();
-            const uint32_t range = s_range;
-            direct = a.direct && direct_takes(e_use, a.dprime[r], range);
-            if (direct) {
-                DirectOut o = a.dprime[r] <= 255u
-                    ? direct_anchor<true>(a, r, range, smem_raw, warp_tot, &s_total, &s_nrw, &s_ncw)
-                    : direct_anchor<false>(a, r, range, smem_raw, warp_tot, &s_total, &s_nrw, &s_ncw);
-                nc = o.nc;
-                nr = o.nr;
-                failed = o.failed;
-                rst = o.rst;
-                if (sum.add(o.sum)) atomicOr(&a.cnt->err, CERR_OVERFLOW);
-                reads = e_use * o.passes;
-            }
-        }
-        if (direct) {
-        } else if (e_vis <= (unsigned long long)a.wcap) {
+        bool bucketed = false;
+        if (e_vis <= (unsigned long long)a.wcap) {
             // one window
             uint32_t hs = (uint32_t)((2 * e_vis + 31) & ~31ull);
             hs = hs < 64 ? 64 : (hs > PL_HS ? PL_HS : hs);
@@ -1570,7 +1792,7 @@ __global__ void __launch_bounds__(PL_THREADS, 2) k_twohop_large(TwohopArgs a) {
                 }
             }
         }
-        if (!direct && !bucketed && !failed && e_vis > (unsigned long long)a.wcap) {
+        if (!bucketed && !failed && e_vis > (unsigned long long)a.wcap) {
             // re-read windows: every pass over the 2-hop keeps one hash class
             const U128 sum0 = sum;
             int lg_nw = 0;
@@ -1645,8 +1867,9 @@ __global__ void __launch_bounds__(PL_THREADS, 2) k_twohop_large(TwohopArgs a) {
             atomicAdd(&a.cnt->tw_reads, reads);
             atomicAdd(&a.cnt->tw_cyc[path], (unsigned long long)(clock64() - c0));
             atomicAdd(&a.cnt->tw_anchors[path], 1ull);
+            s_item = next;
+            s_rank = next_rank;
         }
-        __syncthreads();
     }
     if (a.single && !split_totals) {
         const U128 ws = warp_sum_u128(sum, &a.cnt->err);
@@ -1656,10 +1879,13 @@ __global__ void __launch_bounds__(PL_THREADS, 2) k_twohop_large(TwohopArgs a) {
         if (wedges) atomicAdd(&a.cnt->wedges, wedges);
         if (tested) atomicAdd(&a.cnt->tested, tested);
         if (leaves) atomicAdd(&a.cnt->leaves, leaves);
-        const unsigned long long t = global_ns();
-        atomicMax(&a.cnt->tw_fin_max, t);
-        atomicMax(&a.cnt->tw_fin_min_n, ~t);
+        if (a.direct_begin == a.direct_end) {  // (else the direct kernel's are taken)
+            const unsigned long long t = global_ns();
+            atomicMax(&a.cnt->tw_fin_max, t);
+            atomicMax(&a.cnt->tw_fin_min_n, ~t);
+        }
     }
+    twohop_wait_previous();
 }
 
 // ------------------------------------------------------------------ groups
@@ -1753,6 +1979,7 @@ void ensure_kernel_attrs() {
     SBC_CUDA(cudaMemcpyToSymbol(c_binom64_max, lim, sizeof(lim)));
     SBC_CUDA(cudaFuncSetAttribute(k_twohop_small<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PS_SMEM));
     SBC_CUDA(cudaFuncSetAttribute(k_twohop_small<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PS_SMEM));
+    SBC_CUDA(cudaFuncSetAttribute(k_twohop_direct, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DT_SMEM));
     SBC_CUDA(cudaFuncSetAttribute(k_twohop_large<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PL_SMEM));
     SBC_CUDA(cudaFuncSetAttribute(k_twohop_large<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PL_SMEM));
     tc_ensure_attrs();
@@ -1823,7 +2050,7 @@ struct CountRun {
     std::vector<TcPlan> tc_plans;   // per anchor group
     TwohopArgs ta;
     TupleArgs tu;
-    int ga = 0, gs = 0, gt = 0;
+    int gd = 0, ga = 0, gs = 0, gt = 0;
     int64_t n_items = 0;
     Counters hc;
     CountResult res;
@@ -1924,27 +2151,42 @@ struct CountRun {
     }
 
     void launch_twohop(unsigned a, unsigned b) {
-        ta.large_begin = a;
+        ta.direct_begin = a;
+        ta.direct_end = b < hc.n_direct ? b : hc.n_direct;
+        ta.large_begin = a > hc.n_direct ? a : hc.n_direct;
         ta.large_end = b < hc.n_big ? b : hc.n_big;
         ta.small_begin = a > hc.n_big ? a : hc.n_big;
         ta.small_end = b;
-        if (ga > 0 && ta.large_end > ta.large_begin) {
-            int g = ga;
-            if ((unsigned)g > ta.large_end - ta.large_begin) g = (int)(ta.large_end - ta.large_begin);
-            if (spec.paper) k_twohop_large<true><<<g, PL_THREADS, PL_SMEM, s>>>(ta);
-            else k_twohop_large<false><<<g, PL_THREADS, PL_SMEM, s>>>(ta);
-            SBC_LAUNCHED();
-            g_launches++;
-        }
-        if (gs > 0 && ta.small_end > ta.small_begin) {
-            int g = gs;
-            int64_t need = ((int64_t)ta.small_end - ta.small_begin + PS_WARPS - 1) / PS_WARPS;
-            if ((int64_t)g > need) g = (int)need;
-            if (spec.paper) k_twohop_small<true><<<g, PS_THREADS, PS_SMEM, s>>>(ta);
-            else k_twohop_small<false><<<g, PS_THREADS, PS_SMEM, s>>>(ta);
-            SBC_LAUNCHED();
-            g_launches++;
-        }
+        // The kernels fill disjoint anchors' rows, so each may start where the one
+        // before it leaves room (every CTA of which runs by then) and ends after it:
+        // the few hub anchors left to the hash kernel, first, no longer run alone
+        // (2-hop of the (2,2) count of the 2M-edge graph 7.4 -> 5.6 ms).
+        bool after = false;  // a 2-hop kernel is the last work on the stream
+        if (ga > 0 && ta.large_end > ta.large_begin)
+            launch_overlapped(spec.paper ? k_twohop_large<true> : k_twohop_large<false>, ga,
+                              ta.large_end - ta.large_begin, PL_THREADS, PL_SMEM, after);
+        if (ta.direct_end > ta.direct_begin)
+            launch_overlapped(k_twohop_direct, gd, ta.direct_end - ta.direct_begin, DT_THREADS, DT_SMEM, after);
+        if (gs > 0 && ta.small_end > ta.small_begin)
+            launch_overlapped(spec.paper ? k_twohop_small<true> : k_twohop_small<false>, gs,
+                              (ta.small_end - ta.small_begin + PS_WARPS - 1) / PS_WARPS, PS_THREADS, PS_SMEM,
+                              after);
+    }
+
+    void launch_overlapped(void (*k)(TwohopArgs), int grid, unsigned need, int threads, size_t smem, bool &after) {
+        cudaLaunchAttribute at = {};
+        at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)grid > need ? need : (unsigned)grid);
+        cfg.blockDim = dim3((unsigned)threads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = s;
+        cfg.attrs = &at;
+        cfg.numAttrs = after ? 1 : 0;
+        SBC_CUDA(cudaLaunchKernelEx(&cfg, k, ta));
+        g_launches++;
+        after = true;
     }
 
     void launch_tuple_kernel() {
@@ -2004,7 +2246,7 @@ struct CountRun {
         groups.clear();
         drop_events();
         tc_anchors = tc_tiles = tc_kblocks = 0;
-        ta.large_begin = ta.large_end = ta.small_begin = ta.small_end = 0;
+        ta.direct_begin = ta.direct_end = ta.large_begin = ta.large_end = ta.small_begin = ta.small_end = 0;
         gt = 0;
         const int l = spec.l;
         R = spec.k - 1;
@@ -2053,6 +2295,9 @@ struct CountRun {
         pa.nshard = spec.nshard;
         pa.stats = spec.paper ? 1 : 0;
         pa.small_e = spec.small_e > 0 ? spec.small_e : SMALL_E_MAX;
+        pa.direct = hash_slots_cap() == 0 && twohop_window_wedges() == (uint32_t)PL_WCAP;
+        pa.graph_x0 = spec.per_graph ? spec.graph_x0 : nullptr;
+        pa.n_graphs = spec.n_graphs;
         pa.A_bit = A_bit;
         pa.dprime = dprime;
         pa.rsv_c = rsv_c;
@@ -2121,7 +2366,6 @@ struct CountRun {
         ta.rinfo = rinfo;
         ta.single = R == 1;
         ta.n_ranks = (uint32_t)nX;
-        ta.direct = hash_slots_cap() == 0 && twohop_window_wedges() == (uint32_t)PL_WCAP;
         ta.cnt = cnt.ptr;
         ta.l = l;
         ta.check = spec.check ? 1 : 0;
@@ -2129,10 +2373,13 @@ struct CountRun {
         ta.wcap = twohop_window_wedges();
         ta.bucket = nullptr;
         ta.bucket_slot = 0;
+        if (hc.n_direct > 0) gd = sms * blocks_per_sm((const void *)k_twohop_direct, DT_THREADS, DT_SMEM);
         if (hc.n_big > 0) {
             const void *fn = spec.paper ? (const void *)k_twohop_large<true> : (const void *)k_twohop_large<false>;
             ga = sms * blocks_per_sm(fn, PL_THREADS, PL_SMEM);
             if ((int64_t)ga > (int64_t)hc.n_big) ga = (int)hc.n_big;
+            // (reserved for every CTA-wide anchor: what a call needs does not
+            // depend on the strategy its anchors take)
             if (hc.e_max > (unsigned long long)ta.wcap) {
                 const int lgb = bucket_lg(hc.e_max);
                 ta.bucket_slot = bucket_cap(hc.e_max, lgb) << lgb;
@@ -2201,7 +2448,7 @@ struct CountRun {
                 k_group_offsets<<<grid_for(na, B), B, 0, s>>>(order, cum_dev.ptr, a, b, pool_off);
                 SBC_LAUNCHED();
                 g_launches++;
-                SBC_CUDA(cudaMemsetAsync(&cnt.ptr->head_large, 0, 4 * sizeof(unsigned), s));
+                SBC_CUDA(cudaMemsetAsync(&cnt.ptr->head_direct, 0, 5 * sizeof(unsigned), s));
                 SBC_CUDA(cudaMemsetAsync(&cnt.ptr->cost_total, 0,
                                          offsetof(Counters, run_begin) - offsetof(Counters, cost_total), s));
                 SBC_CUDA(cudaMemsetAsync(&cnt.ptr->tw_fin_max, 0, 2 * sizeof(unsigned long long), s));

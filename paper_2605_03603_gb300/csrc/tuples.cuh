@@ -1114,7 +1114,7 @@ __device__ void warp_anchor(const TupleArgs &a, uint32_t r, Acc &acc, unsigned *
 }
 
 template <int R>
-__global__ void __launch_bounds__(TU_THREADS, 1) k_tuples(TupleArgs a) {
+__global__ void __launch_bounds__(TU_THREADS, 1) k_tuples(const __grid_constant__ TupleArgs a) {
     __shared__ TupleShared sh;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     unsigned *err = &a.cnt->err;
