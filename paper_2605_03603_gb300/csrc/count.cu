@@ -1920,8 +1920,12 @@ constexpr unsigned long long kPosNodeCost = 3;
 // Default tuple work items per half of a resident CTA of a full launch.
 constexpr unsigned long long kSplitPerWarp = 4;
 // Two-partner anchors with at least this many mask words and candidates take
-// the tensor-core pair step.
-constexpr uint32_t kTcMinWords = 2;
+// the tensor-core pair step. A 128-position step is mostly empty for one word,
+// but a pair of rows still costs less there than in the tuple kernel: (4,3) of
+// the 500k-edge graph 5.4 + 0.8 ms (row pairs of one-word anchors + tensor
+// cores) with 2 words, 0.4 + 2.2 ms with 1; (3,3) of the 2M-edge graph
+// 2.0 + 3.1 and 0.7 + 3.6 ms.
+constexpr uint32_t kTcMinWords = 1;
 constexpr uint32_t kTcMinCandidates = 128;
 
 // Largest x with binom(x, l) computable in 64 bits by the multiplicative

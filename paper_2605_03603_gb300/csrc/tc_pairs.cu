@@ -448,7 +448,7 @@ __host__ __device__ constexpr uint32_t tc_fast_max() {
 enum : int { EPI_FLOAT = 0, EPI_INT = 1, EPI_TABLE = 2 };
 
 template <int L, int EPI>
-__global__ void __launch_bounds__(TC_THREADS, 1) k_tcpairs(TcArgs a) {
+__global__ void __launch_bounds__(TC_THREADS, 1) k_tcpairs(const __grid_constant__ TcArgs a) {
     extern __shared__ __align__(16) unsigned char tc_smem_raw[];
     __shared__ __align__(8) uint64_t full_a[TC_A], empty_a[TC_A], full_b[TC_B], empty_b[TC_B];
     __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2], mma_done;
@@ -844,7 +844,8 @@ TcPlan tc_plan(const std::vector<TcInput> &in, int l, int64_t budget_bytes) {
         const uint64_t h = (x.nr + 255) / 256;
         A.RB = (uint32_t)(2 * h);
         A.KB = (x.W + 3) / 4;
-        const uint64_t tiles = h * (h + 1);  // sum over columns J < h of 2J + 2
+        // sum over columns J < h of 2J + 2, less the last tile when it has no rows
+        const uint64_t tiles = h * (h + 1) - (((x.nr + 127) / 128) & 1);
         if (tiles > 0xFFFFFFFFull) fail(SBC_E_UNSUPPORTED, "an anchor with %u rows is too large", x.nr);
         A.tiles = (uint32_t)tiles;
         const int64_t nb = (int64_t)A.RB * A.KB;
