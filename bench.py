@@ -59,9 +59,8 @@ WORKLOAD = "plain-5M-1M-60M"
 PQ = [(3, 3)]
 # DRAM bytes (read + write) of a kernel's launches in one step of a workload
 # (the same unit as the kernel's `achieved`), from one ncu capture of the
-# current kernels; None where not captured. k_twohop: its two CTA-tier
-# launches of the (3,3) count.
-TRAFFIC = {("k_twohop", "plain-5M-1M-60M"): 279_530_419_712}
+# current kernels; None where not captured.
+TRAFFIC = {}
 
 
 def _dist():
@@ -631,7 +630,7 @@ def run_ours(args):
     # index of every anchor-side edge (12 B per edge)
     hop_bytes = sum(4 * s["wedges"] + 12 * g.m for s in s_first)
     hop_gbs = hop_bytes / (t_hop / 1000.0) / 1e9
-    roofs["k_twohop"] = {"kernel": "k_twohop_large + k_twohop_small (2-hop candidates)",
+    roofs["k_twohop"] = {"kernel": "k_twohop_direct + k_twohop_large + k_twohop_small (2-hop candidates)",
                          "bound": "hbm", "achieved": hop_gbs, "peak": peaks["hbm_gbs"],
                          "unit": "GB/s", "frac": hop_gbs / peaks["hbm_gbs"], "ms": t_hop,
                          "traffic": TRAFFIC.get(("k_twohop", WORKLOAD)),
