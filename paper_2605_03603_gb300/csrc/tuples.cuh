@@ -15,14 +15,15 @@
 // * rows (1): the rows are taken in ascending popcount; for every first row a
 //   the later rows that share at least l positions with it are listed and
 //   projected onto a's positions, so the remaining levels run on
-//   ceil(|a| / 32) words (one, for most rows) instead of W. Bound by POPC, a
-//   quarter of a warp per cycle and scheduler.
+//   ceil(|a| / 32) words (one, for most rows) instead of W. Bound by the latency
+//   of AND, POPC and table lookup with four warps per scheduler (POPC pipe 22 to
+//   40 % busy).
 // * column masks (2): for dense rows and few positions, a warp walks the
 //   position subsets depth first over the bitmaps "rows that hold position q",
 //   dropping prefixes contained in fewer than R rows.
 // (Counting every row's l-subsets of positions in shared-memory counters, the
 // third way to evaluate (2), was measured on the 2M-edge graph: (4,4) 231 ms
-// against 118 for the rows, (3,3) 3.2 against 1.7; the counters of a window are
+// against 107 for the rows, (3,3) 3.2 against 1.7; the counters of a window are
 // too sparse to pay for clearing them.)
 #pragma once
 
@@ -416,8 +417,10 @@ __device__ void expand(PrefixBuf<WN> &pb, const uint32_t (&pre)[WN], uint32_t st
 // All pairs of a list's entries (three rows in all) in tiles: a lane keeps
 // four entries, entries b are read once for them (four at a time when W is 1).
 // Blocks of 128 entries c0 = first, first + step, ... as the later entry. Used
-// while every count is at most s_max32. Bound by POPC (one per pair and word,
-// a quarter of a warp per cycle and scheduler).
+// while every count is at most s_max32. A pair costs an AND and a POPC per word
+// (half a warp per cycle and SM) and a table lookup. Taking the counts from the
+// warp matrix instruction instead (bits as fp16 or fp8, the same lookups) was
+// slower: (4,4) of the 2M-edge graph 137 and 153 against 105 ms.
 template <int WN>
 __device__ __forceinline__ void list_pairs_tiled(uint32_t off, uint32_t m, uint32_t ms, uint32_t first,
                                                  uint32_t step, Acc &acc) {
