@@ -737,11 +737,13 @@ __device__ __forceinline__ void first_row(const RowsV<ST> &v, uint32_t a, int l,
         if (!fits) {
             // (row_units leaves room for every warp's entry)
             if (lane == 0) sh.defer[atomicAdd(&sh.ndefer, 1u)] = a;
+            __syncwarp();
             return;
         }
         if (m < (uint32_t)(R - 1)) return;
         if (R > 3 && m >= CTA_LIST) {
             if (lane == 0) sh.defer[atomicAdd(&sh.ndefer, 1u)] = a;
+            __syncwarp();
             return;
         }
         const uint32_t ms = (m + 3) & ~3u;
@@ -828,9 +830,16 @@ __device__ void row_units(const RowsV<ST> &v, uint32_t n_first, unsigned *claim,
         __syncthreads();
         bool more = false;
         for (;;) {
-            if (R > 2 && *(volatile unsigned *)&sh.ndefer > DEFER_MAX - TU_WARPS * BATCH) {
-                more = true;
-                break;
+            if constexpr (R > 2) {
+                // other warps add to the counter meanwhile: one lane reads it, so
+                // that the warp leaves the loop together
+                unsigned nd = 0;
+                if (lane == 0) nd = *(volatile unsigned *)&sh.ndefer;
+                nd = __shfl_sync(FULL, nd, 0);
+                if (nd > DEFER_MAX - TU_WARPS * BATCH) {
+                    more = true;
+                    break;
+                }
             }
             unsigned u = 0;
             if (lane == 0) u = atomicAdd(claim, BATCH);
