@@ -688,7 +688,7 @@ __device__ __forceinline__ void add_totals(const Totals &t, uint32_t r, const U1
 }
 
 // What the tuple step's plan wants to know about an anchor's rows: positions
-// of all of them, and of the longest.
+// of all of them, and of the longest (after it: the plan, see AnchorPlan).
 struct RowInfo {
     float pops = 0;
     uint32_t longest = 0;

@@ -73,7 +73,7 @@ constexpr int SCRATCH_SLOTS = 7;                  // per-warp prefix masks of th
 
 struct ItemArgs {
     const uint32_t *ncand, *npaper, *nrow, *dprime;
-    const RowInfo *rinfo;    // per anchor, set when it has rows
+    RowInfo *rinfo;          // per anchor, set when it has rows; k_anchor_cost leaves its plan here
     const uint32_t *order;   // anchors of the group: order[begin .. begin + nX)
     int64_t begin;
     int64_t nX;              // anchors in the group
@@ -109,9 +109,15 @@ __device__ __forceinline__ float rows_cost(float n, float dp, float pops, int R,
     return c;
 }
 
+// An anchor's path, and the cost of its items (row and column paths). Kept in its
+// RowInfo (the cost in place of the positions, the path above the longest row) from
+// k_anchor_cost on, so that the items are made of the very costs that were totalled:
+// the room for them rests on that.
+enum : uint32_t { PATH_NONE = 0, PATH_TC = 1, PATH_WARP = 2, PATH_ROWS = 3, PATH_COLS = 4 };
+constexpr int PATH_SHIFT = 28;  // (rows have fewer than 2^21 positions)
 struct AnchorPlan {
-    float cost = 0;          // of the items
-    bool tc = false, warp = false, rows = false, cols = false;
+    float cost = 0;
+    uint32_t path = PATH_NONE;
 };
 
 // Which path(s) an anchor's tuples take.
@@ -139,23 +145,23 @@ __device__ __forceinline__ AnchorPlan plan_anchor(const ItemArgs &a, uint32_t r)
             cc = nodes * CW_NODE * a.pos_unit * (float)((wc + 31) / 32);
         }
         if (cc < 3.0e38f && (a.method == 2 || cc < alt)) {
-            p.cols = true;
+            p.path = PATH_COLS;
             p.cost = cc;
             return p;
         }
     }
     if (tc_ok) {
-        p.tc = true;
+        p.path = PATH_TC;
     } else if (n * W <= WG_WORDS && n <= WG_ROWS && W <= 4 && rc <= 65536.0f) {
-        p.warp = true;
+        p.path = PATH_WARP;
     } else {
-        p.rows = true;
+        p.path = PATH_ROWS;
         p.cost = rc;
     }
     return p;
 }
 
-// Reported tuple counts, and the cost total that sizes the work items.
+// Reported tuple counts, every anchor's plan, and the cost total that sizes the work items.
 __global__ void k_anchor_cost(ItemArgs a) {
     U128 tp, to;
     unsigned long long cand = 0;
@@ -186,7 +192,12 @@ __global__ void k_anchor_cost(ItemArgs a) {
             cand += nc;
         }
         if (nc >= (uint32_t)a.R) to.add(binom_sat(nc, a.R));
-        cost += (double)plan_anchor(a, r).cost;
+        if (a.R > 1) {
+            const AnchorPlan p = plan_anchor(a, r);
+            a.rinfo[r].pops = p.cost;
+            a.rinfo[r].longest |= p.path << PATH_SHIFT;
+            cost += (double)p.cost;
+        }
     }
     tp = warp_sum_u128(tp, nullptr);
     to = warp_sum_u128(to, nullptr);
@@ -206,33 +217,36 @@ __global__ void k_anchor_cost(ItemArgs a) {
 // Work items, warp list and tensor-core list of every anchor. An anchor's items
 // depend on its sizes and the cost total only (a few operations per anchor: how
 // its first rows are shared among its items is settled while they run). The
-// items beyond one per anchor sum to at most items_per_launch.
+// items beyond one per anchor sum to at most items_per_launch: an anchor of
+// several has at most cost / item_cost of them, the costs sum to cost_total, and the
+// roundings (2^-22 of the sum together) cannot make another whole item.
 __global__ void k_items(ItemArgs a) {
     const float item_cost = fmaxf((float)(a.cnt->cost_total / (double)a.items_per_launch), 16384.0f);
     for (int64_t ix = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; ix < a.nX;
          ix += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t r = a.order[a.begin + ix];
-        const AnchorPlan p = plan_anchor(a, r);
-        if (p.tc) {
+        const RowInfo info = a.rinfo[r];
+        const uint32_t path = info.longest >> PATH_SHIFT;
+        if (path == PATH_TC) {
             TcInput t;
             t.r = r;
             t.nr = a.nrow[r];
             t.W = (a.dprime[r] + 31) / 32;
             t.rsv = a.rsv_c[r];
-            t.longest = a.rinfo[r].longest;
+            t.longest = info.longest & ((1u << PATH_SHIFT) - 1u);
             t.pool_off = a.pool_off[r];
             a.tc_in[atomicAdd(&a.cnt->n_tc, 1u)] = t;
-        } else if (p.warp) {
+        } else if (path == PATH_WARP) {
             a.warp_list[atomicAdd(&a.cnt->n_warp, 1u)] = r;
-        } else if (p.rows || p.cols) {
-            const uint32_t total = (uint32_t)fminf(fmaxf(p.cost / item_cost, 1.0f), 1024.0f);
+        } else if (path != PATH_NONE) {
+            const uint32_t total = (uint32_t)fminf(fmaxf(info.pops / item_cost, 1.0f), 1024.0f);
             const unsigned k0 = atomicAdd(&a.cnt->n_items, total);
             const unsigned claim = total > 1 ? atomicAdd(&a.cnt->n_claims, 1u) : NO_CLAIM;
             for (uint32_t i = 0; i < total; i++) {
                 Item it;
                 it.anchor = r;
                 it.claim = claim;
-                it.cols = p.cols;
+                it.cols = path == PATH_COLS;
                 a.items[k0 + i] = it;
             }
         }

@@ -43,3 +43,22 @@ def test_deferred_rows(sbc, m):
                                        tune={"split_per_warp": 1})
     assert got == 6 * comb(m, 5) * comb(8, 2)
     assert sorted(per) == sorted(comb(r, 4) * comb(8, 2) for r in range(m) for _ in range(6))
+
+
+@pytest.mark.parametrize("split", [1, 4, 64])
+@pytest.mark.parametrize("p,q", [(3, 3), (4, 4), (5, 5)])
+@pytest.mark.parametrize("method", ["auto", "candidate", "position"])
+def test_work_items_within_their_room(sbc, split, p, q, method):
+    """One item per anchor and at most 2 x SMs x split_per_warp more, whichever
+    path an anchor's plan names; the count is the same for every split."""
+    import torch
+
+    g = sbc_synth.plain_small()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    with sbc.graph_from_synth(g) as h:
+        want = sbc.sbc_count(h, p, q)
+        for tc in (-1, 1):
+            got, st, _ = sbc.sbc_count_ex(h, p, q, anchor_side=0, method=method,
+                                          tune={"split_per_warp": split, "tc_min_words": tc})
+            assert got == want
+            assert st["work_items"] + st["tc_anchors"] <= g.n_u + 2 * sms * split
