@@ -442,7 +442,9 @@ uint64_t sbc_launch_count(void);
 /*
  * Route the library's device allocations through caller functions (for
  * example a framework's caching allocator). alloc returns a device pointer of
- * at least `bytes` bytes usable on `stream`, or NULL; free releases it.
+ * at least `bytes` bytes usable on `stream`, or NULL; free releases it. The
+ * *_destroy calls wait for the device and free on the default stream (NULL),
+ * since the stream a block came from may be gone by then.
  * Passing NULL functions restores cudaMallocAsync / cudaFreeAsync.
  */
 typedef void *(*sbc_alloc_fn)(size_t bytes, void *stream, void *ctx);

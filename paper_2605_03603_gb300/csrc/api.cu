@@ -12,6 +12,7 @@ std::atomic<int64_t> g_launches{0};
 namespace {
 thread_local std::string t_err;
 thread_local Arena *t_arena = nullptr;
+thread_local const cudaStream_t *t_free_stream = nullptr;  // of the innermost FreeOnStream
 sbc_alloc_fn g_alloc = nullptr;
 sbc_free_fn g_free = nullptr;
 void *g_alloc_ctx = nullptr;
@@ -30,6 +31,8 @@ void fail(sbc_status s, const char *fmt, ...) {
 
 void set_thread_arena(Arena *a) { t_arena = a; }
 bool thread_arena_active() { return t_arena != nullptr; }
+FreeOnStream::FreeOnStream(cudaStream_t s) : stream(s), outer(t_free_stream) { t_free_stream = &stream; }
+FreeOnStream::~FreeOnStream() { t_free_stream = outer; }
 
 void *dev_alloc(size_t bytes, cudaStream_t s) {
     void *p = nullptr;
@@ -65,6 +68,7 @@ void dev_free(void *p, size_t bytes, cudaStream_t s) {
         if ((char *)p + need == t_arena->base + t_arena->top) t_arena->top -= need;
         return;
     }
+    if (t_free_stream) s = *t_free_stream;
     if (g_free) {
         g_free(p, bytes, (void *)s, g_alloc_ctx);
         return;
@@ -139,7 +143,10 @@ sbc_status sbc_graph_destroy(sbc_graph *g) {
     cudaGetDevice(&cur);
     if (cur != dev) cudaSetDevice(dev);
     cudaDeviceSynchronize();
-    delete g;
+    {
+        FreeOnStream frees(nullptr);
+        delete g;
+    }
     if (cur != dev) cudaSetDevice(cur);
     SBC_API_END
 }

@@ -503,8 +503,16 @@ sbc_status sbc_batch_run(sbc_batch *b, sbc_u128 *out, void *stream) {
 sbc_status sbc_batch_destroy(sbc_batch *b) {
     SBC_BATCH_TRY
     if (!b) return SBC_OK;
+    int cur = 0;
+    const int dev = b->device;
+    cudaGetDevice(&cur);
+    if (cur != dev) cudaSetDevice(dev);
     cudaDeviceSynchronize();
-    delete b;
+    {
+        FreeOnStream frees(nullptr);
+        delete b;
+    }
+    if (cur != dev) cudaSetDevice(cur);
     SBC_BATCH_END
 }
 

@@ -2245,6 +2245,7 @@ struct CountRun {
     // its 2-hop kernels, item planning, tuple kernel and tensor-core step.
     void plan_and_run(EventTimer *tm) {
         NvtxRange nr("sbc/count");
+        FreeOnStream frees(s);  // (a plan made again drops the one before it)
         const bool timing = tm != nullptr;
         const int B = 256;
         groups.clear();
@@ -2611,7 +2612,14 @@ void countrun_launch(CountRun *r, cudaStream_t s) {
             fail(SBC_E_UNSUPPORTED, "a count planned in %zu anchor groups cannot be captured",
                  r->groups.size());
         }
-        r->plan_and_run(nullptr);
+        try {
+            r->plan_and_run(nullptr);
+        } catch (...) {
+            // the blocks stay with the plan and may next be freed on another stream
+            (void)cudaStreamSynchronize(s);
+            r->s = keep;
+            throw;
+        }
     } else {
         r->launch_count();
     }

@@ -190,11 +190,8 @@ uint32_t read_err(uint32_t *d_err, cudaStream_t s) {
     return h;
 }
 
-}  // namespace
-
-void build_orientation(sbc_graph *g, int x, cudaStream_t s) {
+void orient_side(sbc_graph *g, int x, cudaStream_t s) {
     Orient &o = g->side[x];
-    if (o.built) return;
     const int64_t nnz = g->nnz;
     const int x_is_v = x == 1;
     o.nX = x_is_v ? g->n_v : g->n_u;
@@ -274,12 +271,20 @@ void build_orientation(sbc_graph *g, int x, cudaStream_t s) {
     o.built = true;
 }
 
-}  // namespace sbc
+}  // namespace
 
-
-
-
-namespace sbc {
+void build_orientation(sbc_graph *g, int x, cudaStream_t s) {
+    Orient &o = g->side[x];
+    if (o.built) return;
+    try {
+        orient_side(g, x, s);
+    } catch (...) {
+        // nothing is left behind: a later call could only free it on this
+        // call's stream, which may be gone by then
+        o = Orient();
+        throw;
+    }
+}
 
 // Upload, validate and prepare a graph; builds the orientation of the side
 // the cost model prefers (which also checks for duplicate edges).

@@ -55,6 +55,22 @@ struct NvtxRange {
 void *dev_alloc(size_t bytes, cudaStream_t s);
 void dev_free(void *p, size_t bytes, cudaStream_t s);
 
+// While one lives on the calling thread, dev_free frees on `s` whatever stream
+// the block came from: that one may be gone (a server's lane, a stream of the
+// caller's). For the calls that drop blocks of earlier calls, which all
+// waited for their streams: a plan made again on its own stream, and the destroy
+// calls, on the default stream once the device is idle.
+struct FreeOnStream {
+    explicit FreeOnStream(cudaStream_t s);
+    ~FreeOnStream();
+    FreeOnStream(const FreeOnStream &) = delete;
+    FreeOnStream &operator=(const FreeOnStream &) = delete;
+
+  private:
+    cudaStream_t stream;
+    const cudaStream_t *outer;
+};
+
 // A caller-provided region of device memory that dev_alloc carves from (a
 // stack: blocks freed in reverse order are reclaimed) while it is installed on
 // the calling thread with set_thread_arena. Only the no-allocation entry point
