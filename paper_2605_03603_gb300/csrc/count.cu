@@ -2206,6 +2206,7 @@ struct CountRun {
     }
 
     std::vector<std::pair<int64_t, int64_t>> groups;  // ranges of the sorted anchors
+    bool several = false;      // more than one (kept while a new plan is made, which may fail)
     int64_t words_big = 0, words_small = 0;  // pool words of the two 2-hop tiers
     std::vector<int64_t> cum;  // several groups: pool words before each ordered anchor
     float tw_tail_ms = 0;      // largest finish spread of the CTA-wide 2-hop kernel's CTAs
@@ -2349,6 +2350,7 @@ struct CountRun {
             }
             cum_dev = std::move(dcum);
         }
+        several = groups.size() > 1;
         pool.alloc((size_t)std::max<int64_t>(most, 1), s);
         const int sms = sm_count();
 
@@ -2603,7 +2605,7 @@ void countrun_launch(CountRun *r, cudaStream_t s) {
     }
     cudaStream_t keep = r->s;
     r->s = s;
-    if (r->groups.size() > 1) {
+    if (r->several) {
         // a multi-group plan re-plans (host reads between groups)
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
         SBC_CUDA(cudaStreamIsCapturing(s, &cs));
@@ -2626,7 +2628,7 @@ void countrun_launch(CountRun *r, cudaStream_t s) {
     r->s = keep;
 }
 
-bool countrun_replayable(const CountRun *r) { return r->groups.size() <= 1; }
+bool countrun_replayable(const CountRun *r) { return !r->several; }
 
 void countrun_collect(CountRun *r, cudaStream_t s) {
     if (r->nnz == 0 || r->nX == 0) return;

@@ -30,16 +30,21 @@ def sbc():
 
 class RecordingAllocator:
     """Device memory from torch through the allocator hook; `frees` lists the
-    streams the library freed on (0: the default stream)."""
+    streams the library freed on (0: the default stream). The block numbered
+    `fail_at` (1-based, counted in `calls`) is refused."""
 
-    def __init__(self, sbc):
+    def __init__(self, sbc, fail_at=0):
         import torch
 
         self.torch, self.sbc = torch, sbc
         self.live, self.frees = {}, []
+        self.fail_at, self.calls = fail_at, 0
         self._a, self._f = ALLOC_FN(self._alloc), FREE_FN(self._free)
 
     def _alloc(self, nbytes, stream, ctx):
+        self.calls += 1
+        if self.calls == self.fail_at:
+            return None
         p = self.torch.cuda.caching_allocator_alloc(max(int(nbytes), 1))
         self.live[p] = stream or 0
         return p
@@ -123,18 +128,28 @@ def test_failed_orientation_leaves_nothing(sbc):
     for k in range(1, 20):
         with sbc.graph_from_synth(g) as h:
             held = sbc.sbc_graph_info(h)["device_bytes"]
-            with RecordingAllocator(sbc) as a:
-                alloc, calls = a._alloc, [0]
-
-                def dry(nbytes, stream, ctx):
-                    calls[0] += 1
-                    return None if calls[0] == k else alloc(nbytes, stream, ctx)
-
-                a._a = ALLOC_FN(dry)
-                a.__enter__()
+            with RecordingAllocator(sbc, fail_at=k) as a:
                 with pytest.raises(sbc.SbcError) as e:
                     sbc.sbc_count(h, 3, 4)
                 assert e.value.status == 3  # SBC_E_NOMEM
                 assert not a.live
             assert sbc.sbc_graph_info(h)["device_bytes"] == held
             assert sbc.sbc_count(h, 3, 4) == want
+
+
+def test_batch_counts_again_after_a_failed_run(sbc, monkeypatch):
+    """A run of a batch of several anchor groups plans again; when that runs out
+    of memory at its k-th block, the next run is exact."""
+    g = two_sided()
+    want = oracle.count(g, 3, 3, side=0)
+    monkeypatch.setenv("SBC_POOL_BUDGET_KB", "4")
+    with RecordingAllocator(sbc) as a:
+        with sbc.graph_from_synth(g) as h, sbc.Batch([h], 3, 3) as b:
+            for k in range(1, 12):
+                a.calls, a.fail_at = 0, k
+                with pytest.raises(sbc.SbcError) as e:
+                    b.run()
+                assert e.value.status == 3  # SBC_E_NOMEM
+                a.fail_at = 0
+                assert b.run() == [want]
+        assert not a.live
