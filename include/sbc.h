@@ -130,11 +130,11 @@ sbc_status sbc_graph_info(const sbc_graph *g, sbc_graph_info_t *out);
 #define SBC_COUNT_CANDIDATE_SIDE (1 << 1) /* enumerate candidate subsets for every anchor */
 #define SBC_COUNT_POSITION_SIDE (1 << 2)  /* enumerate position subsets wherever they fit
                                              (default: the cheaper side per anchor) */
-#define SBC_COUNT_CHECK (1 << 3) /* device self-checks: after the 2-hop step every kept
-                                    candidate's mask popcounts are compared with the
-                                    counters of its hash-table entry; a mismatch gives
-                                    SBC_E_CUDA. Also enabled for every count by the
-                                    environment variable SBC_DEBUG=1. Slower. */
+#define SBC_COUNT_CHECK (1 << 3) /* device self-checks: in the 2-hop step the mask popcounts
+                                    of every kept candidate's parts are compared with its
+                                    counters; a mismatch gives SBC_E_CUDA. Also enabled
+                                    for every count by the environment variable
+                                    SBC_DEBUG=1. Slower. */
 
 /*
  * Launch parameters of the counting kernels: the search space of the
@@ -199,7 +199,8 @@ typedef struct {
     uint64_t tuples_tested; /* tuples whose common-neighbour mask was tested (after
                                nested pruning) */
     uint64_t tuples_typed;  /* tuples with at least q common neighbours (type counts taken) */
-    uint64_t popc_words;    /* mask words popcounted by the tuple kernel */
+    uint64_t popc_words;    /* mask words popcounted by the tuple kernel (and, where they
+                               are on, by the self-checks) */
     int32_t anchor_side;    /* side used */
     int32_t kernels;        /* kernel launches issued by the call */
     float ms_prepare;       /* orientation build (first use of a side) + plan */

@@ -67,7 +67,7 @@ struct Counters {
     unsigned long long wedges;         // 2-hop entries visited
     unsigned long long tested;         // tuples whose common-neighbour mask was tested
     unsigned long long leaves;         // tuples with |T| >= l (type counts taken)
-    unsigned long long popc_words;     // mask words popcounted by the tuple kernel
+    unsigned long long popc_words;     // mask words popcounted by the tuple kernel and the self-checks
     // CTA-wide 2-hop kernel, by strategy (one window, bucketed, re-read windows,
     // bucketed with a second scatter)
     unsigned long long tw_reads;       // 2-hop entries read, all passes
@@ -645,9 +645,8 @@ __device__ __forceinline__ uint32_t row_index(unsigned long long v, uint32_t sdi
 }
 
 // Self-check of one row after its mask is written: its popcount must equal
-// the positions the hash table counted in the first pass. Consecutive words
-// are `stride` apart. Reads of global rows bypass L1 (the words were written
-// by atomics at L2).
+// the positions its counter holds. Consecutive words are `stride` apart. Reads
+// of global rows bypass L1 (the words were written by atomics at L2).
 __device__ __forceinline__ bool row_matches(const uint32_t *row, size_t stride, uint32_t W, uint32_t want,
                                             bool global) {
     uint32_t n = 0;
@@ -655,8 +654,9 @@ __device__ __forceinline__ bool row_matches(const uint32_t *row, size_t stride, 
     return n == want;
 }
 __device__ __forceinline__ bool rows_match(const uint32_t *rows, size_t stride, uint32_t W,
-                                           unsigned long long v, int l, bool global) {
+                                           unsigned long long v, int l, bool global, unsigned long long &words) {
     const uint32_t s = row_index(v, 0, l), d = row_index(v, 1, l);
+    words += (unsigned long long)W * ((s != EMPTY) + (d != EMPTY));
     return (s == EMPTY || row_matches(rows + s, stride, W, use_count(v) - diff_count(v), global)) &&
            (d == EMPTY || row_matches(rows + d, stride, W, diff_count(v), global));
 }
@@ -904,11 +904,13 @@ __global__ void __launch_bounds__(PS_THREADS) k_twohop_small(const __grid_consta
                 if (a.check) {
                     __syncwarp();
                     bool bad = false;
+                    unsigned long long words = 0;
                     for (uint32_t i = lane; i < hs; i += 32) {
                         if (keys[i] == EMPTY) continue;
                         unsigned long long v = vals[i];
-                        if ((v & CAND) && !rows_match(region, rsv, W, v, l, true)) bad = true;
+                        if ((v & CAND) && !rows_match(region, rsv, W, v, l, true, words)) bad = true;
                     }
+                    if (words) atomicAdd(&a.cnt->popc_words, words);
                     if (__any_sync(FULL, bad) && lane == 0) atomicOr(&a.cnt->err, CERR_MASK);
                 }
             }
@@ -1153,7 +1155,14 @@ __device__ __forceinline__ uint32_t part_bit(uint32_t idx, uint32_t sdiff) {
     else return (sdiff << 4) + (idx & 15u);
 }
 
+// Count of the part at bit k of bitmap word j (the counters' memory as bytes).
 template <bool C8>
+__device__ __forceinline__ uint32_t part_count(const unsigned char *tbl, uint32_t j, uint32_t k) {
+    if constexpr (C8) return tbl[32 * j + 4 * (k & 7u) + (k >> 3)];
+    else return reinterpret_cast<const uint16_t *>(tbl)[32 * j + 2 * (k & 15u) + (k >> 4)];
+}
+
+template <bool C8, bool CHECK>
 __device__ __forceinline__ DirectOut direct_anchor(const TwohopArgs &a, uint32_t r, uint32_t range,
                                                 unsigned char *smem, unsigned long long *warp_tot,
                                                 unsigned *s_nrw, unsigned *s_ncw) {
@@ -1231,9 +1240,20 @@ __device__ __forceinline__ DirectOut direct_anchor(const TwohopArgs &a, uint32_t
     for (uint32_t w0 = 0; w0 < range; w0 += CELLS) {
         const uint32_t base = r + 1 + w0, nw = range - w0 < CELLS ? range - w0 : CELLS;
         const uint32_t nbm = (nw + 15) / 16;
+        auto clear = [&]() {
+            for (uint32_t i = tid; i < nbm * (C8 ? 2u : 4u); i += DT_THREADS)
+                reinterpret_cast<uint4 *>(tbl)[i] = make_uint4(0, 0, 0, 0);
+        };
+        auto count = [&](uint32_t ent, uint32_t inf) {
+            const uint32_t idx = (ent & VMASK) - base;
+            if (idx < nw) {
+                const uint32_t sdiff = (ent ^ inf) >> 31;
+                if constexpr (C8) atomicAdd(&tbl[idx >> 1], 1u << ((idx & 1u) * 16u + sdiff * 8u));
+                else atomicAdd(&tbl[idx], sdiff ? 65536u : 1u);
+            }
+        };
         // counts
-        for (uint32_t i = tid; i < nbm * (C8 ? 2u : 4u); i += DT_THREADS)
-            reinterpret_cast<uint4 *>(tbl)[i] = make_uint4(0, 0, 0, 0);
+        clear();
         if (one) {
             uint32_t cut = en;
             if (w0 + CELLS < range && info != EMPTY) {  // first entry past the window
@@ -1256,16 +1276,8 @@ __device__ __forceinline__ DirectOut direct_anchor(const TwohopArgs &a, uint32_t
         }
         __syncthreads();
         const uint32_t nr0 = *s_nrw;
-        visit(0, dp, [&](uint32_t ent, uint32_t inf) {
-            const uint32_t idx = (ent & VMASK) - base;
-            if (idx < nw) {
-                const uint32_t sdiff = (ent ^ inf) >> 31;
-                if constexpr (C8) atomicAdd(&tbl[idx >> 1], 1u << ((idx & 1u) * 16u + sdiff * 8u));
-                else atomicAdd(&tbl[idx], sdiff ? 65536u : 1u);
-            }
-        });
+        visit(0, dp, count);
         out.passes++;
-        long long check = 0;  // self-check: bits written minus bits counted
         // rows: a bit per rank and part (part_bit)
         uint32_t all = 0;     // OR (8-bit) or maximum (16-bit) of the counters: bounds the longest row
         for (uint32_t j0 = 0; j0 < nbm; j0 += DT_THREADS) {
@@ -1319,15 +1331,12 @@ __device__ __forceinline__ DirectOut direct_anchor(const TwohopArgs &a, uint32_t
                 }
                 at = __shfl_sync(FULL, at, 31) + incl - cnt;
                 if (j < nbm) pre[j] = at;
-                if (a.single || a.check) {
+                if (a.single) {
                     uint32_t b = bits;
                     while (b) {
                         const uint32_t k = __ffs(b) - 1;
                         b &= b - 1;
-                        const uint32_t x = C8 ? (uint32_t)smem[32 * j + 4 * (k & 7u) + (k >> 3)]
-                                              : (uint32_t)((uint16_t *)smem)[32 * j + 2 * (k & 15u) + (k >> 4)];
-                        if (a.single) binom_add(out.sum, x, l, &a.cnt->err);
-                        check -= x;
+                        binom_add(out.sum, part_count<C8>(smem, j, k), l, &a.cnt->err);
                     }
                 }
             }
@@ -1386,21 +1395,34 @@ __device__ __forceinline__ DirectOut direct_anchor(const TwohopArgs &a, uint32_t
                         region[(size_t)(wa + wd) * rsv + nr0 + (i - wd * nrw)] = tbl[i];
                     }
                 }
-                if (a.check)
-                    for (uint32_t i = tid; i < wn * nrw; i += DT_THREADS) check += __popc(tbl[i]);
                 __syncthreads();
             }
         }
         out.rst.pops += (float)hits;
         out.passes++;
-        if (a.check && staged) {
-            // self-check: the window's rows hold as many bits as its counters say
-            unsigned long long *scr = (unsigned long long *)(smem + DT_OFF_BM);  // (free now)
-            if (tid == 0) *scr = 0;
+        if constexpr (CHECK) {
+            // self-check: the staged words took the counters' memory, so the window
+            // is counted once more; the parts with at least l positions must be
+            // the rows numbered above, and every row must hold its part's count
+            clear();
             __syncthreads();
-            atomicAdd(scr, (unsigned long long)check);
-            __syncthreads();
-            if (tid == 0 && *scr != 0) atomicOr(&a.cnt->err, CERR_MASK);
+            visit(0, dp, count);
+            out.passes++;
+            bool bad = false;
+            unsigned long long words = 0;
+            for (uint32_t j = tid; j < nbm; j += DT_THREADS) {
+                const uint32_t bits = bm[j];
+                for (uint32_t k = 0; k < 32; k++) {
+                    const uint32_t x = part_count<C8>(smem, j, k);
+                    const bool row = (bits >> k) & 1u;
+                    bad |= row != (x >= (uint32_t)l);
+                    if (!row) continue;
+                    bad |= !row_matches(region + pre[j] + __popc(bits & ((1u << k) - 1u)), rsv, W, x, true);
+                    words += W;
+                }
+            }
+            if (words) atomicAdd(&a.cnt->popc_words, words);
+            if (bad) atomicOr(&a.cnt->err, CERR_MASK);
             __syncthreads();
         }
     }
@@ -1416,7 +1438,9 @@ __device__ __forceinline__ unsigned long long global_ns() {
     return t;
 }
 
-// Direct counters, one CTA per anchor.
+// Direct counters, one CTA per anchor. (The self-check is a build of its own: its
+// registers would cost the other one occupancy or spills.)
+template <bool CHECK>
 __global__ void __launch_bounds__(DT_THREADS, 2) k_twohop_direct(const __grid_constant__ TwohopArgs a) {
     twohop_let_next_start();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1448,8 +1472,9 @@ __global__ void __launch_bounds__(DT_THREADS, 2) k_twohop_direct(const __grid_co
             s_longest = 0;
         }
         __syncthreads();
-        DirectOut o = a.dprime[r] <= 255u ? direct_anchor<true>(a, r, s_range, smem_raw, warp_tot, &s_nrw, &s_ncw)
-                                          : direct_anchor<false>(a, r, s_range, smem_raw, warp_tot, &s_nrw, &s_ncw);
+        DirectOut o = a.dprime[r] <= 255u
+            ? direct_anchor<true, CHECK>(a, r, s_range, smem_raw, warp_tot, &s_nrw, &s_ncw)
+            : direct_anchor<false, CHECK>(a, r, s_range, smem_raw, warp_tot, &s_nrw, &s_ncw);
         if (o.failed) o.nc = o.nr = 0;
         if (a.single) {
             if (sum.add(o.sum)) atomicOr(&a.cnt->err, CERR_OVERFLOW);
@@ -1632,11 +1657,13 @@ __global__ void __launch_bounds__(PL_THREADS, 2) k_twohop_large(const __grid_con
                 __syncthreads();
                 if (a.check) {
                     bool bad = false;
+                    unsigned long long words = 0;
                     for (uint32_t i = tid; i < hs; i += PL_THREADS) {
                         if (keys[i] == EMPTY) continue;
                         const unsigned long long v = vals[i];
-                        if ((v & CAND) && !rows_match(bb, bstride, W, v, l, !staged)) bad = true;
+                        if ((v & CAND) && !rows_match(bb, bstride, W, v, l, !staged, words)) bad = true;
                     }
+                    if (words) atomicAdd(&a.cnt->popc_words, words);
                     if (bad) atomicOr(&a.cnt->err, CERR_MASK);
                     __syncthreads();
                 }
@@ -1983,7 +2010,8 @@ void ensure_kernel_attrs() {
     SBC_CUDA(cudaMemcpyToSymbol(c_binom64_max, lim, sizeof(lim)));
     SBC_CUDA(cudaFuncSetAttribute(k_twohop_small<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PS_SMEM));
     SBC_CUDA(cudaFuncSetAttribute(k_twohop_small<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PS_SMEM));
-    SBC_CUDA(cudaFuncSetAttribute(k_twohop_direct, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DT_SMEM));
+    SBC_CUDA(cudaFuncSetAttribute(k_twohop_direct<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DT_SMEM));
+    SBC_CUDA(cudaFuncSetAttribute(k_twohop_direct<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DT_SMEM));
     SBC_CUDA(cudaFuncSetAttribute(k_twohop_large<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PL_SMEM));
     SBC_CUDA(cudaFuncSetAttribute(k_twohop_large<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PL_SMEM));
     tc_ensure_attrs();
@@ -2170,7 +2198,7 @@ struct CountRun {
             launch_overlapped(spec.paper ? k_twohop_large<true> : k_twohop_large<false>, ga,
                               ta.large_end - ta.large_begin, PL_THREADS, PL_SMEM, after);
         if (ta.direct_end > ta.direct_begin)
-            launch_overlapped(k_twohop_direct, gd, ta.direct_end - ta.direct_begin, DT_THREADS, DT_SMEM, after);
+            launch_overlapped(spec.check ? k_twohop_direct<true> : k_twohop_direct<false>, gd, ta.direct_end - ta.direct_begin, DT_THREADS, DT_SMEM, after);
         if (gs > 0 && ta.small_end > ta.small_begin)
             launch_overlapped(spec.paper ? k_twohop_small<true> : k_twohop_small<false>, gs,
                               (ta.small_end - ta.small_begin + PS_WARPS - 1) / PS_WARPS, PS_THREADS, PS_SMEM,
@@ -2380,7 +2408,10 @@ struct CountRun {
         ta.wcap = twohop_window_wedges();
         ta.bucket = nullptr;
         ta.bucket_slot = 0;
-        if (hc.n_direct > 0) gd = sms * blocks_per_sm((const void *)k_twohop_direct, DT_THREADS, DT_SMEM);
+        if (hc.n_direct > 0) {
+            const void *fn = spec.check ? (const void *)k_twohop_direct<true> : (const void *)k_twohop_direct<false>;
+            gd = sms * blocks_per_sm(fn, DT_THREADS, DT_SMEM);
+        }
         if (hc.n_big > 0) {
             const void *fn = spec.paper ? (const void *)k_twohop_large<true> : (const void *)k_twohop_large<false>;
             ga = sms * blocks_per_sm(fn, PL_THREADS, PL_SMEM);
