@@ -2125,7 +2125,7 @@ struct CountRun {
         size_t fr = 0, tot = 0;
         SBC_CUDA(cudaMemGetInfo(&fr, &tot));
         int64_t b = (int64_t)(fr / 8);
-        return std::max<int64_t>(256ll << 20, std::min<int64_t>(b, 1ll << 30));
+        return std::max<int64_t>(256ll << 20, std::min<int64_t>(b, kTcArenaMax));
     }
 
     // Events around the 2-hop and tuple launches of each group (pairs).

@@ -332,6 +332,8 @@ void tc_ensure_attrs();
 // Expansion + pair kernels of every chunk, in stream order (no host sync).
 void tc_launch(const TcPlan &plan, TcArgs base, unsigned char *z, cudaStream_t s);
 constexpr int64_t kTcBlockBytes = 16384;
+// Most Z bytes of one chunk (an anchor larger than that is a chunk of its own).
+constexpr int64_t kTcArenaMax = 1ll << 30;
 
 }  // namespace sbc
 

@@ -72,7 +72,6 @@ struct sbc_server {
     sbc_server_opts opts;
     int device = 0;
     std::vector<const sbc_graph *> graphs;
-    std::vector<uint64_t> footprint;  // estimated device bytes of one count per graph
     std::mutex mu;
     std::condition_variable cv_sched, cv_done;
     std::deque<sbc::Request *> waiting;
@@ -93,13 +92,23 @@ struct sbc_server {
 namespace sbc {
 namespace {
 
-// Rough device footprint of one count: oriented structures are resident, a
+// Rough device footprint of one (p,q) count: oriented structures are resident, a
 // count allocates plan arrays per edge and anchor, candidate masks bounded by
-// the wedges, and work items.
-uint64_t estimate_bytes(const sbc_graph *g) {
-    const uint64_t w = std::min(g->wedges_u, g->wedges_v);
+// the wedges of the side it takes, and work items ...
+uint64_t estimate_bytes(const sbc_graph *g, int p, int q) {
+    const uint64_t w = preferred_side(g, p, q) == 0 ? g->wedges_u : g->wedges_v;
     return 32ull * (uint64_t)g->nnz + 64ull * (uint64_t)std::max(g->n_u, g->n_v) + 4ull * w +
            (1ull << 20);
+}
+
+// ... and, for tuples of three, the graph's share of the job's tensor-core arena
+// (kTcArenaMax at most): 128 bytes per row and 128 positions, rows padded to 256
+// per anchor of at least 128, each row with at least l wedges of its own.
+uint64_t estimate_arena(const sbc_graph *g, int p, int q) {
+    const int side = preferred_side(g, p, q);
+    if ((side == 0 ? p : q) != 3) return 0;
+    const uint64_t rows = side == 0 ? g->wedges_u / (uint64_t)q : g->wedges_v / (uint64_t)p;
+    return 256ull * std::min(rows, (uint64_t)kTcArenaMax);
 }
 
 void lane_main(sbc_server *s, Lane *lane) {
@@ -192,7 +201,7 @@ void scheduler_main(sbc_server *s) {
         job->p = head->p;
         job->q = head->q;
         job->batched = small;
-        uint64_t bytes = 0;
+        uint64_t bytes = 0, arena = 0;  // estimated for the job, and the arena's part of it
         std::vector<uint32_t> seen;
         for (auto it = s->waiting.begin(); it != s->waiting.end();) {
             Request *r = *it;
@@ -205,9 +214,11 @@ void scheduler_main(sbc_server *s) {
                 fit = true;
             }
             if (fit) {
-                uint64_t add = 0;
+                uint64_t add = 0, share = 0;
                 if (std::find(seen.begin(), seen.end(), r->gid) == seen.end()) {
-                    add = s->footprint[r->gid];
+                    share = estimate_arena(s->graphs[r->gid], r->p, r->q);
+                    share = std::min(share, (uint64_t)kTcArenaMax - arena);
+                    add = estimate_bytes(s->graphs[r->gid], r->p, r->q) + share;
                     if (!take_head && bytes + add + s->in_flight_bytes > s->opts.mem_budget_bytes) {
                         ++it;
                         continue;
@@ -215,6 +226,7 @@ void scheduler_main(sbc_server *s) {
                     seen.push_back(r->gid);
                 }
                 bytes += add;
+                arena += share;
                 job->reqs.push_back(r);
                 it = s->waiting.erase(it);
             } else {
@@ -301,7 +313,6 @@ sbc_status sbc_server_add_graph(sbc_server *s, const sbc_graph *g, uint32_t *gid
     std::lock_guard<std::mutex> lock(s->mu);
     *gid = (uint32_t)s->graphs.size();
     s->graphs.push_back(g);
-    s->footprint.push_back(estimate_bytes(g));
     SBC_SRV_END
 }
 
