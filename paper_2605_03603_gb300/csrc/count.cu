@@ -228,6 +228,7 @@ struct PlanArgs {
     const uint32_t *A_ent, *A_pos;
     const int64_t *B_off;
     int64_t nX;
+    int64_t chunks;            // of rows (k_plan): at least nX / PLAN_ROWS
     int R, l, shard, nshard, stats, small_e;
     int direct;                // direct counters allowed (not when a test forces the hash strategies)
     const int64_t *graph_x0;   // batches: first rank per graph (n_graphs + 1), else null
@@ -329,7 +330,7 @@ __global__ void __launch_bounds__(PLAN_THREADS) k_plan(PlanArgs a) {
     };
     // The rows of a step are chunks apart: the hubs, which rank next to one
     // another, go to different CTAs (32 of them on one were 1.1 ms)
-    const int64_t chunks = (a.nX + PLAN_ROWS - 1) / PLAN_ROWS;
+    const int64_t chunks = a.chunks;
     for (int64_t ch = blockIdx.x; ch < chunks; ch += gridDim.x) {
         // four rows per warp, eight lanes each
         const int64_t r = ch + chunks * (4 * warp + (lane >> 3));
@@ -2340,7 +2341,12 @@ struct CountRun {
         pa.key = key;
         pa.hist = hist;
         pa.cnt = cnt.ptr;
-        k_plan<<<grid_for((nX + 3) / 4 * 32, PLAN_THREADS, 152 * 8), PLAN_THREADS, 0, s>>>(pa);
+        // Full chunks, but on a side with rows for the CTA enough chunks to give few
+        // anchors a CTA each (plan of 60 anchors of 50,000 entries: 4.2 ms on two
+        // CTAs, 0.2 on sixty)
+        const int64_t full = (nX + PLAN_ROWS - 1) / PLAN_ROWS;
+        pa.chunks = o->max_deg_x > PLAN_WARP ? std::max(full, std::min<int64_t>(nX, 4 * sm_count())) : full;
+        k_plan<<<(int)std::min<int64_t>(pa.chunks, 152 * 8), PLAN_THREADS, 0, s>>>(pa);
         SBC_LAUNCHED();
         k_order<<<grid_for(nX, 256, 152 * 8), 256, 0, s>>>(key, nX, hist, dprime, rsv_c, cursor, word_cursor,
                                                            cnt.ptr, order, pool_off);
