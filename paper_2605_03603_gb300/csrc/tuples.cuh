@@ -571,6 +571,20 @@ __device__ __forceinline__ void list_all(uint32_t off, uint32_t m, uint32_t ms, 
     else if constexpr (R == 3) list_pairs_wide(off, m, ms, W, wi, warps, l, acc, err);
 }
 
+// Positions of row a, whose first four words are in A (every lane gets the sum).
+template <bool ST>
+__device__ __forceinline__ uint32_t row_positions(const RowsV<ST> &v, uint32_t a, const uint32_t (&A)[4]) {
+    uint32_t n = 0;
+#pragma unroll
+    for (int w = 0; w < 4; w++) n += __popc(A[w]);
+    if (v.W > 4) {
+        uint32_t x = 0;
+        for (uint32_t w = 4 + (threadIdx.x & 31); w < v.W; w += 32) x += __popc(v.word(w, a));
+        n += __reduce_add_sync(FULL, x);
+    }
+    return n;
+}
+
 // Positions shared by row a (words A when W <= WN, else read again) and row c.
 template <int WN, bool ST>
 __device__ __forceinline__ uint32_t shared_count(const RowsV<ST> &v, const uint32_t (&A)[WN],
@@ -673,6 +687,36 @@ __device__ __forceinline__ void project_row(const RowsV<ST> &v, uint32_t a, uint
     if (nb && k < m) sm_dyn[off + plane * ms + k] = out;
 }
 
+// The part of project_row that a's words [w0, w1) give, ORed into a list of zeros
+// (several warps share the walk).
+template <bool ST>
+__device__ __noinline__ void project_words(const RowsV<ST> &v, uint32_t a, uint32_t c, uint32_t w0,
+                                              uint32_t w1, uint32_t off, uint32_t m, uint32_t ms, uint32_t k) {
+    uint32_t at = 0;  // position of the next bit
+    for (uint32_t w = threadIdx.x & 31; w < w0; w += 32) at += __popc(v.word(w, a));
+    at = __reduce_add_sync(FULL, at);
+    uint32_t out = 0;
+    uint32_t na = w0 < w1 ? v.word(w0, a) : 0u, nx = w0 < w1 ? v.word(w0, c) : 0u;
+    for (uint32_t w = w0; w < w1; w++) {
+        uint32_t aw = na;
+        const uint32_t x = nx;
+        if (w + 1 < w1) {
+            na = v.word(w + 1, a);
+            nx = v.word(w + 1, c);
+        }
+        while (aw) {
+            const int b = __ffs(aw) - 1;
+            aw &= aw - 1;
+            out |= ((x >> b) & 1u) << (at & 31);
+            if ((++at & 31) == 0) {
+                if (k < m) atomicOr(&sm_dyn[off + (at / 32 - 1) * ms + k], out);
+                out = 0;
+            }
+        }
+    }
+    if (out && k < m) atomicOr(&sm_dyn[off + (at / 32) * ms + k], out);
+}
+
 // ---- prefixes too wide for the lists: the prefix masks sit in the warp's
 // list area (or its global scratch when they do not fit), every level tests
 // the anchor's own rows.
@@ -714,7 +758,7 @@ constexpr uint32_t DEFER_MAX = 256;
 constexpr uint32_t CTA_LIST = 40;
 
 struct TupleShared {
-    unsigned item, unit, ndefer, m, n_units;
+    unsigned item, unit, ndefer, m, n_units, words;
     uint32_t defer[DEFER_MAX];
     uint32_t hist[256];
 };
@@ -729,13 +773,10 @@ __device__ __forceinline__ void first_row(const RowsV<ST> &v, uint32_t a, int l,
     } else {
         const uint32_t off = TU_OFF_LIST + (uint32_t)warp * TU_LIST_W;
         const uint32_t lt = (1u << lane) - 1u;
-        uint32_t A[4], pa = 0;
+        uint32_t A[4];
 #pragma unroll
-        for (int w = 0; w < 4; w++) {
-            A[w] = w < (int)v.W ? v.word(w, a) : 0u;
-            pa += __popc(A[w]);
-        }
-        for (uint32_t w = 4; w < v.W; w++) pa += __popc(v.word(w, a));
+        for (int w = 0; w < 4; w++) A[w] = w < (int)v.W ? v.word(w, a) : 0u;
+        const uint32_t pa = row_positions<ST>(v, a, A);
         const uint32_t Wp = (pa + 31) / 32;
         bool fits = Wp <= 4 || R == 3;
         uint32_t m = 0;
@@ -783,13 +824,10 @@ __device__ void first_row_cta(const RowsV<ST> &v, uint32_t a, int l, Acc &acc, u
     __syncthreads();
     if (tid == 0) sh.m = 0;
     __syncthreads();
-    uint32_t A[4], pa = 0;
+    uint32_t A[4];
 #pragma unroll
-    for (int w = 0; w < 4; w++) {
-        A[w] = w < (int)v.W ? v.word(w, a) : 0u;
-        pa += __popc(A[w]);
-    }
-    for (uint32_t w = 4; w < v.W; w++) pa += __popc(v.word(w, a));
+    for (int w = 0; w < 4; w++) A[w] = w < (int)v.W ? v.word(w, a) : 0u;
+    const uint32_t pa = row_positions<ST>(v, a, A);
     const uint32_t Wp = (pa + 31) / 32;
     bool fits = Wp <= 4 || R == 3;
     if (fits) {
@@ -808,12 +846,25 @@ __device__ void first_row_cta(const RowsV<ST> &v, uint32_t a, int l, Acc &acc, u
     fits = fits && (unsigned long long)ms * Wp <= TU_LISTS_W;
     if (fits) {
         if (m < (uint32_t)(R - 1)) return;
-        // entry k of the index list is overwritten by its own first word only
-        for (uint32_t kb = 32u * warp; kb < m; kb += 32u * TU_WARPS) {
-            const uint32_t k = kb + lane;
-            const uint32_t c = sm_dyn[TU_OFF_LIST + (k < m ? k : kb)];
-            __syncwarp();
-            project_row<ST>(v, a, c, TU_OFF_LIST, m, ms, k);
+        const uint32_t nb = (m + 31) / 32;
+        if (v.W > 4 && nb <= TU_WARPS / 2) {
+            // few rows of many words: the warps share the words too
+            const uint32_t segs = TU_WARPS / nb, blk = (uint32_t)warp % nb, seg = (uint32_t)warp / nb;
+            const uint32_t k = 32 * blk + lane;
+            const uint32_t c = sm_dyn[TU_OFF_LIST + (k < m ? k : 32 * blk)];
+            __syncthreads();
+            for (uint32_t t = tid; t < ms * Wp; t += TU_THREADS) sm_dyn[TU_OFF_LIST + t] = 0;
+            __syncthreads();
+            if (seg < segs)
+                project_words<ST>(v, a, c, v.W * seg / segs, v.W * (seg + 1) / segs, TU_OFF_LIST, m, ms, k);
+        } else {
+            // entry k of the index list is overwritten by its own first word only
+            for (uint32_t kb = 32u * warp; kb < m; kb += 32u * TU_WARPS) {
+                const uint32_t k = kb + lane;
+                const uint32_t c = sm_dyn[TU_OFF_LIST + (k < m ? k : kb)];
+                __syncwarp();
+                project_row<ST>(v, a, c, TU_OFF_LIST, m, ms, k);
+            }
         }
         __syncthreads();
         list_all<R>(TU_OFF_LIST, m, ms, Wp, pa, (uint32_t)warp, TU_WARPS, l, acc, err);
@@ -831,26 +882,35 @@ __device__ void first_row_cta(const RowsV<ST> &v, uint32_t a, int l, Acc &acc, u
 }
 
 // First rows of an anchor, claimed in batches by the warps (and by the
-// anchor's other items when claim is set).
+// anchor's other items when claim is set); with `wide` (see row_item) one at a
+// time by the CTA.
 template <int R, bool ST>
-__device__ void row_units(const RowsV<ST> &v, uint32_t n_first, unsigned *claim, int l, Acc &acc,
+__device__ void row_units(const RowsV<ST> &v, uint32_t n_first, unsigned *claim, bool wide, int l, Acc &acc,
                           unsigned *err, TupleShared &sh, uint32_t *scratch, uint32_t wmax) {
     const int lane = threadIdx.x & 31;
-    constexpr unsigned BATCH = R == 2 ? 4 : 1;
+    constexpr unsigned BATCH_MAX = R == 2 ? 4 : 1;
+    const unsigned BATCH = v.W <= 8 ? BATCH_MAX : 1u;  // (a wide first row is work enough)
     for (;;) {
         // a round ends when the deferred rows could no longer be recorded
         __syncthreads();
-        if (threadIdx.x == 0) sh.ndefer = 0;
+        if (threadIdx.x == 0) {
+            sh.ndefer = 0;
+            if (R == 3 && wide) {
+                const unsigned u = atomicAdd(claim, 1u);
+                sh.defer[0] = u;
+                sh.ndefer = u < n_first;
+            }
+        }
         __syncthreads();
-        bool more = false;
-        for (;;) {
+        bool more = R == 3 && wide && sh.ndefer != 0;
+        while (R != 3 || !wide) {
             if constexpr (R > 2) {
                 // other warps add to the counter meanwhile: one lane reads it, so
                 // that the warp leaves the loop together
                 unsigned nd = 0;
                 if (lane == 0) nd = *(volatile unsigned *)&sh.ndefer;
                 nd = __shfl_sync(FULL, nd, 0);
-                if (nd > DEFER_MAX - TU_WARPS * BATCH) {
+                if (nd > DEFER_MAX - TU_WARPS * BATCH_MAX) {
                     more = true;
                     break;
                 }
@@ -889,20 +949,40 @@ __device__ void row_item(const TupleArgs &a, const Item &it, Acc &acc, unsigned 
     if (tid == 0) {
         sh.unit = 0;
         sh.n_units = it.claim == NO_CLAIM ? 0u : *(volatile unsigned *)claim;
+        sh.words = 0;
     }
+    bool wide = false;
     if (ordered) {
         for (int i = tid; i < 256; i += TU_THREADS) sh.hist[i] = 0;
         __syncthreads();
         if (sh.n_units >= n_first) return;  // the anchor's other items took everything
         uint16_t *key = (uint16_t *)(sm_dyn + TU_OFF_LIST);
+        uint32_t words = 0;  // of the rows, each projected on itself
         for (uint32_t i = tid; i < n; i += TU_THREADS) {
             uint32_t p = 0;
             for (uint32_t w = 0; w < W; w++) p += __popc(region[(size_t)w * stride + i]);
+            words += (p + 31) / 32;
             const uint32_t k = p < 255u ? p : 255u;
             key[i] = (uint16_t)k;
             atomicAdd(&sh.hist[k], 1u);
         }
+        if (R == 3 && W > 4) {
+            words = __reduce_add_sync(FULL, words);
+            if (lane == 0) atomicAdd(&sh.words, words);
+        }
         __syncthreads();
+        // Three partners: where a typical first row with a quarter of the rows exceeds
+        // a warp's list, nearly every first row goes to the CTA. Warps would defer
+        // them as fast as they claim them, all to the first CTA that comes, and
+        // the anchor's other items would find none left; the CTA takes them one at a
+        // time. Tuples of four in 60 hubs of 500,000: 48 -> 8.8 ms, (4,2) of
+        // K_{40,9000} 12.4 -> 4.0 (with the words of a projection shared by the
+        // warps). More partners keep the warps: (5,5) of the 20k-edge graph took
+        // 0.75 ms this way against 0.62, short lists being a warp's work there.
+        if (R == 3 && W > 4) {
+            const uint32_t wl = sh.words / n;  // of a typical list entry
+            wide = R == 3 && wl > 4 && (n / 4 + 3) * wl > TU_LIST_W;
+        }
         if (tid < 32) {
             uint32_t carry = 0;
             for (int b = 0; b < 256; b += 32) {  // exclusive scan of the bins
@@ -945,7 +1025,7 @@ __device__ void row_item(const TupleArgs &a, const Item &it, Acc &acc, unsigned 
         v.stride = n;
         v.W = W;
         v.n = n;
-        row_units<R, true>(v, n_first, claim, l, acc, err, sh, scratch, a.wmax);
+        row_units<R, true>(v, n_first, claim, wide, l, acc, err, sh, scratch, a.wmax);
     } else {
         RowsV<false> v;
         v.g = region;
@@ -953,7 +1033,7 @@ __device__ void row_item(const TupleArgs &a, const Item &it, Acc &acc, unsigned 
         v.stride = stride;
         v.W = W;
         v.n = n;
-        row_units<R, false>(v, n_first, claim, l, acc, err, sh, scratch, a.wmax);
+        row_units<R, false>(v, n_first, claim, wide, l, acc, err, sh, scratch, a.wmax);
     }
 }
 

@@ -35,16 +35,33 @@ def dense(m, n, density, flip, seed):
     (40, 25000, 4),   # ... and in global scratch (two masks of 782 words)
     (16, 17000, 5),   # four partners, three masks of 532 words
     (14, 9000, 8),    # seven partners, six masks of 282 words
+    # first rows by the CTA, in lists: 1 to 8 blocks of 32 entries, whose words the
+    # warps share, and 9 and 10 blocks
+    (40, 9000, 4),
+    (300, 2500, 4),
+    (24, 600, 5),
 ])
 @pytest.mark.parametrize("density,flip", [(1.0, 0.0), (0.95, 0.02)])
 def test_prefix_masks_outside_the_lists(sbc, m, n, p, density, flip):
     """Tuples of p with q = 2 on U against the other side, where a pair of anchors
     has one partner and its counters give the sum (no masks at all)."""
     g = dense(m, n, density, flip, seed=m + p)
+    same_on_both_sides(sbc, g, p)
+
+
+def same_on_both_sides(sbc, g, p):
     with sbc.graph_from_synth(g) as h:
         got, _, per = sbc.sbc_count_ex(h, p, 2, anchor_side=0, per_anchor=True, method="candidate")
         assert got == sum(per) == sbc.sbc_count_ex(h, p, 2, anchor_side=1)[0]
         assert got > 0
+
+
+@pytest.mark.parametrize("m,n,p", [(60, 20000, 4), (60, 3001, 4), (45, 1999, 5), (30, 700, 6)])
+@pytest.mark.parametrize("density,flip", [(0.5, 0.1), (0.3, 0.02)])
+def test_projection_shared_by_warps(sbc, m, n, p, density, flip):
+    """Rows of both parts, of unequal lengths: list words cut anywhere between the
+    warps' ranges of mask words."""
+    same_on_both_sides(sbc, dense(m, n, density, flip, seed=n), p)
 
 
 @pytest.mark.parametrize("m,n,shards", [
