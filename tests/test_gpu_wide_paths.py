@@ -2,6 +2,8 @@
 tuple kernel outside its lists, in shared memory and in global scratch, and
 rank-indexed 2-hop windows whose mask words take several passes or do not fit
 the staging memory. Counts are exact."""
+from math import comb
+
 import numpy as np
 import pytest
 
@@ -84,3 +86,27 @@ def test_full_windows_equal_hash_tables(sbc, m, n, shards, p, q):
     n_anchors = (m + shards - 1) // shards
     assert st["twohop_anchors"] == [n_anchors, 0, 0, 0]
     assert pairs["twohop_reads"] == pairs["wedges"]
+
+
+@pytest.mark.parametrize("m", [33, 290, 1000, 1025, 2050, 4001])
+@pytest.mark.parametrize("p,q", [(4, 2), (6, 5)])
+def test_column_walk_words(sbc, m, p, q):
+    """Column masks of 1 to 126 words, cut anywhere within a block of words, leaves
+    on both sides of the binomial table's end."""
+    g = dense(m, 9, 1.0, 0.0, seed=m)
+    with sbc.graph_from_synth(g) as h:
+        got, _, per = sbc.sbc_count_ex(h, p, q, anchor_side=0, per_anchor=True, method="position")
+    assert got == comb(m, p) * comb(9, q)
+    assert sorted(per) == sorted(comb(r, p - 1) * comb(9, q) for r in range(m))
+
+
+@pytest.mark.parametrize("m,n", [(130, 14), (420, 13), (700, 12)])
+@pytest.mark.parametrize("p,q", [(4, 3), (5, 2)])
+def test_column_walk_equals_rows(sbc, m, n, p, q):
+    g = dense(m, n, 0.7, 0.15, seed=m)
+    kw = dict(anchor_side=0, per_anchor=True, shard=0, shard_count=m // 8)
+    with sbc.graph_from_synth(g) as h:
+        walk, _, per = sbc.sbc_count_ex(h, p, q, method="position", **kw)
+        rows, _, want = sbc.sbc_count_ex(h, p, q, method="candidate", **kw)
+    assert walk == rows == sum(per) > 0
+    assert per == want
