@@ -196,9 +196,15 @@ typedef struct {
     uint64_t candidates;    /* sum over anchors of |C(u)| */
     uint64_t wedges;        /* 2-hop entries visited */
     uint64_t work_items;    /* tuple-phase work items launched */
-    uint64_t tuples_tested; /* tuples whose common-neighbour mask was tested (after
-                               nested pruning) */
-    uint64_t tuples_typed;  /* tuples with at least q common neighbours (type counts taken) */
+    /* work of the tuple step, not a property of the graph. A candidate gives one
+     * row of mask words per part of its common neighbours (same sign, different
+     * sign) with at least q of them, so a subset of rows is a tuple with a type.
+     * With one partner (tuples of two): candidates, and their rows. Pairs taken on
+     * the tensor cores are in tc_tiles only. */
+    uint64_t tuples_tested; /* subsets of rows (on the position side: prefixes of positions)
+                               whose intersection was counted, after nested pruning */
+    uint64_t tuples_typed;  /* of those, the ones closed with at least q common positions
+                               (position side: position subsets held by enough rows) */
     uint64_t popc_words;    /* mask words popcounted by the tuple kernel (and, where they
                                are on, by the self-checks) */
     int32_t anchor_side;    /* side used */
@@ -213,14 +219,16 @@ typedef struct {
     uint64_t tc_kblocks;    /* K steps of 128 positions over those tiles: the step made
                                tc_kblocks x 128 x 256 x 128 multiply-adds */
     /* CTA-wide 2-hop kernel (anchors with more than the warp tier's wedges), by
-     * strategy: [0] one hash window, or counters indexed by rank, [1] wedges bucketed once by hash class,
-     * [2] the 2-hop re-read once per hash class (fallback), [3] bucketed, then
-     * scattered a second time at exact class offsets (a class overflowed its
-     * capacity) */
+     * strategy: [0] one hash window, or counters indexed by rank (a kernel of
+     * their own), [1] wedges bucketed once by hash class, [2] the 2-hop re-read
+     * once per hash class (fallback), [3] bucketed, then scattered a second time
+     * at exact class offsets (a class overflowed its capacity) */
     uint64_t twohop_reads;      /* 2-hop entries it read, all passes */
     uint64_t twohop_anchors[4]; /* its anchors per strategy */
     float twohop_share[4];      /* share of its SM time per strategy */
-    float twohop_tail_ms;       /* last minus first finish of its CTAs (load imbalance) */
+    float twohop_tail_ms;       /* last minus first finish of its CTAs (load imbalance); of
+                                   the CTAs with counters indexed by rank where there
+                                   are any, since those start as the others end */
     uint64_t pool_bytes;        /* candidate-mask pool: bytes reserved over all anchor groups */
     uint64_t twohop_split_classes; /* hash classes whose distinct partners overflowed one
                                       table and were hashed in sub-class windows */

@@ -191,9 +191,11 @@ __device__ __forceinline__ void binom_add(U128 &acc, unsigned x, int l, unsigned
 // counts, a bitmap of the parts with at least l positions and its prefix counts
 // number the rows, and the counters' memory stages the mask words of the
 // window's rows, a range of positions at a time.
-// Bound by the shared-memory atomics and the L2 gathers of B_ent. The 2-hop
-// kernels of the (3,3) count took 13.7 -> 4.9 ms on the 2M-edge graph, 74 -> 23
-// ms on a 12M-edge hub graph and 15.6 -> 1.0 ms on a dense 3000 x 800 graph
+// Bound by the latency of the gathers of B_ent, four in flight per lane, and by
+// the barriers between an anchor's passes (stalls per issue 8.0 and 6.4; LSU pipe
+// 22 %, L2 20 % on the 500k-edge graph). The 2-hop kernels of the (3,3) count
+// took 13.7 -> 4.9 ms on the 2M-edge graph, 79 -> 23 ms on a 12M-edge hub
+// graph and 15.6 -> 1.0 ms on a dense 3000 x 800 graph
 // (hash strategies -> direct counters where the rule takes them).
 constexpr int DT_THREADS = 512;
 constexpr int DT_WARPS = DT_THREADS / 32;

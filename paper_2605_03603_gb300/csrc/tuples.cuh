@@ -16,8 +16,8 @@
 //   the later rows that share at least l positions with it are listed and
 //   projected onto a's positions, so the remaining levels run on
 //   ceil(|a| / 32) words (one, for most rows) instead of W. Bound by the latency
-//   of AND, POPC and table lookup with four warps per scheduler (POPC pipe 22 to
-//   40 % busy).
+//   of AND, POPC and table lookup with four warps per scheduler (56 % of the issue
+//   slots, POPC pipe 22 % on the (4,4) count of the 500k-edge graph).
 // * column masks (2): for dense rows and few positions, a warp walks the
 //   position subsets depth first over the bitmaps "rows that hold position q",
 //   dropping prefixes contained in fewer than R rows.
